@@ -3,6 +3,7 @@
 // the latter), the domain kinetic energy sum_i 1/2 rho_i |u_i|^2 V_i with node
 // volume V_i = s_i^2, and the probe-weighted momentum sum_i rho_i (px_i u_i +
 // py_i v_i), with their vector-Jacobian products.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -40,23 +41,56 @@ __global__ void k_conserved_vjp(int64_t N, const T* __restrict__ c, const T* __r
     }
 }
 
-// One block, fixed summation order: the same result on every call.
-template <typename T>
-__global__ void k_kinetic_energy(int64_t N, const T* __restrict__ q, const double* __restrict__ s,
-                                 double* __restrict__ out) {
-    __shared__ double red[1024];
+// Sums over the nodes in a fixed order (the same result on every call) without scratch
+// memory: one cluster of kSumBlocks blocks, each thread summing every kSumBlocks * 1024th
+// node, the blocks' sums added by the first one through distributed shared memory.  The
+// sum is bound by the FP64 pipe (exp of every node, 2 lanes a clock and an SM), so it runs
+// on 16 SMs, the most that can share their memory: 65,536 nodes 432 -> about 17 us.
+constexpr int kSumThreads = 1024;
+constexpr int kSumBlocks = 16;
+
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    return v;
+}
+
+template <class Term>
+__device__ void cluster_sum(int64_t N, const Term& term, double* __restrict__ out) {
+    namespace cg = cooperative_groups;
+    __shared__ double red[kSumThreads / 32];
+    __shared__ double block_sum;
+    cg::cluster_group cluster = cg::this_cluster();
     double acc = 0.0;
-    for (int64_t i = threadIdx.x; i < N; i += blockDim.x) {
-        const double rho = exp(double(q[i])), u = double(q[N + i]), v = double(q[2 * N + i]);
-        acc += 0.5 * rho * (u * u + v * v) * s[i] * s[i];
-    }
-    red[threadIdx.x] = acc;
+    for (int64_t i = int64_t(blockIdx.x) * kSumThreads + threadIdx.x; i < N; i += int64_t(gridDim.x) * kSumThreads)
+        acc += term(i);
+    acc = warp_sum(acc);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
+    if (threadIdx.x < 32) {
+        acc = warp_sum(red[threadIdx.x]);
+        if (threadIdx.x == 0) block_sum = acc;
     }
-    if (threadIdx.x == 0) *out = red[0];
+    cluster.sync();
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
+        double v = 0.0;
+        if (threadIdx.x < gridDim.x) v = *cluster.map_shared_rank(&block_sum, threadIdx.x);
+        v = warp_sum(v);
+        if (threadIdx.x == 0) *out = v;
+    }
+    cluster.sync();  // the other blocks' shared memory stays until it has been read
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kSumThreads)
+    k_kinetic_energy(int64_t N, const T* __restrict__ q, const double* __restrict__ s, double* __restrict__ out) {
+    cluster_sum(
+        N,
+        [&](int64_t i) {
+            const double rho = exp(double(q[i])), u = double(q[N + i]), v = double(q[2 * N + i]);
+            return 0.5 * rho * (u * u + v * v) * s[i] * s[i];
+        },
+        out);
 }
 
 template <typename T>
@@ -72,23 +106,17 @@ __global__ void k_kinetic_energy_grad(int64_t N, const T* __restrict__ q, const 
     }
 }
 
-// One block, fixed summation order (as the kinetic energy).
 template <typename T>
-__global__ void k_probe_momentum(int64_t N, const T* __restrict__ q, const double* __restrict__ px,
-                                 const double* __restrict__ py, double* __restrict__ out) {
-    __shared__ double red[1024];
-    double acc = 0.0;
-    for (int64_t i = threadIdx.x; i < N; i += blockDim.x) {
-        const double rho = exp(double(q[i]));
-        acc += rho * (px[i] * double(q[N + i]) + py[i] * double(q[2 * N + i]));
-    }
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *out = red[0];
+__global__ void __launch_bounds__(kSumThreads)
+    k_probe_momentum(int64_t N, const T* __restrict__ q, const double* __restrict__ px,
+                     const double* __restrict__ py, double* __restrict__ out) {
+    cluster_sum(
+        N,
+        [&](int64_t i) {
+            const double rho = exp(double(q[i]));
+            return rho * (px[i] * double(q[N + i]) + py[i] * double(q[2 * N + i]));
+        },
+        out);
 }
 
 template <typename T>
@@ -101,6 +129,34 @@ __global__ void k_probe_momentum_grad(int64_t N, const T* __restrict__ q, const 
         g[N + i] = T(rs * px[i]);
         g[2 * N + i] = T(rs * py[i]);
     }
+}
+
+// One cluster launch of a summing kernel: as many blocks as have nodes, at most kSumBlocks.
+template <typename... KArgs, typename... Args>
+int launch_sum(const char* what, void (*kernel)(KArgs...), int64_t N, cudaStream_t st, Args... args) {
+    int blocks = 1;
+    while (blocks < kSumBlocks && int64_t(blocks) * kSumThreads < N) blocks *= 2;
+    if (blocks > 8)
+        LABFM_CUDA_TRY(cudaFuncSetAttribute(reinterpret_cast<const void*>(kernel),
+                                            cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(blocks));
+    cfg.blockDim = dim3(kSumThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = unsigned(blocks);
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+    if (e != cudaSuccess && blocks > 8) {  // no group of 16 SMs that share memory: the portable size
+        cudaGetLastError();
+        cfg.gridDim.x = attr[0].val.clusterDim.x = 8;
+        e = cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+    }
+    if (e != cudaSuccess) return cuda_error(e, what);
+    return LABFM_OK;
 }
 
 int grid_of(int64_t N) { return int(std::min<int64_t>((N + 255) / 256, 65535)); }
@@ -149,12 +205,9 @@ extern "C" int labfm_kinetic_energy(const void* q, const double* s, int64_t N, l
     if (int rc = check_n(N, dtype)) return rc;
     if (!q || !s || !ke_out) return set_error(LABFM_EINVAL, "null pointer argument");
     cudaStream_t st = as_stream(stream);
-    if (dtype == LABFM_F32)
-        k_kinetic_energy<float><<<1, 1024, 0, st>>>(N, static_cast<const float*>(q), s, ke_out);
-    else
-        k_kinetic_energy<double><<<1, 1024, 0, st>>>(N, static_cast<const double*>(q), s, ke_out);
-    LABFM_LAUNCH_CHECK("kinetic energy kernel");
-    return LABFM_OK;
+    const char* what = "kinetic energy kernel";
+    return dtype == LABFM_F32 ? launch_sum(what, k_kinetic_energy<float>, N, st, N, static_cast<const float*>(q), s, ke_out)
+                              : launch_sum(what, k_kinetic_energy<double>, N, st, N, static_cast<const double*>(q), s, ke_out);
 }
 
 extern "C" int labfm_kinetic_energy_grad(const void* q, const double* s, int64_t N,
@@ -178,12 +231,10 @@ extern "C" int labfm_probe_momentum(const void* q, const double* px, const doubl
     if (int rc = check_n(N, dtype)) return rc;
     if (!q || !px || !py || !j_out) return set_error(LABFM_EINVAL, "null pointer argument");
     cudaStream_t st = as_stream(stream);
-    if (dtype == LABFM_F32)
-        k_probe_momentum<float><<<1, 1024, 0, st>>>(N, static_cast<const float*>(q), px, py, j_out);
-    else
-        k_probe_momentum<double><<<1, 1024, 0, st>>>(N, static_cast<const double*>(q), px, py, j_out);
-    LABFM_LAUNCH_CHECK("probe momentum kernel");
-    return LABFM_OK;
+    const char* what = "probe momentum kernel";
+    return dtype == LABFM_F32
+               ? launch_sum(what, k_probe_momentum<float>, N, st, N, static_cast<const float*>(q), px, py, j_out)
+               : launch_sum(what, k_probe_momentum<double>, N, st, N, static_cast<const double*>(q), px, py, j_out);
 }
 
 extern "C" int labfm_probe_momentum_grad(const void* q, const double* px, const double* py, int64_t N,
