@@ -19,11 +19,11 @@
  *  - Fault injection (for tests of callers' error handling): the environment
  *    variable LABFM_FAULT, read at each call, makes entry points fail on the
  *    host as they would on a real fault.  "alloc": every call that would
- *    allocate device memory (plan creation, labfm_build_stencils,
+ *    allocate device memory (plan creation, labfm_build_stencils, labfm_stencil_count,
  *    labfm_build_weights with n_failed_out, labfm_plan_set_dt's first call,
  *    labfm_plan_set_staging, labfm_plan_enable_adjoint, labfm_step_graph_create)
  *    returns LABFM_ENOMEM before touching the device.  "capacity":
- *    labfm_build_stencils with a col buffer returns LABFM_ECAPACITY with
+ *    labfm_build_stencils with a col buffer (and labfm_stencil_fill) returns LABFM_ECAPACITY with
  *    *nnz_out = col_capacity + 1 before touching the device.
  *    "singular_node:<i>": labfm_build_weights also flags node i
  *    LABFM_NODE_SINGULAR (and counts it as failed).  "timeout":
@@ -147,6 +147,24 @@ int labfm_abi_version(void);
 int labfm_build_stencils(const double* xy, const double* h, int64_t N, double Lx, double Ly,
                          uint32_t periodic_mask, int32_t* row_ptr, int32_t* col,
                          int64_t col_capacity, int64_t* nnz_out, void* stream);
+
+/*
+ * The neighbour search in two calls over a work buffer of the caller's, so that the
+ * size query need not be repeated to fill the columns: labfm_stencil_count builds the
+ * cell list in `work` and counts (row_ptr, *nnz_out, the longest row's entries;
+ * synchronises once), labfm_stencil_fill writes the columns from the cell list it left
+ * there.  Arguments and errors as for labfm_build_stencils; both calls take the same xy,
+ * h, box and mask, and `work` (device, labfm_stencil_work_bytes(N) bytes, 16-byte
+ * aligned) is not touched in between.  Rows longer than 512 entries take nnz int32 of
+ * stream-ordered scratch in labfm_stencil_fill.
+ */
+size_t labfm_stencil_work_bytes(int64_t N);
+int labfm_stencil_count(const double* xy, const double* h, int64_t N, double Lx, double Ly,
+                        uint32_t periodic_mask, int32_t* row_ptr, void* work, size_t work_bytes,
+                        int64_t* nnz_out, int32_t* longest_out, void* stream);
+int labfm_stencil_fill(const double* xy, const double* h, int64_t N, double Lx, double Ly,
+                       uint32_t periodic_mask, const int32_t* row_ptr, void* work, size_t work_bytes,
+                       int64_t nnz, int32_t longest, int32_t* col, int64_t col_capacity, void* stream);
 
 /*
  * Weight build (Sections 2, 3 and 6), FP64 throughout.  For every node i:

@@ -84,6 +84,11 @@ _SIGS = {
     "labfm_abi_version": (_I32, []),
     "labfm_build_stencils": (_I32, [_P, _P, _I64, _D, _D, ctypes.c_uint32, _P, _P, _I64,
                                     ctypes.POINTER(_I64), _P]),
+    "labfm_stencil_work_bytes": (ctypes.c_size_t, [_I64]),
+    "labfm_stencil_count": (_I32, [_P, _P, _I64, _D, _D, ctypes.c_uint32, _P, _P, ctypes.c_size_t,
+                                   ctypes.POINTER(_I64), ctypes.POINTER(ctypes.c_int32), _P]),
+    "labfm_stencil_fill": (_I32, [_P, _P, _I64, _D, _D, ctypes.c_uint32, _P, _P, ctypes.c_size_t, _I64,
+                                  ctypes.c_int32, _P, _I64, _P]),
     "labfm_build_weights": (_I32, [_P, _P, _P, _I64, _D, _D, ctypes.c_uint32, _P, _P, _I64, _I32,
                                    _P, _P, _P, _P, ctypes.POINTER(_I64), _P]),
     "labfm_stencil_optimise": (_I32, [_P, _P, _P, _I64, _D, _D, ctypes.c_uint32, _P, _P, _I32, _D, _D,
@@ -270,17 +275,22 @@ class Phys:
 
 def build_stencils(xy: torch.Tensor, h: torch.Tensor, Lx: float, Ly: float,
                    periodic=(True, True), stream=None):
-    """CSR (row_ptr int32 [N+1], col int32 [nnz]) of |r_ji| <= 2 h_i (labfm_build_stencils)."""
+    """CSR (row_ptr int32 [N+1], col int32 [nnz]) of |r_ji| <= 2 h_i (labfm_stencil_count, then
+    labfm_stencil_fill over the cell list that the count left in its work buffer)."""
     N = _node_set(xy, h=h)
     mask = (1 if periodic[0] else 0) | (2 if periodic[1] else 0)
     row_ptr = torch.empty(N + 1, dtype=torch.int32, device=xy.device)
-    nnz = _I64(0)
+    work = torch.empty(int(lib.labfm_stencil_work_bytes(N)), dtype=torch.uint8, device=xy.device)
+    nnz, longest = _I64(0), ctypes.c_int32(0)
     st = _stream(stream)
-    _check(lib.labfm_build_stencils(_ptr(xy), _ptr(h), N, Lx, Ly, mask, _ptr(row_ptr), None, 0,
-                                    ctypes.byref(nnz), st))
+    args = (_ptr(xy), _ptr(h), N, Lx, Ly, mask, _ptr(row_ptr), _ptr(work), work.numel())
+    _check(lib.labfm_stencil_count(*args, ctypes.byref(nnz), ctypes.byref(longest), st))
     col = torch.empty(max(nnz.value, 1), dtype=torch.int32, device=xy.device)
-    _check(lib.labfm_build_stencils(_ptr(xy), _ptr(h), N, Lx, Ly, mask, _ptr(row_ptr), _ptr(col),
-                                    col.numel(), ctypes.byref(nnz), st))
+    try:
+        _check(lib.labfm_stencil_fill(*args, nnz, longest, _ptr(col), col.numel(), st))
+    finally:
+        if stream is not None:  # the buffer is the current stream's: it outlives the search on the other
+            work.record_stream(stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(st))
     return row_ptr, col[:nnz.value]
 
 

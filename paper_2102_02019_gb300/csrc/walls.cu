@@ -460,14 +460,19 @@ struct Scratch {
 
 int grid_of(int64_t threads) { return int(std::min<int64_t>((threads + 255) / 256, 65535)); }
 
-// CSR of labfm_build_stencils into scratch (query, allocate, fill).
+// The stencils' CSR into scratch (count, allocate, fill).
 int stencils_into(Scratch& sc, const double* xy, const double* h, int64_t n, double Lx, double Ly, uint32_t mask,
                   int32_t** rp, int32_t** col, int64_t* nnz) {
     int rc;
+    char* work = nullptr;
+    const size_t wb = labfm_stencil_work_bytes(n);
+    int32_t longest = 0;
+    if ((rc = sc.get(&work, wb))) return rc;
     if ((rc = sc.get(rp, size_t(n + 1)))) return rc;
-    if ((rc = labfm_build_stencils(xy, h, n, Lx, Ly, mask, *rp, nullptr, 0, nnz, sc.st))) return rc;
+    if ((rc = labfm_stencil_count(xy, h, n, Lx, Ly, mask, *rp, work, wb, nnz, &longest, sc.st))) return rc;
     if ((rc = sc.get(col, size_t(*nnz)))) return rc;
-    return labfm_build_stencils(xy, h, n, Lx, Ly, mask, *rp, *col, std::max<int64_t>(*nnz, 1), nnz, sc.st);
+    return labfm_stencil_fill(xy, h, n, Lx, Ly, mask, *rp, work, wb, *nnz, longest, *col,
+                              std::max<int64_t>(*nnz, 1), sc.st);
 }
 
 }  // namespace
