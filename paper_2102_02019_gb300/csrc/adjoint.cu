@@ -26,6 +26,7 @@
 #include <string>
 #include <type_traits>
 
+#include "fixed.cuh"
 #include "gather.cuh"
 #include "labfm_internal.cuh"
 #include "nvtx.cuh"
@@ -91,7 +92,7 @@ PlanView<T> tview(const labfm_plan* p) {
     return PlanView<T>{p->N, p->tnnz_pad, p->trow_ptr, nullptr, static_cast<const T*>(p->tw),
                        static_cast<const T*>(p->twf), static_cast<const T*>(p->inv_s), p->dt_node,
                        LABFM_ADJ_PREFETCH ? p->prefetch : 0,
-                       nullptr, nullptr, 0, p->N, nullptr, nullptr, T(0), T(0), T(0), T(0)};
+                       nullptr, nullptr, 0, p->N, nullptr, nullptr, T(0), T(0), T(0), T(0), nullptr};
 }
 
 // ---------------------------------------------------------------- pass A
@@ -176,6 +177,18 @@ __global__ void k_adj_pointwise(PlanView<T> P, const Packed<T>* X, const Packed<
     T c[8];
     own_coeffs<T, SCALED>(d, SCALED ? P.inv_s[i] : T(1), c);
     node_adjoints<T, SCALED>(P, i, a, u, v, c, M, gout, oout, ph);
+}
+
+// Pass A from derivative combinations already gathered (fixed_coeffs).
+__global__ void k_adj_pointwise_d8(PlanView<double> P, const Packed<double>* X, const D8<double>* D,
+                                   const Packed<double>* M, G8<double>* __restrict__ gout,
+                                   Packed<double>* __restrict__ oout, Phys<double> ph) {
+    const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    if (i >= P.N) return;
+    double a, u, v, c[8];
+    unpack(X, int(i), a, u, v);
+    d8_load(D, i, c);
+    node_adjoints<double, false>(P, int(i), a, u, v, c, M, gout, oout, ph);
 }
 
 // ---------------------------------------------------------------- pass B
@@ -337,6 +350,24 @@ __device__ __forceinline__ void adjoint_combinations(const double (&w)[6], T (&c
     adjoint_combinations(v, c);
 }
 
+// Column and weights (RHS operators o = 0..4, o = 5: kappa w^hyp) of entry e of the forward
+// operator's row i.
+__device__ __forceinline__ int entry_col(const PlanView<float>& P, int e) {
+    return *reinterpret_cast<const int32_t*>(reinterpret_cast<const char*>(P.w) + Rec<float>::col_e(e));
+}
+__device__ __forceinline__ int entry_col(const PlanView<double>& P, int e) {
+    const uint32_t c = fixed_col_word(P, e, false);
+    return int(P.wexp ? c & kColMask : c);
+}
+template <typename T>
+__device__ __forceinline__ double entry_weight(const PlanView<T>& P, int i, int e, int o) {
+    if constexpr (std::is_same<T, double>::value)
+        if (P.wexp) return fixed_weight(P, i, e, o);
+    const char* at = o < 5 ? reinterpret_cast<const char*>(P.w) + Rec<T>::w_e(e, o)
+                           : reinterpret_cast<const char*>(P.wf) + Rec<T>::fw_e(e);
+    return double(*reinterpret_cast<const T*>(at));
+}
+
 // Warp per forward row i: count the in-degree of every column k (pads, which
 // point at the row itself, are skipped).
 template <typename T>
@@ -346,7 +377,7 @@ __global__ void k_in_degree(PlanView<T> P, int32_t* __restrict__ cnt) {
     for (int64_t i = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5; i < P.N; i += warps) {
         const int e0 = P.row_ptr[i], e1 = P.row_ptr[i + 1];
         for (int e = e0 + lane; e < e1; e += 32) {
-            const int k = *reinterpret_cast<const int32_t*>(reinterpret_cast<const char*>(P.w) + Rec<T>::col_e(e));
+            const int k = entry_col(P, e);
             if (k != i) atomicAdd(cnt + k, 1);
         }
     }
@@ -368,7 +399,7 @@ __global__ void k_fill_transposed(PlanView<T> P, const int32_t* __restrict__ tro
     for (int64_t i = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5; i < P.N; i += warps) {
         const int e0 = P.row_ptr[i], e1 = P.row_ptr[i + 1];
         for (int e = e0 + lane; e < e1; e += 32) {
-            const int k = *reinterpret_cast<const int32_t*>(reinterpret_cast<const char*>(P.w) + Rec<T>::col_e(e));
+            const int k = entry_col(P, e);
             if (k == i) continue;
             const int slot = trow[k] + atomicAdd(cursor + k, 1);
             ti[slot] = int32_t(i);
@@ -401,12 +432,11 @@ __global__ void k_write_transposed(PlanView<T> P, int64_t N, const int32_t* __re
                 rank = 0;
                 for (int r = 0; r < len; ++r) rank += ti[t0 + r] < src_i;
                 const int e = te[t0 + q];
-                const char* rb = reinterpret_cast<const char*>(P.w);
                 double f[5];
 #pragma unroll
-                for (int d = 0; d < 5; ++d) f[d] = double(*reinterpret_cast<const T*>(rb + Rec<T>::w_e(e, d)));
+                for (int d = 0; d < 5; ++d) f[d] = entry_weight(P, src_i, e, d);
                 adjoint_combinations(f, v);
-                vf = *reinterpret_cast<const T*>(reinterpret_cast<const char*>(P.wf) + Rec<T>::fw_e(e));
+                vf = T(entry_weight(P, src_i, e, 5));
             }
             // the same transposition within 16-entry segments as the forward records,
             // so that the lanes of a group gather consecutive entries
@@ -432,10 +462,8 @@ __global__ void k_row_sums(PlanView<T> P, T* __restrict__ rsum) {
         const int e0 = P.row_ptr[i], e1 = P.row_ptr[i + 1];
         double acc[6] = {0, 0, 0, 0, 0, 0};
         for (int e = e0 + lane; e < e1; e += 32) {
-            const char* rb = reinterpret_cast<const char*>(P.w);
 #pragma unroll
-            for (int d = 0; d < 5; ++d) acc[d] += double(*reinterpret_cast<const T*>(rb + Rec<T>::w_e(e, d)));
-            acc[5] += double(*reinterpret_cast<const T*>(reinterpret_cast<const char*>(P.wf) + Rec<T>::fw_e(e)));
+            for (int d = 0; d < 6; ++d) acc[d] += entry_weight(P, int(i), e, d);
         }
 #pragma unroll
         for (int d = 0; d < 6; ++d) {
@@ -620,7 +648,15 @@ int rhs_adjoint_t(const labfm_plan* p, const void* fields, const void* lambda, v
     int rc;
     if ((rc = pack_fields(p, fields, w.X[0], st))) return rc;
     if ((rc = pack_fields(p, lambda, w.Fb, st))) return rc;
-    if ((rc = pass_a<T>(p, w.X[0], w.Fb, w.g, w.Ob, ph, st))) return rc;
+    if constexpr (std::is_same<T, double>::value) {
+        if (p->wexp) {
+            if ((rc = fixed_coeffs(p, w.X[0], w.D, st))) return rc;
+            k_adj_pointwise_d8<<<unsigned((p->N + 127) / 128), 128, 0, st>>>(view<T>(p), w.X[0], w.D, w.Fb, w.g, w.Ob, ph);
+            LABFM_LAUNCH_CHECK("adjoint pointwise kernel");
+        }
+    }
+    if (!p->wexp)
+        if ((rc = pass_a<T>(p, w.X[0], w.Fb, w.g, w.Ob, ph, st))) return rc;
     const FusedA<T> none{nullptr, nullptr, nullptr, nullptr, ph};
     if ((rc = pass_b<T>(p, 0, w.g, w.Ob, w.Lam, nullptr, nullptr, 0.0, 0.0, 0.0, none, st))) return rc;
     return unpack_fields(p, w.Lam, grad, st);

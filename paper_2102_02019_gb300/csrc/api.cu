@@ -82,6 +82,8 @@ void free_plan_memory(labfm_plan* p) {
     cudaFree(p->w);
     cudaFree(p->wf);
     cudaFree(p->inv_s);
+    cudaFree(p->wexp);
+    p->wexp = nullptr;
     cudaFree(p->inst_off);
     cudaFree(p->dt_node);
     cudaFree(p->trow_ptr);

@@ -1,0 +1,352 @@
+// Kernels of F64 plans whose weights are stored in fixed point (fixed.cuh): the right-hand
+// side, the RK stage (recording or not), the derivative combinations of the adjoint and the
+// filter, and the packing of the rows.
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <algorithm>
+
+#include "fixed.cuh"
+#include "labfm_internal.cuh"
+
+namespace labfm {
+namespace {
+
+// Resident warps per SM that the registers allow for (96 and 64 registers).
+#ifndef LABFM_FIXED_RHS_WARPS
+#define LABFM_FIXED_RHS_WARPS 20
+#endif
+#ifndef LABFM_FIXED_FILTER_WARPS
+#define LABFM_FIXED_FILTER_WARPS 28
+#endif
+#define LABFM_FIXED_BOUNDS __launch_bounds__(32 * kFixedWarps, LABFM_FIXED_RHS_WARPS / kFixedWarps)
+#define LABFM_FIXED_FILTER_BOUNDS __launch_bounds__(32 * kFixedWarps, LABFM_FIXED_FILTER_WARPS / kFixedWarps)
+
+__device__ __forceinline__ void pdl_start() {
+#if LABFM_PDL
+    pdl_launch_dependents();
+    pdl_wait();
+#endif
+}
+
+template <int G, bool WALL>
+__global__ void LABFM_FIXED_BOUNDS k_fixed_rhs(PlanView<double> P, SoA<double> in, double* __restrict__ out,
+                                               Phys<double> ph, int passes) {
+    fixed_nodes<G, false>(P, in, passes,
+                          [&](int i, double a, double u, double v, const double (&d)[12]) {
+                              double Ra, Ru, Rv;
+                              node_rhs<double, false, WALL>(P, i, d, a, u, v, 1.0, ph, Ra, Ru, Rv);
+                              out[i] = Ra;
+                              out[P.N + i] = Ru;
+                              out[2 * P.N + i] = Rv;
+                          });
+}
+
+// REC: also stores the node's derivative combinations (k_stage_rec).
+template <int G, bool WALL, bool REC>
+__global__ void LABFM_FIXED_BOUNDS k_fixed_stage(PlanView<double> P, const Packed<double>* X_in,
+                                                 const Packed<double>* Q_in, Packed<double>* Q_out,
+                                                 Packed<double>* X_out, double dt, double bk, double ck,
+                                                 Phys<double> ph, D8<double>* Dout, int passes) {
+    pdl_start();
+    fixed_nodes<G, false>(P, AoS<double>{X_in}, passes,
+                          [&](int i, double a, double u, double v, const double (&d)[12]) {
+                              stage_epilogue<double, false, WALL>(P, i, 0, d, a, u, v, X_in, Q_in, Q_out, X_out,
+                                                                  dt, bk, ck, ph);
+                              if (REC) {
+                                  double c[8];
+                                  own_coeffs<double, false>(d, 1.0, c);
+                                  d8_store(Dout, i, c);
+                              }
+                          });
+}
+
+template <int G>
+__global__ void LABFM_FIXED_BOUNDS k_fixed_coeffs(PlanView<double> P, const Packed<double>* X, D8<double>* Dout,
+                                                  int passes) {
+    pdl_start();
+    fixed_nodes<G, false>(P, AoS<double>{X}, passes,
+                          [&](int i, double, double, double, const double (&d)[12]) {
+                              double c[8];
+                              own_coeffs<double, false>(d, 1.0, c);
+                              d8_store(Dout, i, c);
+                          });
+}
+
+template <int G>
+__global__ void LABFM_FIXED_FILTER_BOUNDS k_fixed_filter(PlanView<double> P, const Packed<double>* in, Packed<double>* out,
+                                                  double* soa, int passes) {
+    pdl_start();
+    fixed_nodes<G, true>(P, AoS<double>{in}, passes,
+                         [&](int i, double a, double u, double v, const double (&s)[3]) {
+                             store(out, i, a + s[0], u + s[1], v + s[2]);
+                             if (soa) {
+                                 soa[i] = a + s[0];
+                                 soa[P.N + i] = u + s[1];
+                                 soa[2 * P.N + i] = v + s[2];
+                             }
+                         });
+}
+
+template <int G>
+__global__ void LABFM_FIXED_FILTER_BOUNDS k_fixed_filter_soa(PlanView<double> P, SoA<double> in, double* __restrict__ out,
+                                                      int passes) {
+    fixed_nodes<G, true>(P, in, passes,
+                         [&](int i, double a, double u, double v, const double (&s)[3]) {
+                             out[i] = a + s[0];
+                             out[P.N + i] = u + s[1];
+                             out[2 * P.N + i] = v + s[2];
+                         });
+}
+
+// ---------------------------------------------------------------- packing
+
+// s_j from how far (in log2, 2^20 units of the high words) the entry's largest weight lies
+// below the row's largest of the same operator: 3, 2, 1 or 0, so that weights falling as
+// r^-1.4 meet differences growing as r.
+__device__ __forceinline__ int entry_shift(int below) {
+    return below >= -748983 ? 3 : (below >= -2246949 ? 2 : (below >= -3744915 ? 1 : 0));
+}
+
+// Warp per row: the row's exponents, then its records (columns with s_j, digits).
+__global__ void k_pack_fixed(int64_t N, int64_t nnz, int64_t off, const int32_t* __restrict__ row_ptr,
+                             const int32_t* __restrict__ col, const double* __restrict__ w,
+                             const double* __restrict__ kappa, const int32_t* __restrict__ prow,
+                             char* __restrict__ rb, char* __restrict__ fb, int16_t* __restrict__ wexp,
+                             int* __restrict__ unfit) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = int64_t(gridDim.x) * (blockDim.x >> 5);
+    for (int64_t il = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5; il < N; il += warps) {
+        const int64_t i = off + il;
+        const int r0 = row_ptr[il], len = row_ptr[il + 1] - r0;
+        const int p0 = prow[i], plen = prow[i + 1] - p0;
+        const double kap = kappa[il];
+        auto weight = [&](int64_t src, int o) { return o < 5 ? w[o * nnz + src] : kap * w[5 * nnz + src]; };
+        int top[6];  // largest high word of |w|
+        bool odd = false;
+#pragma unroll
+        for (int o = 0; o < 6; ++o) top[o] = 0;
+        for (int e = lane; e < len; e += 32)
+#pragma unroll
+            for (int o = 0; o < 6; ++o) top[o] = max(top[o], __double2hiint(weight(int64_t(r0) + e, o)) & 0x7fffffff);
+#pragma unroll
+        for (int o = 0; o < 6; ++o) {
+            top[o] = __reduce_max_sync(0xffffffffu, top[o]);
+            // not finite, or (but for a zero operator) beyond 2^+-400
+            odd |= top[o] >= (1023 + 400) << 20 || (top[o] < (1023 - 400) << 20 && top[o] > 0);
+        }
+        auto shift_of = [&](const int (&h)[6], int o0, int o1) {
+            int below = -0x7fffffff;
+            for (int o = o0; o < o1; ++o)
+                if (top[o] > 0) below = max(below, h[o] - top[o]);
+            return entry_shift(below);
+        };
+        int exps[6];
+        float sum[6];
+#pragma unroll
+        for (int o = 0; o < 6; ++o) {
+            exps[o] = -2000;
+            sum[o] = 0.0f;
+        }
+        for (int e = lane; e < len; e += 32) {
+            int h[6];
+#pragma unroll
+            for (int o = 0; o < 6; ++o) {
+                const double v = weight(int64_t(r0) + e, o);
+                h[o] = __double2hiint(v) & 0x7fffffff;
+                odd |= h[o] == 0 && __double2loint(v) != 0;  // below 2^-1022
+            }
+            const int sr = shift_of(h, 0, 5), sf = shift_of(h, 5, 6);
+#pragma unroll
+            for (int o = 0; o < 6; ++o) {
+                const int s = o < 5 ? sr : sf;
+                exps[o] = max(exps[o], (h[o] >> 20) - s - 1022);
+                // |w| 2^-s over the power of two above the row's largest |w|
+                const int ex = (h[o] >> 20) - (top[o] >> 20) - s + 126;
+                if (h[o] > 0 && ex > 0) sum[o] += __int_as_float((ex << 23) | ((h[o] & 0xfffff) << 3));
+            }
+        }
+#pragma unroll
+        for (int o = 0; o < 6; ++o) {
+            exps[o] = __reduce_max_sync(0xffffffffu, exps[o]);
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) sum[o] += __shfl_xor_sync(0xffffffffu, sum[o], d);
+            if (top[o] == 0 || odd) {
+                exps[o] = 0;
+            } else {
+                float a = ldexpf(sum[o], (top[o] >> 20) - 1022 - exps[o]);
+                while (a > 31.9f) {
+                    a *= 0.5f;
+                    ++exps[o];
+                }
+            }
+        }
+        odd = __any_sync(0xffffffffu, odd);
+        if (odd && lane == 0) atomicOr(unfit, 1);
+        if (odd) continue;
+        if (lane == 0) {
+            int4 v;
+            v.x = (exps[0] & 0xffff) | (exps[1] << 16);
+            v.y = (exps[2] & 0xffff) | (exps[3] << 16);
+            v.z = (exps[4] & 0xffff) | (exps[5] << 16);
+            v.w = 0;
+            reinterpret_cast<int4*>(wexp)[i] = v;
+        }
+        for (int e = lane; e < plen; e += 32) {
+            const int64_t dst = int64_t(p0) + entry_slot(e, plen);
+            uint32_t c = uint32_t(i), sr = 0, sf = 0;
+            int W1[6], W0[6];
+#pragma unroll
+            for (int o = 0; o < 6; ++o) W1[o] = W0[o] = 0;
+            if (e < len) {
+                const int64_t src = int64_t(r0) + e;
+                c = uint32_t(off + col[src]);
+                double v[6];
+                int h[6];
+#pragma unroll
+                for (int o = 0; o < 6; ++o) {
+                    v[o] = weight(src, o);
+                    h[o] = __double2hiint(v[o]) & 0x7fffffff;
+                }
+                sr = uint32_t(shift_of(h, 0, 5));
+                sf = uint32_t(shift_of(h, 5, 6));
+#pragma unroll
+                for (int o = 0; o < 6; ++o) {
+                    const long long W = __double2ll_rn(v[o] * pow2(56 - exps[o] - int(o < 5 ? sr : sf)));
+                    W1[o] = int((W + (1ll << 27)) >> 28);
+                    W0[o] = int(W - ((long long)W1[o] << 28));
+                }
+            }
+            *reinterpret_cast<uint32_t*>(rb + Rec<double>::col_e(dst)) = c | (sr << 30);
+            *reinterpret_cast<uint32_t*>(fb + Rec<double>::fcol_e(dst)) = c | (sf << 30);
+#pragma unroll
+            for (int o = 0; o < 6; ++o) {
+                *reinterpret_cast<int2*>((o < 5 ? rb : fb) + fixed_at(dst, o)) = make_int2(W1[o], W0[o]);
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------- dispatch
+
+// Lanes per node: the plan's, 16 at most.  They do not depend on the number of nodes, so
+// that an instance's sums are the same alone and in a batch.
+int lanes_for(int group) { return std::min(group, 16); }
+
+// The filter gives a lane whole chunks where the right-hand side gives a chunk to two
+// lanes: half the lanes take as many chunks at a time and idle less at the rows' ends
+// (262,144 nodes, order 8: 207 -> 192 us).
+int filter_lanes_for(int group) { return std::max(2, lanes_for(group) / 2); }
+
+// Passes per warp: all the lanes' worth (32 nodes a warp, so that the work after the sums
+// runs on 32 lanes: 262,144 nodes of order 8, one pass 463 us, two 411, four 384) where
+// that still leaves every SM half its warps, else fewer, so that small node sets spread
+// over the chip (40,000 nodes of order 6: one pass 69 us, two 58, four 78).
+int passes_for(int64_t nodes, int g) {
+    int passes = g;
+    while (passes > 1 && nodes * g / (32 * passes) < int64_t(152) * LABFM_FIXED_RHS_WARPS / 2) passes /= 2;
+    return passes;
+}
+
+int grid_of(int64_t nodes, int g, int passes) {
+    const int64_t per = int64_t(passes) * kFixedWarps * (32 / g);
+    return int((nodes + per - 1) / per);
+}
+
+#define LABFM_FIXED_DISPATCH(g, call)                         \
+    switch (g) {                                              \
+        case 2: { constexpr int G = 2; call; break; }         \
+        case 4: { constexpr int G = 4; call; break; }         \
+        case 8: { constexpr int G = 8; call; break; }         \
+        case 16: { constexpr int G = 16; call; break; }       \
+        default: return set_error(LABFM_EINVAL, "unsupported group size"); \
+    }
+
+Phys<double> phys_of(const labfm_phys& ph) { return Phys<double>{ph.c2, ph.mu, ph.gx, ph.gy}; }
+
+PlanView<double> view_of(const labfm_plan* p, int64_t n_lo, int64_t n_hi) {
+    PlanView<double> v = view<double>(p);
+    v.n_lo = n_lo;
+    v.n_hi = n_hi;
+    return v;
+}
+
+}  // namespace
+
+int fixed_rhs(const labfm_plan* p, const void* fields, void* rhs, const labfm_phys& php, int group, cudaStream_t st) {
+    const double* f = static_cast<const double*>(fields);
+    const SoA<double> in{f, f + p->N, f + 2 * p->N};
+    const int g = lanes_for(group), passes = passes_for(p->N, g), grid = grid_of(p->N, g, passes);
+    double* out = static_cast<double*>(rhs);
+    if (p->wall_slot) {
+        LABFM_FIXED_DISPATCH(g, (k_fixed_rhs<G, true><<<grid, 32 * kFixedWarps, 0, st>>>(view<double>(p), in, out, phys_of(php), passes)));
+    } else {
+        LABFM_FIXED_DISPATCH(g, (k_fixed_rhs<G, false><<<grid, 32 * kFixedWarps, 0, st>>>(view<double>(p), in, out, phys_of(php), passes)));
+    }
+    LABFM_LAUNCH_CHECK("fixed-point rhs kernel");
+    return LABFM_OK;
+}
+
+int fixed_stage(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, const void* xin, const void* qin,
+                void* qout, void* xout, double dt, double bk, double ck, const labfm_phys& php, void* D,
+                cudaStream_t st) {
+    if (n_hi <= n_lo) return LABFM_OK;
+    const int g = lanes_for(group), passes = passes_for(n_hi - n_lo, g), grid = grid_of(n_hi - n_lo, g, passes);
+    const PlanView<double> v = view_of(p, n_lo, n_hi);
+    auto launch = [&](auto* kernel) {
+        return launch_pdl(p, kernel, grid, 32 * kFixedWarps, st, v, static_cast<const Packed<double>*>(xin),
+                          static_cast<const Packed<double>*>(qin), static_cast<Packed<double>*>(qout),
+                          static_cast<Packed<double>*>(xout), dt, bk, ck, phys_of(php), static_cast<D8<double>*>(D),
+                          passes);
+    };
+    cudaError_t e = cudaSuccess;
+    if (D) {
+        LABFM_FIXED_DISPATCH(g, (e = launch(k_fixed_stage<G, false, true>)));
+    } else if (p->wall_slot) {
+        LABFM_FIXED_DISPATCH(g, (e = launch(k_fixed_stage<G, true, false>)));
+    } else {
+        LABFM_FIXED_DISPATCH(g, (e = launch(k_fixed_stage<G, false, false>)));
+    }
+    if (e != cudaSuccess) return cuda_error(e, "fixed-point rk stage kernel");
+    return LABFM_OK;
+}
+
+int fixed_coeffs(const labfm_plan* p, const void* X, void* D, cudaStream_t st) {
+    const int g = lanes_for(p->group), passes = passes_for(p->N, g), grid = grid_of(p->N, g, passes);
+    cudaError_t e = cudaSuccess;
+    LABFM_FIXED_DISPATCH(g, (e = launch_pdl(p, k_fixed_coeffs<G>, grid, 32 * kFixedWarps, st, view<double>(p),
+                                            static_cast<const Packed<double>*>(X), static_cast<D8<double>*>(D), passes)));
+    if (e != cudaSuccess) return cuda_error(e, "fixed-point derivative kernel");
+    return LABFM_OK;
+}
+
+int fixed_filter(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, const void* in, void* out, void* soa,
+                 cudaStream_t st) {
+    if (n_hi <= n_lo) return LABFM_OK;
+    const int g = filter_lanes_for(group), passes = passes_for(n_hi - n_lo, g), grid = grid_of(n_hi - n_lo, g, passes);
+    const PlanView<double> v = view_of(p, n_lo, n_hi);
+    cudaError_t e = cudaSuccess;
+    LABFM_FIXED_DISPATCH(g, (e = launch_pdl(p, k_fixed_filter<G>, grid, 32 * kFixedWarps, st, v, static_cast<const Packed<double>*>(in),
+                                            static_cast<Packed<double>*>(out), static_cast<double*>(soa), passes)));
+    if (e != cudaSuccess) return cuda_error(e, "fixed-point filter kernel");
+    return LABFM_OK;
+}
+
+int fixed_filter_soa(const labfm_plan* p, const void* in, void* out, cudaStream_t st) {
+    const double* f = static_cast<const double*>(in);
+    const SoA<double> src{f, f + p->N, f + 2 * p->N};
+    const int g = filter_lanes_for(p->group), passes = passes_for(p->N, g), grid = grid_of(p->N, g, passes);
+    LABFM_FIXED_DISPATCH(g, (k_fixed_filter_soa<G><<<grid, 32 * kFixedWarps, 0, st>>>(view<double>(p), src, static_cast<double*>(out), passes)));
+    LABFM_LAUNCH_CHECK("fixed-point filter kernel");
+    return LABFM_OK;
+}
+
+int fixed_pack(const PlanInput& in, int64_t off, labfm_plan* p, int* unfit, cudaStream_t st) {
+    const int gw = int(std::min<int64_t>((in.N * 32 + 255) / 256, 1 << 20));
+    k_pack_fixed<<<gw, 256, 0, st>>>(in.N, in.nnz, off, in.row_ptr, in.col, in.w, in.kappa, p->row_ptr,
+                                     static_cast<char*>(p->w), static_cast<char*>(p->wf), p->wexp, unfit);
+    LABFM_LAUNCH_CHECK("fixed-point pack kernel");
+    return LABFM_OK;
+}
+
+}  // namespace labfm

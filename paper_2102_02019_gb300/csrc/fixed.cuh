@@ -1,0 +1,452 @@
+// FP64 gathers in fixed point on the integer pipe.
+//
+// GB300 runs 2 FP64 lanes a clock and an SM but 64 lanes of 32 x 32 + 64-bit integer
+// multiply-add (measured: 2.05 DFMA, 65 IMAD.WIDE), so the sums
+// sum_j w_ji (phi_j - phi_i) of an FP64 plan, 12 multiply-adds and 3 subtractions per
+// stencil entry, are bound by the FP64 pipe at 0.2 of the memory rate.  Here only the
+// differences d = phi_j - phi_i are taken in FP64 (as before, rounded once); the products
+// and sums run on integers:
+//
+//   weights, once when the plan is packed:  w_ji 2^-s_j ~ (w1 2^28 + w0) 2^(E_w - 56),
+//     w1 2^28 + w0 = rint(.), |w0| <= 2^27, E_w per row and operator;
+//   differences, per entry:  |d| 2^s_j ~ (d1 2^28 + d0) 2^(E_d - 57), truncated,
+//     0 <= d0 < 2^28, E_d per row and field, raised as larger differences turn up;
+//   sum_j w_ji d_j ~ 2^(E_w + E_d - 113 + 28) (2^28 sum w1 d1 + sum (w1 d0 + w0 d1)),
+//     two exact 64-bit sums; w0 d0 (below 2^-57 of the bounds) is dropped.
+//
+// The shift s_j (0 to 3, two bits of the column word) is the same for an entry's weights
+// and its difference and cancels: it moves the large weights near the node, where the
+// differences are small, down and those differences up, which gains two bits.  Against
+// exact sums, on jittered lattices of orders 4 to 10 (120 rows each, every operator and
+// field), the error of these sums is 0.12-0.69 of the FP64 sums' it replaces on average,
+// 0.93 at most.
+//
+// No overflow: E_w is raised until sum_j |w_ji| 2^-s_j <= 32 2^E_w, so |sum w1 d1| <=
+// 2^(5 + 28 + 29) over a whole row; |sum (w1 d0 + w0 d1)| <= 2^61 + n 2^56 over n entries,
+// whose carries a lane moves up after every 64.  Weights that are not finite or beyond
+// 2^+-400, and plans of 2^30 nodes or more, keep the FP64 weights and kernels
+// (plan.wexp == nullptr).  A row whose differences are not finite or beyond 2^+-500 is
+// summed in FP64 from the decoded weights, so that infinities and NaN come out as they
+// would.  Differences below 2^-1022 count as zero.
+#pragma once
+
+#include "gather.cuh"
+
+namespace labfm {
+namespace {
+
+constexpr uint32_t kColMask = 0x3fffffffu;  // the column word: s_j in the two bits above
+constexpr int kFixedWarps = 2;  // warps a block
+constexpr int kOne20 = 1 << 20;
+constexpr int kFloorT = 65 << 20;           // T below: no difference but zero seen
+constexpr int kLeastT = 524 << 20;          // smallest bound of the fixed-point sums
+constexpr uint32_t kMostT = 1500u << 20;
+
+__device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
+
+// Eight 32-bit words of the record stream, past the L1, which keeps the gathered states
+// (the 262,144-node order-8 stage 384 -> 369 us against evict-first loads).
+__device__ __forceinline__ void ld8i(const void* p, int (&v)[8]) {
+    asm("ld.global.nc.L1::no_allocate.L2::256B.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+        : "l"(p));
+}
+
+// Exponent field of d, in place (biased, times 2^20).
+__device__ __forceinline__ int exponent20(double d) { return __double2hiint(d) & 0x7ff00000; }
+
+// Digits of d for t = T - exponent20(d) - s 2^20 >= 0, T = (E_d - 1) 2^20 (biased): the 53
+// significant bits, leading bit at 60, shifted down by t / 2^20; shifts of 64 and more
+// give zero, so a zero difference (exponent field 0) does.
+__device__ __forceinline__ void digits(double d, int t, int& d1, int& d0) {
+    const int h = __double2hiint(d), l = __double2loint(d);
+    const uint32_t sh = uint32_t(t) >> 20;
+    const uint32_t x1 = (__funnelshift_l(uint32_t(l), uint32_t(h), 8) & 0x1fffffffu) | 0x10000000u;
+    const uint64_t x = (uint64_t(x1) << 32) | (uint32_t(l) << 8);
+    uint32_t top;
+    uint64_t low;
+    asm("shr.u32 %0, %1, %2;" : "=r"(top) : "r"(x1), "r"(sh));
+    asm("shr.u64 %0, %1, %2;" : "=l"(low) : "l"(x), "r"(sh));
+    const int sign = (h >> 31) | 1;
+    d1 = int(top) * sign;
+    d0 = int(uint32_t(low) >> 4) * sign;
+}
+
+// s += a b, 32 x 32 + 64 bits.  As a carry pair, which the assembler makes one wide
+// multiply-add: given as a plain 64-bit sum it regroups the sums of a chunk into products
+// and additions (half as many instructions again, and spills).
+__device__ __forceinline__ void mad_wide(long long& s, int a, int b) {
+    asm("{\n\t.reg .u32 lo, hi;\n\t"
+        "mov.b64 {lo, hi}, %0;\n\t"
+        "mad.lo.cc.s32 lo, %1, %2, lo;\n\t"
+        "madc.hi.s32 hi, %1, %2, hi;\n\t"
+        "mov.b64 %0, {lo, hi};\n\t}"
+        : "+l"(s)
+        : "r"(a), "r"(b));
+}
+__device__ __forceinline__ void mac(long long& hi, long long& mid, int w1, int w0, int d1, int d0) {
+    mad_wide(hi, w1, d1);
+    mad_wide(mid, w1, d0);
+    mad_wide(mid, w0, d1);
+}
+
+// Largest v over the lanes of the group that lie a multiple of STEP apart.
+template <int STEP, int G>
+__device__ __forceinline__ uint32_t group_max(uint32_t v) {
+#pragma unroll
+    for (int off = G / 2; off >= STEP; off >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, off));
+    return v;
+}
+
+// Raises the bound T of one field for the whole lane group when the chunk's largest
+// exponent m (over the group) exceeds it (and only then: other rows of the warp do not
+// change a row's sums), shifting the K sums taken so far.
+template <int K>
+__device__ __forceinline__ void raise_bound(uint32_t m, int& T, long long* hi, long long* mid, bool& cold) {
+    if (m <= uint32_t(T)) return;
+    if (m >= kMostT) {
+        cold = true;
+        return;
+    }
+    const int by = min((int(m) + kOne20 - T) >> 20, 63);
+    T = int(m) + kOne20;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        hi[k] >>= by;
+        mid[k] >>= by;
+    }
+}
+
+// Moves the carries of the low sums up, so that a lane can take rows of any length: due
+// every kFold chunks (64 entries).
+constexpr int kFold = 16;
+template <int K>
+__device__ __forceinline__ void fold(long long (&hi)[K], long long (&mid)[K]) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        hi[k] += mid[k] >> 28;
+        mid[k] &= 0xfffffffll;
+    }
+}
+
+__device__ __forceinline__ void load_cols(const double* w, int64_t off, uint32_t (&c)[4]) {
+    const int4 v = ld_na(reinterpret_cast<const int4*>(reinterpret_cast<const char*>(w) + off));
+    c[0] = uint32_t(v.x);
+    c[1] = uint32_t(v.y);
+    c[2] = uint32_t(v.z);
+    c[3] = uint32_t(v.w);
+}
+
+// Where the values of one field lie: node j's at p[j * stride].
+struct Column {
+    const double* p;
+    int stride;
+    __device__ __forceinline__ double operator[](int j) const { return __ldg(p + int64_t(j) * stride); }
+};
+__device__ __forceinline__ Column column(const SoA<double>& f, int k) { return {k == 0 ? f.a : (k == 1 ? f.u : f.v), 1}; }
+__device__ __forceinline__ Column column(const AoS<double>& f, int k) {
+    return {reinterpret_cast<const double*>(f.p) + k, 4};
+}
+
+// The filter's sums of one row over the lanes of its group, kappa w^hyp on three fields.
+// hi, mid: this lane's sums; T: the three bounds; cold (the same in the whole group): the
+// row needs FP64.  Every lane of the warp takes the same number of iterations (a lane
+// without a chunk adds zeros).
+template <int G, class F>
+__device__ __forceinline__ void filter_row(const PlanView<double>& P, const F& fld, int i, int e0, int e1, int gl,
+                                           long long (&hi)[3], long long (&mid)[3], int (&T)[3], bool& cold) {
+    const int trips = __reduce_max_sync(0xffffffffu, (e1 - e0 + 4 * G - 1) / (4 * G));
+    double own[3];
+    fld.get(i, own[0], own[1], own[2]);
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+        hi[f] = mid[f] = 0;
+        T[f] = kFloorT;
+    }
+    cold = false;
+    int e = e0 + 4 * gl;
+#pragma unroll 1
+    for (int it = 0; it < trips; ++it, e += 4 * G) {
+        const bool on = e < e1;
+        const int64_t c = on ? e >> 2 : 0;  // past the row: any chunk, with the node's own (zero) differences
+        uint32_t cj[4];
+        load_cols(P.wf, Rec<double>::fcol(c), cj);
+        int w[8];
+        ld8i(reinterpret_cast<const char*>(P.wf) + Rec<double>::fw(c), w);
+        double d[3][4];
+        int s20[4], t[3][4], low = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t cw = on ? cj[k] : uint32_t(i);
+            double v[3];
+            fld.get(int(cw & kColMask), v[0], v[1], v[2]);
+            s20[k] = int((cw >> 30) << 20);
+#pragma unroll
+            for (int f = 0; f < 3; ++f) {
+                d[f][k] = v[f] - own[f];
+                t[f][k] = T[f] - exponent20(d[f][k]) - s20[k];
+                low |= t[f][k];
+            }
+        }
+        if (__any_sync(0xffffffffu, low < 0)) {
+#pragma unroll
+            for (int f = 0; f < 3; ++f) {
+                uint32_t m = 0;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) m = max(m, uint32_t(exponent20(d[f][k])) + uint32_t(s20[k]));
+                raise_bound<1>(group_max<1, G>(m), T[f], hi + f, mid + f, cold);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) t[f][k] = T[f] - exponent20(d[f][k]) - s20[k];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int f = 0; f < 3; ++f) {
+                int d1, d0;
+                digits(d[f][k], t[f][k], d1, d0);
+                mac(hi[f], mid[f], w[2 * k], w[2 * k + 1], d1, d0);
+            }
+        if (it % kFold == kFold - 1) fold(hi, mid);
+    }
+    fold(hi, mid);
+#pragma unroll
+    for (int f = 0; f < 3; ++f) cold = cold || (T[f] > kFloorT && T[f] < kLeastT);
+}
+
+// The twelve derivative sums of one row over the lanes of its group, two lanes to a chunk:
+// the even one sums x, y, xx, xy, yy of u, the odd one of v, and each x and y of ln rho
+// over two of the chunk's four entries.  One lane for all twelve sums needed 128 registers
+// (16 warps an SM) and waited for its gathers.  hi, mid: [ln rho x, y, then five]; T:
+// bounds of ln rho and of the lane's own field.
+template <int G, class F>
+__device__ __forceinline__ void rhs_row(const PlanView<double>& P, const F& fld, int i, int e0, int e1, int gl,
+                                        long long (&hi)[7], long long (&mid)[7], int (&T)[2], bool& cold) {
+    const int trips = __reduce_max_sync(0xffffffffu, (e1 - e0 + 2 * G - 1) / (2 * G));
+    const bool odd = gl & 1;
+    const Column fa = column(fld, 0), ff = column(fld, odd ? 2 : 1);
+    const double oa = fa[i], of = ff[i];
+#pragma unroll
+    for (int k = 0; k < 7; ++k) hi[k] = mid[k] = 0;
+    T[0] = T[1] = kFloorT;
+    cold = false;
+    const char* rec = reinterpret_cast<const char*>(P.w);
+    int e = e0 + 4 * (gl >> 1);
+    // columns of the chunk at entry q; past the row the node itself (zero differences)
+    auto columns = [&](int q, uint32_t (&cj)[4]) {
+        load_cols(P.w, Rec<double>::col(q < e1 ? q >> 2 : 0), cj);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) cj[k] = q < e1 ? cj[k] : uint32_t(i);
+    };
+    auto values = [&](const uint32_t (&cj)[4], double (&g)[6]) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) g[k] = ff[int(cj[k] & kColMask)];
+        g[4] = fa[int((odd ? cj[2] : cj[0]) & kColMask)];
+        g[5] = fa[int((odd ? cj[3] : cj[1]) & kColMask)];
+    };
+    uint32_t cj[4];
+    double g[6];
+#pragma unroll 1
+    for (int it = 0; it < trips; ++it, e += 2 * G) {
+        const int64_t c = e < e1 ? e >> 2 : 0;
+        // the chunks of two iterations on into L2, six lines a chunk among its lanes (444 -> 385 us)
+        if (e + 4 * G < e1) {
+            const char* ahead = rec + Rec<double>::col((e + 4 * G) >> 2);
+            constexpr int NR = G < 8 ? G : 8;
+#pragma unroll
+            for (int l = 0; l < 6; l += NR)
+                if (l + (gl & (NR - 1)) < 6)
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(ahead + (l + (gl & (NR - 1))) * 128));
+        }
+        columns(e, cj);
+        values(cj, g);
+        double d[4], da[2];
+        int t[4], ta[2], low = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            d[k] = g[k] - of;
+            t[k] = T[1] - exponent20(d[k]) - int((cj[k] >> 30) << 20);
+            low |= t[k];
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            da[k] = g[4 + k] - oa;
+            ta[k] = T[0] - exponent20(da[k]) - int(((odd ? cj[k + 2] : cj[k]) >> 30) << 20);
+            low |= ta[k];
+        }
+        if (__any_sync(0xffffffffu, low < 0)) {
+            const int T0 = T[0], T1 = T[1];
+            uint32_t m = 0, ma = 0;  // exponents with their shifts: T - t
+#pragma unroll
+            for (int k = 0; k < 4; ++k) m = max(m, uint32_t(T1) - uint32_t(t[k]));
+#pragma unroll
+            for (int k = 0; k < 2; ++k) ma = max(ma, uint32_t(T0) - uint32_t(ta[k]));
+            raise_bound<2>(group_max<1, G>(ma), T[0], hi, mid, cold);
+            raise_bound<5>(group_max<2, G>(m), T[1], hi + 2, mid + 2, cold);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) t[k] += T[1] - T1;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) ta[k] += T[0] - T0;
+        }
+        int last[8];  // the fifth operator's digits of the four entries
+        ld8i(rec + Rec<double>::w(c, 4), last);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {  // entries k and k + 2
+            int w[2][8];
+            ld8i(rec + Rec<double>::w(c, k), w[0]);
+            ld8i(rec + Rec<double>::w(c, k + 2), w[1]);
+#pragma unroll
+            for (int z = 0; z < 2; ++z) {
+                int d1, d0;
+                digits(d[k + 2 * z], t[k + 2 * z], d1, d0);
+#pragma unroll
+                for (int o = 0; o < 4; ++o) mac(hi[2 + o], mid[2 + o], w[z][2 * o], w[z][2 * o + 1], d1, d0);
+                mac(hi[6], mid[6], last[2 * (k + 2 * z)], last[2 * (k + 2 * z) + 1], d1, d0);
+            }
+            int a1, a0;
+            digits(da[k], ta[k], a1, a0);
+#pragma unroll
+            for (int o = 0; o < 2; ++o)
+                mac(hi[o], mid[o], odd ? w[1][2 * o] : w[0][2 * o], odd ? w[1][2 * o + 1] : w[0][2 * o + 1], a1, a0);
+        }
+        if (it % kFold == kFold - 1) fold(hi, mid);
+    }
+    fold(hi, mid);
+#pragma unroll
+    for (int f = 0; f < 2; ++f) cold = cold || (T[f] > kFloorT && T[f] < kLeastT);
+    cold = group_max<1, G>(uint32_t(cold)) != 0;
+}
+
+// Byte offset of the digits (w1, w0) of operator o (5: the filter's kappa w^hyp) at entry e
+// in the RHS (o < 5) or filter records.  The five 32-byte segments of a chunk hold its four
+// entries' first four operators, entry by entry, then the fifth operator of all four, so
+// that a lane needs one entry's words at a time (operator by operator, as the FP64 records
+// are, the kernel needed 164 registers).
+__host__ __device__ __forceinline__ int64_t fixed_at(int64_t e, int o) {
+    if (o == 5) return Rec<double>::fw(e >> 2) + 8 * (e & 3);
+    return o < 4 ? Rec<double>::w(e >> 2, int(e & 3)) + 8 * o : Rec<double>::w(e >> 2, 4) + 8 * (e & 3);
+}
+
+__device__ __forceinline__ uint32_t fixed_col_word(const PlanView<double>& P, int e, bool filter) {
+    const char* at = filter ? reinterpret_cast<const char*>(P.wf) + Rec<double>::fcol_e(e)
+                            : reinterpret_cast<const char*>(P.w) + Rec<double>::col_e(e);
+    return *reinterpret_cast<const uint32_t*>(at);
+}
+
+// Weight of operator o at entry e of row i of a fixed-point plan.
+__device__ __forceinline__ double fixed_weight(const PlanView<double>& P, int i, int e, int o) {
+    const char* rec = o == 5 ? reinterpret_cast<const char*>(P.wf) : reinterpret_cast<const char*>(P.w);
+    const int2 v = *reinterpret_cast<const int2*>(rec + fixed_at(e, o));
+    const long long W = ((long long)v.x << 28) + v.y;
+    return double(W) * pow2(P.wexp[int64_t(i) * 8 + o] - 56 + int(fixed_col_word(P, e, o == 5) >> 30));
+}
+
+// Row i in FP64 from its decoded weights, by one lane.
+template <bool FILTER, int K, class F>
+__device__ __noinline__ void cold_row(const PlanView<double>& P, const F& fld, int i, double (&sum)[K]) {
+    constexpr int KA = FILTER ? 1 : 2, KV = FILTER ? 1 : 5;
+    double ai, ui, vi;
+    fld.get(i, ai, ui, vi);
+#pragma unroll
+    for (int k = 0; k < K; ++k) sum[k] = 0.0;
+    const int e1 = P.row_ptr[i + 1];
+    for (int e = P.row_ptr[i]; e < e1; ++e) {
+        double a, u, v;
+        fld.get(int(fixed_col_word(P, e, FILTER) & kColMask), a, u, v);
+        a -= ai;
+        u -= ui;
+        v -= vi;
+#pragma unroll
+        for (int o = 0; o < KV; ++o) {
+            const double w = fixed_weight(P, i, e, FILTER ? 5 : o);
+            if (o < KA) sum[o] = fma(a, w, sum[o]);
+            sum[KA + o] = fma(u, w, sum[KA + o]);
+            sum[KA + KV + o] = fma(v, w, sum[KA + KV + o]);
+        }
+    }
+}
+
+// The sums of the block's nodes, epi(node, a, u, v, sums) for each.  A pass takes 32/G nodes
+// a warp and kFixedWarps warps' worth of consecutive nodes a block; after the last pass
+// lane l of a warp finishes one node of the warp's: the FP64 work after the sums (about 130
+// instructions, which cost the pipe the same for one lane as for 32) runs on as many lanes
+// as the warp has had nodes.
+template <int G, bool FILTER, class F, class Epi>
+__device__ __forceinline__ void fixed_nodes(const PlanView<double>& P, const F& fld, int passes, const Epi& epi) {
+    constexpr int K = FILTER ? 3 : 12, R = 32 / G, LK = FILTER ? 3 : 7, LT = FILTER ? 3 : 2;
+    __shared__ long long s_hi[kFixedWarps][K][32];
+    __shared__ int s_lo[kFixedWarps][K][32];
+    __shared__ int s_T[kFixedWarps][3][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, gl = lane % G;
+    const int64_t first = P.n_lo + int64_t(blockIdx.x) * passes * (kFixedWarps * R) + warp * R;
+    uint32_t cold_slots = 0;  // of this warp's nodes, those to be summed in FP64
+#pragma unroll 1
+    for (int p = 0; p < passes; ++p) {
+        const int64_t node = first + p * (kFixedWarps * R) + lane / G;
+        if (node - lane / G >= P.n_hi) break;
+        const int i = int(node < P.n_hi ? node : P.n_hi - 1);
+        const int e0 = P.row_ptr[i], e1 = node < P.n_hi ? P.row_ptr[i + 1] : e0;
+        long long hi[LK], lo[LK];
+        int T[LT];
+        bool cold;
+        if constexpr (FILTER) filter_row<G>(P, fld, i, e0, e1, gl, hi, lo, T, cold);
+        else rhs_row<G>(P, fld, i, e0, e1, gl, hi, lo, T, cold);
+        // over the lanes that share a sum: all of them (filter, ln rho), or every second one
+#pragma unroll
+        for (int k = 0; k < LK; ++k) {
+#pragma unroll
+            for (int off = G / 2; off >= (FILTER || k < 2 ? 1 : 2); off >>= 1) {
+                hi[k] += __shfl_xor_sync(0xffffffffu, hi[k], off);
+                lo[k] += __shfl_xor_sync(0xffffffffu, int(lo[k]), off);
+            }
+        }
+        const int slot = p * R + lane / G;
+        if (FILTER ? gl == 0 : gl < 2) {
+            const int k0 = FILTER ? 0 : (gl ? 7 : 2);  // this lane's own field
+#pragma unroll
+            for (int k = 0; k < LK; ++k) {
+                if (!FILTER && k < 2 && gl) continue;
+                const int at = FILTER || k < 2 ? k : k0 + k - 2;
+                s_hi[warp][at][slot] = hi[k] + (lo[k] >> 28);
+                s_lo[warp][at][slot] = int(lo[k]) & 0xfffffff;
+            }
+            if (FILTER) {
+#pragma unroll
+                for (int f = 0; f < LT; ++f) s_T[warp][f][slot] = T[f];
+            } else {
+                if (!gl) s_T[warp][0][slot] = T[0];
+                s_T[warp][1 + gl][slot] = T[1];
+            }
+        }
+        const uint32_t groups = __ballot_sync(0xffffffffu, cold && gl == 0);
+        if (groups)
+            for (int n = 0; n < R; ++n)
+                if (groups >> (n * G) & 1) cold_slots |= 1u << (p * R + n);
+    }
+    __syncwarp();
+    const int64_t node = first + (lane / R) * (kFixedWarps * R) + lane % R;
+    const bool mine = lane < passes * R && node < P.n_hi;
+    double sum[K];
+    if (mine) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int f = FILTER ? k : (k < 2 ? 0 : (k < 7 ? 1 : 2));
+            const int o = FILTER ? 5 : (k < 2 ? k : (k < 7 ? k - 2 : k - 7));
+            // E_w + E_d - 113 + 28, E_d = T / 2^20 + 1 - 1023
+            const double S = pow2(max(P.wexp[node * 8 + o] + (s_T[warp][f][lane] >> 20) - 1107, -1000));
+            sum[k] = fma(double(s_hi[warp][k][lane]), S * 268435456.0, double(s_lo[warp][k][lane]) * S);
+        }
+    }
+    if (cold_slots) {
+        // one lane per row in FP64: rare, and no other lane's business
+        if (mine && (cold_slots >> lane & 1)) cold_row<FILTER, K>(P, fld, int(node), sum);
+    }
+    if (mine) {
+        double a, u, v;
+        fld.get(int(node), a, u, v);
+        epi(int(node), a, u, v, sum);
+    }
+}
+
+}  // namespace
+}  // namespace labfm

@@ -323,6 +323,7 @@ struct PlanView {
     const int32_t* bnd_kind;   // per slot: LABFM_WALL, LABFM_INFLOW, LABFM_OUTFLOW (null: all walls)
     const T* bnd_target;       // per slot: (u_xi,IN, u_eta,IN) of an inflow, p_inf (first) of an outflow
     T sigma, Lb, mach, rho0;   // relaxation coefficient, length, Mach number, reference density
+    const int16_t* wexp;       // F64 plans in fixed point (fixed.cuh): per row the operators' exponents, 8 values
 };
 
 // Operator loads of one 4-entry chunk starting at entry e (a multiple of 4).
@@ -400,7 +401,7 @@ PlanView<T> view(const labfm_plan* p) {
                        static_cast<const T*>(p->wf), static_cast<const T*>(p->inv_s), p->dt_node,
                        p->prefetch, p->wall_slot, static_cast<const T*>(p->wall_n), 0, p->N,
                        p->bnd_kind, static_cast<const T*>(p->bnd_target), T(p->nscbc.sigma), T(p->nscbc.L),
-                       T(p->nscbc.mach), T(p->nscbc.rho0)};
+                       T(p->nscbc.mach), T(p->nscbc.rho0), p->wexp};
 }
 
 // Chunk loaders for the gathers: from the plan's record stream in global memory,
@@ -853,6 +854,39 @@ __device__ __forceinline__ void node_rhs(const PlanView<T>& P, int i, const T (&
         }
     }
     pointwise_rhs<T, SCALED>(d, a, u, v, inv_s, ph.c2, ph.mu, ph.gx, ph.gy, Ra, Ru, Rv);
+}
+
+// The RK stage update at node i from its 12 derivatives: F = R(X_in);
+// Q_out = Q_in + dt_i b_k F; X_out = Q_out + dt_i (a - b) F (skipped when X_out
+// is null).  Q_in may equal Q_out, and Q_in may equal X_in (first stage, where
+// X = Q).  dt_i is the uniform dt or the plan's per-node dt.  Lane 0 of the
+// group stores.  WALL: R is the wall's right-hand side at the plan's wall nodes.
+template <typename T, bool SCALED, bool WALL = false>
+__device__ __forceinline__ void stage_epilogue(const PlanView<T>& P, int i, int gl, const T (&d)[12],
+                                               T ai, T ui, T vi, const Packed<T>* X_in,
+                                               const Packed<T>* Q_in, Packed<T>* Q_out,
+                                               Packed<T>* X_out, double dt, double bk, double ck,
+                                               const Phys<T>& ph) {
+    if (i >= 0 && gl == 0) {
+        T Ra, Ru, Rv;
+        const T is = SCALED ? P.inv_s[i] : T(1);
+        node_rhs<T, SCALED, WALL>(P, i, d, ai, ui, vi, is, ph, Ra, Ru, Rv);
+        const double dti = P.dt_node ? P.dt_node[i] : dt;
+        const T cb = T(dti * bk), cx = T(dti * ck);
+        T qa, qu, qv;
+        if (Q_in == X_in) {
+            qa = ai;
+            qu = ui;
+            qv = vi;
+        } else {
+            unpack_rw(Q_in, i, qa, qu, qv);
+        }
+        qa = fma(cb, Ra, qa);
+        qu = fma(cb, Ru, qu);
+        qv = fma(cb, Rv, qv);
+        store(Q_out, i, qa, qu, qv);
+        if (X_out) store(X_out, i, fma(cx, Ra, qa), fma(cx, Ru, qu), fma(cx, Rv, qv));
+    }
 }
 
 // The eight combinations of a node's derivatives through which the transpose of

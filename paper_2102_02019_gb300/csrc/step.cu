@@ -65,39 +65,6 @@ __global__ void LABFM_STAGE_BOUNDS k_rhs_soa(PlanView<T> P, SoA<T> in, T* __rest
     }
 }
 
-// The RK stage update at node i from its 12 derivatives: F = R(X_in);
-// Q_out = Q_in + dt_i b_k F; X_out = Q_out + dt_i (a - b) F (skipped when X_out
-// is null).  Q_in may equal Q_out, and Q_in may equal X_in (first stage, where
-// X = Q).  dt_i is the uniform dt or the plan's per-node dt.  Lane 0 of the
-// group stores.  WALL: R is the wall's right-hand side at the plan's wall nodes.
-template <typename T, bool SCALED, bool WALL = false>
-__device__ __forceinline__ void stage_epilogue(const PlanView<T>& P, int i, int gl, const T (&d)[12],
-                                               T ai, T ui, T vi, const Packed<T>* X_in,
-                                               const Packed<T>* Q_in, Packed<T>* Q_out,
-                                               Packed<T>* X_out, double dt, double bk, double ck,
-                                               const Phys<T>& ph) {
-    if (i >= 0 && gl == 0) {
-        T Ra, Ru, Rv;
-        const T is = SCALED ? P.inv_s[i] : T(1);
-        node_rhs<T, SCALED, WALL>(P, i, d, ai, ui, vi, is, ph, Ra, Ru, Rv);
-        const double dti = P.dt_node ? P.dt_node[i] : dt;
-        const T cb = T(dti * bk), cx = T(dti * ck);
-        T qa, qu, qv;
-        if (Q_in == X_in) {
-            qa = ai;
-            qu = ui;
-            qv = vi;
-        } else {
-            unpack_rw(Q_in, i, qa, qu, qv);
-        }
-        qa = fma(cb, Ra, qa);
-        qu = fma(cb, Ru, qu);
-        qv = fma(cb, Rv, qv);
-        store(Q_out, i, qa, qu, qv);
-        if (X_out) store(X_out, i, fma(cx, Ra, qa), fma(cx, Ru, qu), fma(cx, Rv, qv));
-    }
-}
-
 // One fused RK stage at node i (i < 0: an idle group that still joins the
 // shuffles).
 template <typename T, int G, bool KAHAN, bool SCALED, bool WALL = false>
@@ -599,6 +566,12 @@ int grid_for(int64_t threads, int block) { return int((threads + block - 1) / bl
 
 // ---------------------------------------------------------------- dispatch
 
+// The constants of a step kernel as the caller gave them (fixed-point launches take these).
+template <typename T>
+labfm_phys as_phys(const Phys<T>& ph) {
+    return labfm_phys{double(ph.c2), double(ph.mu), double(ph.gx), double(ph.gy)};
+}
+
 template <typename T, int G>
 int rhs_launch_g(const labfm_plan* p, const void* fields, void* rhs, const Phys<T>& ph, int block,
                  cudaStream_t st) {
@@ -618,6 +591,7 @@ int rhs_launch_g(const labfm_plan* p, const void* fields, void* rhs, const Phys<
 template <typename T>
 int rhs_launch(const labfm_plan* p, const void* fields, void* rhs, const labfm_phys* php, int group,
                int block, cudaStream_t st) {
+    if (p->wexp) return fixed_rhs(p, fields, rhs, *php, group, st);
     const Phys<T> ph{T(php->c2), T(php->mu), T(php->gx), T(php->gy)};
     switch (group) {
         case 2: return rhs_launch_g<T, 2>(p, fields, rhs, ph, block, st);
@@ -712,6 +686,7 @@ template <typename T>
 int stage_launch(const labfm_plan* p, const Packed<T>* xin, const Packed<T>* qin, Packed<T>* qout,
                  Packed<T>* xout, double dt, double bk, double ck, const Phys<T>& ph, int* counter,
                  cudaStream_t st) {
+    if (p->wexp) return fixed_stage(p, 0, p->N, p->group, xin, qin, qout, xout, dt, bk, ck, as_phys(ph), nullptr, st);
     if constexpr (std::is_same<T, float>::value) {
         if (staged(p)) {
             if (p->group == 32) return stage_bulk_launch_s<32>(p, xin, qin, qout, xout, dt, bk, ck, ph, st);
@@ -766,6 +741,12 @@ int stage_ranges(const labfm_plan* p, const Packed<T>* xin, const Packed<T>* qin
                  Packed<T>* xout, double dt, double bk, double ck, const Phys<T>& ph, cudaStream_t st) {
     for (int r = 0; r < p->n_ranges; ++r) {
         int rc = LABFM_EINVAL;
+        if (p->wexp) {
+            if ((rc = fixed_stage(p, p->range_begin[r], p->range_begin[r + 1], p->range_group[r], xin, qin, qout, xout,
+                                  dt, bk, ck, as_phys(ph), nullptr, st)))
+                return rc;
+            continue;
+        }
         switch (p->range_group[r]) {
             case 2: rc = stage_range_launch_g<T, 2>(p, r, xin, qin, qout, xout, dt, bk, ck, ph, st); break;
             case 4: rc = stage_range_launch_g<T, 4>(p, r, xin, qin, qout, xout, dt, bk, ck, ph, st); break;
@@ -782,6 +763,11 @@ template <typename T>
 int filter_ranges(const labfm_plan* p, const Packed<T>* in, Packed<T>* out, cudaStream_t st, T* soa = nullptr) {
     for (int r = 0; r < p->n_ranges; ++r) {
         int rc = LABFM_EINVAL;
+        if (p->wexp) {
+            if ((rc = fixed_filter(p, p->range_begin[r], p->range_begin[r + 1], p->range_group[r], in, out, soa, st)))
+                return rc;
+            continue;
+        }
         switch (p->range_group[r]) {
             case 2: rc = filter_range_launch_g<T, 2>(p, r, in, out, soa, st); break;
             case 4: rc = filter_range_launch_g<T, 4>(p, r, in, out, soa, st); break;
@@ -796,6 +782,7 @@ int filter_ranges(const labfm_plan* p, const Packed<T>* in, Packed<T>* out, cuda
 
 template <typename T>
 int filter_aos(const labfm_plan* p, const Packed<T>* in, Packed<T>* out, cudaStream_t st, T* soa = nullptr) {
+    if (p->wexp) return fixed_filter(p, 0, p->N, filter_lanes(p), in, out, soa, st);
     switch (filter_lanes(p)) {
         case 2: return filter_aos_g<T, 2>(p, in, out, soa, st);
         case 4: return filter_aos_g<T, 4>(p, in, out, soa, st);
@@ -819,6 +806,7 @@ int filter_soa_g(const labfm_plan* p, const void* in, void* out, cudaStream_t st
 
 template <typename T>
 int filter_soa(const labfm_plan* p, const void* in, void* out, cudaStream_t st) {
+    if (p->wexp) return fixed_filter_soa(p, in, out, st);
     switch (p->group) {
         case 2: return filter_soa_g<T, 2>(p, in, out, st);
         case 4: return filter_soa_g<T, 4>(p, in, out, st);
@@ -846,7 +834,7 @@ int rk_one_step_t(const labfm_plan* p, void* work, double dt, const labfm_phys* 
     Packed<T>* X = P + p->N;
     Packed<T>* Y = X + p->N;
     int* tickets = reinterpret_cast<int*>(Y + p->N);
-    if (p->persistent) LABFM_CUDA_TRY(cudaMemsetAsync(tickets, 0, 4 * sizeof(int), st));
+    if (p->persistent && !p->wexp) LABFM_CUDA_TRY(cudaMemsetAsync(tickets, 0, 4 * sizeof(int), st));
     int rc;
     labfm_plan* pm = const_cast<labfm_plan*>(p);  // only the launch-timing record changes
     const Packed<T>* xin[4] = {X, Y, X, Y};
@@ -912,6 +900,7 @@ template <typename T>
 int stage_rec_launch(const labfm_plan* p, const Packed<T>* xin, const Packed<T>* qin, Packed<T>* qout,
                      Packed<T>* xout, double dt, double bk, double ck, const Phys<T>& ph, D8<T>* D,
                      cudaStream_t st) {
+    if (p->wexp) return fixed_stage(p, 0, p->N, p->group, xin, qin, qout, xout, dt, bk, ck, as_phys(ph), D, st);
     switch (p->group) {
         case 2: return stage_rec_launch_g<T, 2>(p, xin, qin, qout, xout, dt, bk, ck, ph, D, st);
         case 4: return stage_rec_launch_g<T, 4>(p, xin, qin, qout, xout, dt, bk, ck, ph, D, st);
@@ -1224,6 +1213,27 @@ int pack_plan(labfm_plan* p, const PlanInput* in, int n_inst, cudaStream_t st) {
     if (p->dtype == LABFM_F32) {
         LABFM_CUDA_TRY(cudaMalloc(&p->inv_s, size_t(N) * es));
         p->device_bytes += N * es;
+    }
+    // F64: in fixed point (fixed.cuh) where every row can be, else FP64 weights
+    if (p->dtype == LABFM_F64 && N < (int64_t(1) << 30)) {
+        LABFM_CUDA_TRY(cudaMalloc(reinterpret_cast<void**>(&p->wexp), size_t(N) * 8 * sizeof(int16_t)));
+        int* unfit_dev = nullptr;
+        int unfit = 0;
+        LABFM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&unfit_dev), sizeof(int), st));
+        cudaError_t e = cudaMemsetAsync(unfit_dev, 0, sizeof(int), st);
+        for (int k = 0; k < n_inst && e == cudaSuccess && rc == LABFM_OK; ++k)
+            rc = fixed_pack(in[k], p->inst_off_host[k], p, unfit_dev, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&unfit, unfit_dev, sizeof(int), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        cudaFreeAsync(unfit_dev, st);
+        if (rc) return rc;
+        if (e != cudaSuccess) return cuda_error(e, "packing in fixed point");
+        if (!unfit) {
+            p->device_bytes += int64_t(N) * 8 * sizeof(int16_t);
+            return LABFM_OK;
+        }
+        cudaFree(p->wexp);
+        p->wexp = nullptr;
     }
     for (int k = 0; k < n_inst; ++k) {
         const PlanInput& I = in[k];

@@ -1,0 +1,139 @@
+"""FP64 plans, whose sums run in fixed point: against extended-precision sums of the same
+weights and differences, over row lengths, lanes, ranges of magnitude and plans that keep
+FP64 weights; infinities and NaN; exact zeros."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lb():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    import __graft_entry__ as g
+    g.build()
+    import paper_2102_02019_gb300 as lb
+    return lb
+
+
+def _operator(N, lengths, scale, seed):
+    """Random rows: weights falling off by five orders along the row, columns at random."""
+    rng = np.random.default_rng(seed)
+    rp = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int32)
+    col = np.concatenate([np.sort(rng.choice(N, n, replace=False)) for n in lengths]).astype(np.int32)
+    fall = np.concatenate([10.0 ** rng.uniform(-5, 0, n) for n in lengths])
+    w = scale * fall * rng.standard_normal((6, len(col)))
+    return rp, col, w, rng.uniform(0.5, 1.5, N)
+
+
+def _plan(lb, rp, col, w, kappa):
+    dev = lambda a: torch.tensor(a, device="cuda")  # noqa: E731
+    return lb.Plan(dev(rp), dev(col), dev(w), dev(kappa), dev(np.ones(len(rp) - 1)), dtype=torch.float64)
+
+
+def _sums(rp, col, w, q):
+    """Per operator and field sum_j w (q_j - q_i) in extended precision, and the bound
+    n 2^-50 max|w| max|d| on the fixed-point error: 2^-57 of the bound of |w| (at most 4
+    max|w|) and 2^-57 of the bound of |d| (at most 16 max|d|, shifts included) per term,
+    2^-56 for the dropped product, and FP64's n 2^-53 besides."""
+    N = len(rp) - 1
+    out, tol = np.zeros((len(w), 3, N), np.longdouble), np.zeros((len(w), 3, N))
+    for i in range(N):
+        s = slice(rp[i], rp[i + 1])
+        d = (q[:, col[s]] - q[:, i:i + 1])
+        out[:, :, i] = w[:, s].astype(np.longdouble) @ d.astype(np.longdouble).T
+        if rp[i + 1] > rp[i]:
+            tol[:, :, i] = (rp[i + 1] - rp[i]) * 2.0 ** -50 * np.abs(w[:, s]).max(1)[:, None] * np.abs(d).max(1)[None, :]
+    return out, tol
+
+
+def _check(lb, plan, rp, col, w, kappa, q):
+    Q = torch.tensor(q, device="cuda")
+    f, tf = _sums(rp, col, kappa[np.repeat(np.arange(len(rp) - 1), np.diff(rp))] * w[5:], q)
+    got = lb.filter(plan, Q).cpu().numpy()
+    assert np.all(np.abs(got - (q + f[0])) <= tf[0] + 2.0 ** -52 * np.abs(q + f[0]))
+    # rho du/dt with c^2 = 0, mu = 0: R_a = -(u a_x + v a_y) - (u_x + v_y), R_u = -(u u_x + v u_y)
+    s, t = _sums(rp, col, w[:2], q)
+    a, u, v = q
+    R = np.stack([-(u * s[0, 0] + v * s[1, 0]) - (s[0, 1] + s[1, 2])] + [-(u * s[0, k] + v * s[1, k]) for k in (1, 2)])
+    T = np.stack([np.abs(u) * t[0, 0] + np.abs(v) * t[1, 0] + t[0, 1] + t[1, 2]]
+                 + [np.abs(u) * t[0, k] + np.abs(v) * t[1, k] for k in (1, 2)])
+    mag = np.stack([np.abs(u * s[0, 0]) + np.abs(v * s[1, 0]) + np.abs(s[0, 1]) + np.abs(s[1, 2])]
+                   + [np.abs(u * s[0, k]) + np.abs(v * s[1, k]) for k in (1, 2)])
+    with np.errstate(over="ignore", invalid="ignore"):
+        R[1:] += 0.0 * np.exp(-a)  # the viscous term: mu / rho = 0, not a number where rho underflows
+    got = lb.rhs(plan, Q, lb.Phys(0.0, 0.0)).cpu().numpy()
+    assert np.array_equal(np.isnan(got), np.isnan(R))
+    ok = ~np.isnan(R)
+    assert np.all(np.abs(got - R)[ok] <= (T + 2.0 ** -50 * mag)[ok])
+
+
+@pytest.mark.parametrize("group", [2, 4, 8, 16, 32])
+@pytest.mark.parametrize("scale,spread", [(1.0, 1.0), (1e9, 1e-9), (1e-30, 1e40)])
+def test_sums_over_row_lengths(lb, group, scale, spread):
+    # empty rows, chunk edges, and rows past the 64 entries a lane sums between carries
+    lengths = [0, 1, 3, 4, 5, 15, 16, 17, 63, 64, 65, 127, 128, 129, 255, 256, 257, 600] * 3
+    rng = np.random.default_rng(1)
+    N = 620
+    lengths = np.array(lengths + list(rng.integers(0, 40, N - len(lengths))))
+    rp, col, w, kappa = _operator(N, lengths, scale, 2)
+    plan = _plan(lb, rp, col, w, kappa)
+    plan.set_launch(group, 128)
+    _check(lb, plan, rp, col, w, kappa, spread * rng.standard_normal((3, N)))
+    plan.close()
+
+
+@pytest.mark.parametrize("what", ["wide_weights", "tiny_weights", "huge_differences", "tiny_differences"])
+def test_magnitudes_out_of_the_fixed_range(lb, what):
+    rng = np.random.default_rng(5)
+    N = 200
+    rp, col, w, kappa = _operator(N, np.full(N, 30), 1.0, 3)
+    q = rng.standard_normal((3, N))
+    if what == "wide_weights":
+        w[:, ::7] *= 1e130  # beyond 2^400: FP64 weights
+    if what == "tiny_weights":
+        w *= 1e-130
+    if what == "huge_differences":
+        q[0] *= 1e155  # beyond 2^500: those rows in FP64
+    if what == "tiny_differences":
+        q[1] *= 1e-160
+    plan = _plan(lb, rp, col, w, kappa)
+    _check(lb, plan, rp, col, w, kappa, q)
+    plan.close()
+
+
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("where", ["state", "weight"])
+def test_not_finite_values_come_out_as_in_fp64(lb, bad, where):
+    rng = np.random.default_rng(6)
+    N = 150
+    rp, col, w, kappa = _operator(N, np.full(N, 20), 1.0, 4)
+    q = rng.standard_normal((3, N))
+    if where == "state":
+        q[1, 17] = bad
+    else:
+        w[5, rp[40] + 3] = bad
+    plan = _plan(lb, rp, col, w, kappa)
+    got = lb.filter(plan, torch.tensor(q, device="cuda")).cpu().numpy()
+    with np.errstate(invalid="ignore"):
+        ref = np.stack([[q[f, i] + (kappa[i] * w[5, rp[i]:rp[i + 1]] * (q[f, col[rp[i]:rp[i + 1]]] - q[f, i])).sum()
+                         for i in range(N)] for f in range(3)])
+    assert np.array_equal(np.isnan(got), np.isnan(ref))
+    fin = np.isfinite(ref)
+    assert np.array_equal(got[~fin & ~np.isnan(ref)], ref[~fin & ~np.isnan(ref)])
+    assert np.allclose(got[fin], ref[fin], rtol=1e-12, atol=1e-12)
+    plan.close()
+
+
+def test_uniform_fields_give_exact_zeros(lb):
+    rng = np.random.default_rng(7)
+    N = 300
+    rp, col, w, kappa = _operator(N, np.full(N, 25), 1e6, 8)
+    plan = _plan(lb, rp, col, w, kappa)
+    q = torch.tensor(np.repeat(rng.standard_normal((3, 1)), N, axis=1), device="cuda")
+    q[2] = torch.where(torch.arange(N, device="cuda") % 2 == 0, 0.0, -0.0)  # differences of -0
+    assert torch.equal(lb.filter(plan, q), q)
+    assert not lb.rhs(plan, q, lb.Phys(100.0, 0.1)).any()
+    plan.close()
