@@ -186,6 +186,9 @@ namespace {
 struct CellGrid {
     double csx, csy;  // cell sizes
     int ncx, ncy;
+    // in units of max(Lx, Ly), for the FP32 tests: box, cells and their inverses, and the
+    // slack (in cells) that covers the rounding of a position and a radius
+    float Lx, Ly, wx, wy, iwx, iwy, slx, sly;
 };
 
 // Head of the search's work buffer: what the kernels hand to one another and to the host.
@@ -275,7 +278,10 @@ __global__ void k_search_init(SearchState* st) {
 // Cells of about h_min, at most max_cells of them; on the device, so that the whole
 // search synchronises once, after its count.
 __global__ void k_make_grid(SearchState* st, Box b, int64_t max_cells) {
-    CellGrid g{b.Lx, b.Ly, 1, 1};
+    CellGrid g{};
+    g.csx = b.Lx;
+    g.csy = b.Ly;
+    g.ncx = g.ncy = 1;
     if (!st->bad) {
         double cs = __longlong_as_double(static_cast<long long>(st->hmin));
         const double cap = double(max_cells);
@@ -288,6 +294,15 @@ __global__ void k_make_grid(SearchState* st, Box b, int64_t max_cells) {
         g.csx = b.Lx / g.ncx;
         g.csy = b.Ly / g.ncy;
     }
+    const double inv_L = 1.0 / fmax(b.Lx, b.Ly);
+    g.Lx = float(b.Lx * inv_L);
+    g.Ly = float(b.Ly * inv_L);
+    g.wx = float(g.csx * inv_L);
+    g.wy = float(g.csy * inv_L);
+    g.iwx = 1.0f / g.wx;
+    g.iwy = 1.0f / g.wy;
+    g.slx = 1e-4f + 1e-6f * float(g.ncx);
+    g.sly = 1e-4f + 1e-6f * float(g.ncy);
     st->g = g;
 }
 
@@ -372,8 +387,14 @@ __device__ __forceinline__ void bitonic_sort(int (&v)[P], int lane) {
                     if (p & j) continue;
                     const bool up = k < P ? (p & k) == 0 : ((lane * P) & k) == 0;
                     const int a = v[p], b = v[p | j];
-                    v[p] = up ? min(a, b) : max(a, b);
-                    v[p | j] = up ? max(a, b) : min(a, b);
+                    if (k < P) {
+                        v[p] = up ? min(a, b) : max(a, b);
+                        v[p | j] = up ? max(a, b) : min(a, b);
+                    } else {
+                        const bool swap = (a > b) == up;
+                        v[p] = swap ? b : a;
+                        v[p | j] = swap ? a : b;
+                    }
                 }
             }
         }
@@ -424,9 +445,10 @@ __device__ __forceinline__ void rank_row(const int32_t* src, int n, int lane, in
 // rows' prefix sums; the row is compacted in shared memory and sorted in registers
 // (256 keys in about 500 instructions, against 1,550 for ranking 152).  Bound by
 // instruction issue.  1.0M nodes of varying h at order 10 (152 entries): the whole search
-// 44.1 -> 3.27 ms, against a thread per node testing every candidate in FP64, twice for
-// the count and once to fill, and a ranking sort.  48 registers (10 blocks an SM): with
-// 92 the fill took 2.7 ms.
+// 44.1 -> 2.46 ms, against a thread per node testing every candidate in FP64, twice for
+// the count and once to fill, and a ranking sort; half of it is the sort.  40 registers
+// (10 blocks an SM; with 92 the fill alone took 2.7 ms), and a grid of 16 blocks for each
+// that is resident (4: 2.68 ms, one node a warp: 2.72).
 template <int MODE>
 __global__ void __launch_bounds__(32 * kSearchWarps, 10)
     k_neighbours(const double* __restrict__ xy, const double* __restrict__ h, int64_t N, Box b, double inv_L,
@@ -437,10 +459,7 @@ __global__ void __launch_bounds__(32 * kSearchWarps, 10)
     if (st->bad) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const CellGrid g = st->g;
-    const float Lxf = float(b.Lx * inv_L), Lyf = float(b.Ly * inv_L);
-    const float csx = float(g.csx * inv_L), csy = float(g.csy * inv_L);
-    const float icsx = 1.0f / csx, icsy = 1.0f / csy;
-    const float slx = 1e-4f + 1e-6f * float(g.ncx), sly = 1e-4f + 1e-6f * float(g.ncy);
+    const float Lxf = g.Lx, Lyf = g.Ly;
     constexpr float kBand = 24.0f / 16777216.0f;
     int longest = 0;
     for (int64_t slot = int64_t(blockIdx.x) * kSearchWarps + warp; slot < N;
@@ -452,27 +471,27 @@ __global__ void __launch_bounds__(32 * kSearchWarps, 10)
         const float rin = r - kBand, rout = r + kBand;
         const float in2 = rin > 0.0f ? rin * rin * (1.0f - 4e-6f) : -1.0f;
         const float out2 = rout * rout * (1.0f + 4e-6f);
-        const float X = c.x * icsx, Y = c.y * icsy;
+        const float X = c.x * g.iwx, Y = c.y * g.iwy;
         const int r0 = MODE == 0 ? 0 : row_ptr[i];
         const int room = MODE == 0 ? 0 : row_ptr[i + 1] - r0;  // nothing is written past the counted row
         // whether any candidate can be another image of its node (wide enough for every rounding)
         const bool image_x = b.px && (c.x < rout + 1e-5f || c.x > Lxf - rout - 1e-5f);
         const bool image_y = b.py && (c.y < rout + 1e-5f || c.y > Lyf - rout - 1e-5f);
         int ylo, yhi, cnt = 0;
-        const bool all_rows = axis_range(Y, r * icsy, sly, g.ncy, b.py, &ylo, &yhi);
+        const bool all_rows = axis_range(Y, r * g.iwy, g.sly, g.ncy, b.py, &ylo, &yhi);
         for (int y0 = ylo; y0 <= yhi; y0 += 32) {
             // lane -> one row of cells: a run of consecutive slots [s1, s1 + len1), and where
             // the row meets the edge of the box a second one from s2
             const int cy = y0 + lane;
             int s1 = 0, len1 = 0, s2 = 0, len = 0;
             if (cy <= yhi) {
-                float half = r * icsx;
+                float half = r * g.iwx;
                 if (!all_rows) {
-                    const float gap = fmaxf(fmaxf(float(cy) - Y, Y - float(cy + 1)) - sly, 0.0f) * csy;
-                    half = sqrtf(fmaxf(out2 - gap * gap, 0.0f)) * icsx;
+                    const float gap = fmaxf(fmaxf(float(cy) - Y, Y - float(cy + 1)) - g.sly, 0.0f) * g.wy;
+                    half = sqrtf(fmaxf(out2 - gap * gap, 0.0f)) * g.iwx;
                 }
                 int xlo, xhi;
-                axis_range(X, half, slx, g.ncx, b.px, &xlo, &xhi);
+                axis_range(X, half, g.slx, g.ncx, b.px, &xlo, &xhi);
                 const int32_t* cs = cell_start + int64_t(cy < 0 ? cy + g.ncy : (cy >= g.ncy ? cy - g.ncy : cy)) * g.ncx;
                 if (xlo < 0 || xhi >= g.ncx) {
                     s2 = cs[0];
@@ -496,35 +515,41 @@ __global__ void __launch_bounds__(32 * kSearchWarps, 10)
             const int end1 = incl - len + len1;             // up to here,
             const int wrap = s2 - s1 - len1;                // and from here on first + t + wrap
             const bool wraps = __any_sync(0xffffffffu, len > len1);
-            const int top = rows > 1 ? 1 << (31 - __clz(rows - 1)) : 0;  // first step of the search below
             for (int t0 = 0; t0 < total; t0 += 32) {
                 const int t = t0 + lane;
                 // the row holding candidate t: how many of the rows end at or before t
                 int q = 0;
-                for (int step = top; step > 0; step >>= 1) {
-                    const int e = __shfl_sync(0xffffffffu, incl, (q + step - 1) & 31);
-                    if (q + step <= 31 && t >= e) q += step;
+                auto descend = [&](int step) {
+                    const int e = __shfl_sync(0xffffffffu, incl, q + step - 1);
+                    if (t >= e && t < total) q += step;
+                };
+                if (rows > 8) {
+                    descend(16);
+                    descend(8);
                 }
+                descend(4);
+                descend(2);
+                descend(1);
                 int k = __shfl_sync(0xffffffffu, first, q) + t;
                 if (wraps) {
                     const int e = __shfl_sync(0xffffffffu, end1, q), d = __shfl_sync(0xffffffffu, wrap, q);
                     if (t >= e) k += d;
                 }
-                bool in = false;
-                if (t < total) {
-                    const float2 p = pos[k];
-                    float dx = p.x - c.x, dy = p.y - c.y;
-                    if (image_x) dx = dx > 0.5f * Lxf ? dx - Lxf : (dx < -0.5f * Lxf ? dx + Lxf : dx);
-                    if (image_y) dy = dy > 0.5f * Lyf ? dy - Lyf : (dy < -0.5f * Lyf ? dy + Lyf : dy);
-                    const float d2 = dx * dx + dy * dy;
-                    in = d2 <= in2;
-                    if (!in && d2 < out2) {  // too close to the radius for FP32
+                k = t < total ? k : int(slot);  // past the last candidate the node itself, which is none
+                const float2 p = pos[k];
+                float dx = p.x - c.x, dy = p.y - c.y;
+                if (image_x) dx = dx > 0.5f * Lxf ? dx - Lxf : (dx < -0.5f * Lxf ? dx + Lxf : dx);
+                if (image_y) dy = dy > 0.5f * Lyf ? dy - Lyf : (dy < -0.5f * Lyf ? dy + Lyf : dy);
+                const float d2 = dx * dx + dy * dy;
+                const bool near = d2 < out2 && k != int(slot);
+                bool in = near && d2 <= in2;
+                if (__any_sync(0xffffffffu, near && !in)) {  // too close to the radius for FP32
+                    if (near && !in) {
                         const int64_t j = node[k];
                         const double ex = min_image(__dsub_rn(xy[2 * j], xy[2 * int64_t(i)]), b.Lx, b.px);
                         const double ey = min_image(__dsub_rn(xy[2 * j + 1], xy[2 * int64_t(i) + 1]), b.Ly, b.py);
                         in = __dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)) <= __dmul_rn(two_h, two_h);
                     }
-                    in = in && k != int(slot);
                 }
                 const unsigned hits = __ballot_sync(0xffffffffu, in);
                 if (MODE != 0 && in) {
@@ -590,7 +615,7 @@ int check_search_args(const double* xy, const double* h, int64_t N, double Lx, d
 
 Box make_box(double Lx, double Ly, uint32_t mask) { return Box{Lx, Ly, (mask & 1u) != 0, (mask & 2u) != 0}; }
 
-int search_grid(int64_t N) { return int(std::min<int64_t>((N + kSearchWarps - 1) / kSearchWarps, 1 << 20)); }
+int search_grid(int64_t N) { return int(std::min<int64_t>((N + kSearchWarps - 1) / kSearchWarps, 152 * 10 * 16)); }
 
 // Cell list and row counts: row_ptr, nnz and the longest row; synchronises once.
 int count_stencils(const double* xy, const double* h, int64_t N, double Lx, double Ly, uint32_t mask,
