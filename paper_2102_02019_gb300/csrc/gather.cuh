@@ -706,22 +706,34 @@ __device__ __forceinline__ void gather_derivatives(const PlanView<T>& P, const F
 __device__ __forceinline__ float exp_neg(float a) { return expf(-a); }
 __device__ __forceinline__ double exp_neg(double a) { return exp(-a); }
 
+// Rounded products and sums that the compiler does not contract.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+
 // Pointwise right-hand side of eq. icns from the derivatives.  F32 weights are
-// nondimensional (w s^l), so the sums are scaled by s^-1 or s^-2 here.
+// nondimensional (w s^l), so the sums are scaled by s^-1 or s^-2 here.  The fused
+// products are written out: which of them the compiler would fuse depends on the code
+// around the call, and every stage kernel is to give the same bits.
 template <typename T, bool SCALED>
 __device__ __forceinline__ void pointwise_rhs(const T (&d)[12], T a, T u, T v, T inv_s, T c2, T mu,
                                               T gx, T gy, T& Ra, T& Ru, T& Rv) {
     const T s1 = SCALED ? inv_s : T(1);
-    const T s2 = SCALED ? inv_s * inv_s : T(1);
-    const T ax = d[0] * s1, ay = d[1] * s1;
-    const T ux = d[2] * s1, uy = d[3] * s1, uxx = d[4] * s2, uxy = d[5] * s2, uyy = d[6] * s2;
-    const T vx = d[7] * s1, vy = d[8] * s1, vxx = d[9] * s2, vxy = d[10] * s2, vyy = d[11] * s2;
-    const T nu = mu * exp_neg(a);
+    const T s2 = SCALED ? mul_rn(inv_s, inv_s) : T(1);
+    const T ax = mul_rn(d[0], s1), ay = mul_rn(d[1], s1);
+    const T ux = mul_rn(d[2], s1), uy = mul_rn(d[3], s1);
+    const T uxx = mul_rn(d[4], s2), uxy = mul_rn(d[5], s2);
+    const T vx = mul_rn(d[7], s1), vy = mul_rn(d[8], s1);
+    const T vxy = mul_rn(d[10], s2), vyy = mul_rn(d[11], s2);
+    const T nu = mul_rn(mu, exp_neg(a));
     const T third = T(1) / T(3);
     const T four_thirds = T(4) / T(3);
-    Ra = -(u * ax + v * ay) - (ux + vy);
-    Ru = -(u * ux + v * uy) - c2 * ax + nu * (four_thirds * uxx + uyy + third * vxy) + gx;
-    Rv = -(u * vx + v * vy) - c2 * ay + nu * (four_thirds * vyy + vxx + third * uxy) + gy;
+    Ra = add_rn(-fma(u, ax, mul_rn(v, ay)), -add_rn(ux, vy));
+    Ru = fma(-c2, ax, -fma(u, ux, mul_rn(v, uy)));
+    Rv = fma(-c2, ay, -fma(u, vx, mul_rn(v, vy)));
+    Ru = add_rn(fma(nu, fma(third, vxy, fma(d[6], s2, mul_rn(four_thirds, uxx))), Ru), gx);
+    Rv = add_rn(fma(nu, fma(third, uxy, fma(d[9], s2, mul_rn(four_thirds, vyy))), Rv), gy);
 }
 
 template <typename T>
@@ -901,7 +913,7 @@ template <> struct D8<double> { double2 q[4]; };
 template <typename T, bool SCALED>
 __device__ __forceinline__ void own_coeffs(const T (&d)[12], T inv_s, T (&c)[8]) {
     const T s1 = SCALED ? inv_s : T(1);
-    const T s2 = SCALED ? inv_s * inv_s : T(1);
+    const T s2 = SCALED ? mul_rn(inv_s, inv_s) : T(1);
     const T third = T(1) / T(3);
     const T four_thirds = T(4) / T(3);
     c[0] = d[0] * s1;
@@ -910,8 +922,8 @@ __device__ __forceinline__ void own_coeffs(const T (&d)[12], T inv_s, T (&c)[8])
     c[3] = d[3] * s1;
     c[4] = d[7] * s1;
     c[5] = d[8] * s1;
-    c[6] = four_thirds * (d[4] * s2) + d[6] * s2 + third * (d[10] * s2);
-    c[7] = four_thirds * (d[11] * s2) + d[9] * s2 + third * (d[5] * s2);
+    c[6] = fma(third, mul_rn(d[10], s2), fma(d[6], s2, mul_rn(four_thirds, mul_rn(d[4], s2))));
+    c[7] = fma(third, mul_rn(d[5], s2), fma(d[9], s2, mul_rn(four_thirds, mul_rn(d[11], s2))));
 }
 
 __device__ __forceinline__ void d8_store(D8<float>* p, int64_t i, const float (&c)[8]) {

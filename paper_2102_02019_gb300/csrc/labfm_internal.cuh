@@ -188,6 +188,15 @@ void prof_end(labfm_plan* p, int idx, cudaStream_t st);
 int set_walls(labfm_plan* p, int64_t n_wall, const int32_t* nodes, const double* normal, const int32_t* kind,
               const double* target, cudaStream_t st);
 
+// F32 stage (recording when D is not null) and filter launches over nodes [n_lo, n_hi) that
+// keep several chunks in flight (ahead.cu); ahead_serves: for launches of this size.
+bool ahead_serves(int64_t nodes, int group);
+int ahead_stage(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, const void* xin, const void* qin,
+                void* qout, void* xout, double dt, double bk, double ck, const labfm_phys& ph, void* D,
+                cudaStream_t st);
+int ahead_filter(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, const void* in, void* out, void* soa,
+                 cudaStream_t st);
+
 // The gathers of F64 plans in fixed point (fixed.cu), on `group` lanes per node or more.
 // Packed states, D8 records and SoA fields as in step.cu; nodes [n_lo, n_hi).
 int fixed_rhs(const labfm_plan* p, const void* fields, void* rhs, const labfm_phys& ph, int group, cudaStream_t st);

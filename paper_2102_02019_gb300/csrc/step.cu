@@ -688,6 +688,8 @@ int stage_launch(const labfm_plan* p, const Packed<T>* xin, const Packed<T>* qin
                  cudaStream_t st) {
     if (p->wexp) return fixed_stage(p, 0, p->N, p->group, xin, qin, qout, xout, dt, bk, ck, as_phys(ph), nullptr, st);
     if constexpr (std::is_same<T, float>::value) {
+        if (!staged(p) && !p->persistent && ahead_serves(p->N, p->group))
+            return ahead_stage(p, 0, p->N, p->group, xin, qin, qout, xout, dt, bk, ck, as_phys(ph), nullptr, st);
         if (staged(p)) {
             if (p->group == 32) return stage_bulk_launch_s<32>(p, xin, qin, qout, xout, dt, bk, ck, ph, st);
             return stage_bulk_launch_s<16>(p, xin, qin, qout, xout, dt, bk, ck, ph, st);
@@ -747,6 +749,12 @@ int stage_ranges(const labfm_plan* p, const Packed<T>* xin, const Packed<T>* qin
                 return rc;
             continue;
         }
+        if (std::is_same<T, float>::value && ahead_serves(p->range_begin[r + 1] - p->range_begin[r], p->range_group[r])) {
+            if ((rc = ahead_stage(p, p->range_begin[r], p->range_begin[r + 1], p->range_group[r], xin, qin,
+                                  qout, xout, dt, bk, ck, as_phys(ph), nullptr, st)))
+                return rc;
+            continue;
+        }
         switch (p->range_group[r]) {
             case 2: rc = stage_range_launch_g<T, 2>(p, r, xin, qin, qout, xout, dt, bk, ck, ph, st); break;
             case 4: rc = stage_range_launch_g<T, 4>(p, r, xin, qin, qout, xout, dt, bk, ck, ph, st); break;
@@ -768,6 +776,11 @@ int filter_ranges(const labfm_plan* p, const Packed<T>* in, Packed<T>* out, cuda
                 return rc;
             continue;
         }
+        if (std::is_same<T, float>::value && ahead_serves(p->range_begin[r + 1] - p->range_begin[r], p->range_group[r])) {
+            if ((rc = ahead_filter(p, p->range_begin[r], p->range_begin[r + 1], p->range_group[r], in, out, soa, st)))
+                return rc;
+            continue;
+        }
         switch (p->range_group[r]) {
             case 2: rc = filter_range_launch_g<T, 2>(p, r, in, out, soa, st); break;
             case 4: rc = filter_range_launch_g<T, 4>(p, r, in, out, soa, st); break;
@@ -783,6 +796,8 @@ int filter_ranges(const labfm_plan* p, const Packed<T>* in, Packed<T>* out, cuda
 template <typename T>
 int filter_aos(const labfm_plan* p, const Packed<T>* in, Packed<T>* out, cudaStream_t st, T* soa = nullptr) {
     if (p->wexp) return fixed_filter(p, 0, p->N, filter_lanes(p), in, out, soa, st);
+    if (std::is_same<T, float>::value && !p->filter_persistent && ahead_serves(p->N, filter_lanes(p)))
+        return ahead_filter(p, 0, p->N, filter_lanes(p), in, out, soa, st);
     switch (filter_lanes(p)) {
         case 2: return filter_aos_g<T, 2>(p, in, out, soa, st);
         case 4: return filter_aos_g<T, 4>(p, in, out, soa, st);
@@ -901,6 +916,8 @@ int stage_rec_launch(const labfm_plan* p, const Packed<T>* xin, const Packed<T>*
                      Packed<T>* xout, double dt, double bk, double ck, const Phys<T>& ph, D8<T>* D,
                      cudaStream_t st) {
     if (p->wexp) return fixed_stage(p, 0, p->N, p->group, xin, qin, qout, xout, dt, bk, ck, as_phys(ph), D, st);
+    if (std::is_same<T, float>::value && !p->wall_slot && ahead_serves(p->N, p->group))
+        return ahead_stage(p, 0, p->N, p->group, xin, qin, qout, xout, dt, bk, ck, as_phys(ph), D, st);
     switch (p->group) {
         case 2: return stage_rec_launch_g<T, 2>(p, xin, qin, qout, xout, dt, bk, ck, ph, D, st);
         case 4: return stage_rec_launch_g<T, 4>(p, xin, qin, qout, xout, dt, bk, ck, ph, D, st);
