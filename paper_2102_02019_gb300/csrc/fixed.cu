@@ -49,7 +49,7 @@ __global__ void LABFM_FIXED_BOUNDS k_fixed_stage(PlanView<double> P, const Packe
                                                  Packed<double>* X_out, double dt, double bk, double ck,
                                                  Phys<double> ph, D8<double>* Dout, int passes) {
     pdl_start();
-    fixed_nodes<G, false>(P, AoS<double>{X_in}, passes,
+    fixed_nodes<G, false>(P, State{X_in}, passes,
                           [&](int i, double a, double u, double v, const double (&d)[12]) {
                               stage_epilogue<double, false, WALL>(P, i, 0, d, a, u, v, X_in, Q_in, Q_out, X_out,
                                                                   dt, bk, ck, ph);
@@ -65,7 +65,7 @@ template <int G>
 __global__ void LABFM_FIXED_BOUNDS k_fixed_coeffs(PlanView<double> P, const Packed<double>* X, D8<double>* Dout,
                                                   int passes) {
     pdl_start();
-    fixed_nodes<G, false>(P, AoS<double>{X}, passes,
+    fixed_nodes<G, false>(P, State{X}, passes,
                           [&](int i, double, double, double, const double (&d)[12]) {
                               double c[8];
                               own_coeffs<double, false>(d, 1.0, c);
@@ -77,7 +77,7 @@ template <int G>
 __global__ void LABFM_FIXED_FILTER_BOUNDS k_fixed_filter(PlanView<double> P, const Packed<double>* in, Packed<double>* out,
                                                   double* soa, int passes) {
     pdl_start();
-    fixed_nodes<G, true>(P, AoS<double>{in}, passes,
+    fixed_nodes<G, true>(P, State{in}, passes,
                          [&](int i, double a, double u, double v, const double (&s)[3]) {
                              store(out, i, a + s[0], u + s[1], v + s[2]);
                              if (soa) {

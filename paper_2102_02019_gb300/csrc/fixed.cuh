@@ -137,14 +137,21 @@ __device__ __forceinline__ void load_cols(const double* w, int64_t off, uint32_t
     c[3] = uint32_t(v.w);
 }
 
+// A packed state that the launch before may write.  Plain loads: read-only ones (__ldg) the
+// compiler may move above the wait for that launch.
+struct State {
+    const Packed<double>* p;
+    __device__ __forceinline__ void get(int j, double& x, double& y, double& z) const { unpack_rw(p, j, x, y, z); }
+};
+
 // Where the values of one field lie: node j's at p[j * stride].
 struct Column {
     const double* p;
     int stride;
-    __device__ __forceinline__ double operator[](int j) const { return __ldg(p + int64_t(j) * stride); }
+    __device__ __forceinline__ double operator[](int j) const { return p[int64_t(j) * stride]; }
 };
 __device__ __forceinline__ Column column(const SoA<double>& f, int k) { return {k == 0 ? f.a : (k == 1 ? f.u : f.v), 1}; }
-__device__ __forceinline__ Column column(const AoS<double>& f, int k) {
+__device__ __forceinline__ Column column(const State& f, int k) {
     return {reinterpret_cast<const double*>(f.p) + k, 4};
 }
 
