@@ -22,15 +22,15 @@ namespace {
 #define LABFM_FIXED_BOUNDS __launch_bounds__(32 * kFixedWarps, LABFM_FIXED_RHS_WARPS / kFixedWarps)
 #define LABFM_FIXED_FILTER_BOUNDS __launch_bounds__(32 * kFixedWarps, LABFM_FIXED_FILTER_WARPS / kFixedWarps)
 
-__device__ __forceinline__ void pdl_start() {
-#if LABFM_PDL
-    pdl_launch_dependents();
-    pdl_wait();
-#endif
-}
+// Launched so that they may start when the launch before ends (launch_pdl), with the row
+// pointers read before the wait for it, but without an early griddepcontrol.launch_dependents:
+// the next launch's blocks, placed beside this one's, crowd some SMs' pipes while others
+// idle.  A step of 10,000 nodes of order 6 takes 173 us with it and 108 without, of 40,000
+// 268 and 243, a right-hand side of 4,096 nodes of order 4 23.3 and 11.6; a right-hand side
+// of 1,073 nodes 14.3 us launched plainly and 11.8 so.
 
 template <int G, bool WALL>
-__global__ void LABFM_FIXED_BOUNDS k_fixed_rhs(PlanView<double> P, SoA<double> in, double* __restrict__ out,
+__global__ void LABFM_FIXED_BOUNDS k_fixed_rhs(PlanView<double> P, Fields in, double* __restrict__ out,
                                                Phys<double> ph, int passes) {
     fixed_nodes<G, false>(P, in, passes,
                           [&](int i, double a, double u, double v, const double (&d)[12]) {
@@ -48,7 +48,6 @@ __global__ void LABFM_FIXED_BOUNDS k_fixed_stage(PlanView<double> P, const Packe
                                                  const Packed<double>* Q_in, Packed<double>* Q_out,
                                                  Packed<double>* X_out, double dt, double bk, double ck,
                                                  Phys<double> ph, D8<double>* Dout, int passes) {
-    pdl_start();
     fixed_nodes<G, false>(P, State{X_in}, passes,
                           [&](int i, double a, double u, double v, const double (&d)[12]) {
                               stage_epilogue<double, false, WALL>(P, i, 0, d, a, u, v, X_in, Q_in, Q_out, X_out,
@@ -64,7 +63,6 @@ __global__ void LABFM_FIXED_BOUNDS k_fixed_stage(PlanView<double> P, const Packe
 template <int G>
 __global__ void LABFM_FIXED_BOUNDS k_fixed_coeffs(PlanView<double> P, const Packed<double>* X, D8<double>* Dout,
                                                   int passes) {
-    pdl_start();
     fixed_nodes<G, false>(P, State{X}, passes,
                           [&](int i, double, double, double, const double (&d)[12]) {
                               double c[8];
@@ -76,7 +74,6 @@ __global__ void LABFM_FIXED_BOUNDS k_fixed_coeffs(PlanView<double> P, const Pack
 template <int G>
 __global__ void LABFM_FIXED_FILTER_BOUNDS k_fixed_filter(PlanView<double> P, const Packed<double>* in, Packed<double>* out,
                                                   double* soa, int passes) {
-    pdl_start();
     fixed_nodes<G, true>(P, State{in}, passes,
                          [&](int i, double a, double u, double v, const double (&s)[3]) {
                              store(out, i, a + s[0], u + s[1], v + s[2]);
@@ -89,7 +86,7 @@ __global__ void LABFM_FIXED_FILTER_BOUNDS k_fixed_filter(PlanView<double> P, con
 }
 
 template <int G>
-__global__ void LABFM_FIXED_FILTER_BOUNDS k_fixed_filter_soa(PlanView<double> P, SoA<double> in, double* __restrict__ out,
+__global__ void LABFM_FIXED_FILTER_BOUNDS k_fixed_filter_soa(PlanView<double> P, Fields in, double* __restrict__ out,
                                                       int passes) {
     fixed_nodes<G, true>(P, in, passes,
                          [&](int i, double a, double u, double v, const double (&s)[3]) {
@@ -275,15 +272,20 @@ PlanView<double> view_of(const labfm_plan* p, int64_t n_lo, int64_t n_hi) {
 
 int fixed_rhs(const labfm_plan* p, const void* fields, void* rhs, const labfm_phys& php, int group, cudaStream_t st) {
     const double* f = static_cast<const double*>(fields);
-    const SoA<double> in{f, f + p->N, f + 2 * p->N};
-    const int g = lanes_for(group), passes = passes_for(p->N, g), grid = grid_of(p->N, g, passes);
+    const Fields in{f, f + p->N, f + 2 * p->N};
+    const int g = lanes_for(group), passes = passes_for(p->N, g);
+    const int grid = grid_of(p->N, g, passes);
     double* out = static_cast<double*>(rhs);
+    auto launch = [&](auto* kernel) {
+        return launch_pdl(p, kernel, grid, 32 * kFixedWarps, st, view<double>(p), in, out, phys_of(php), passes);
+    };
+    cudaError_t e = cudaSuccess;
     if (p->wall_slot) {
-        LABFM_FIXED_DISPATCH(g, (k_fixed_rhs<G, true><<<grid, 32 * kFixedWarps, 0, st>>>(view<double>(p), in, out, phys_of(php), passes)));
+        LABFM_FIXED_DISPATCH(g, (e = launch(k_fixed_rhs<G, true>)));
     } else {
-        LABFM_FIXED_DISPATCH(g, (k_fixed_rhs<G, false><<<grid, 32 * kFixedWarps, 0, st>>>(view<double>(p), in, out, phys_of(php), passes)));
+        LABFM_FIXED_DISPATCH(g, (e = launch(k_fixed_rhs<G, false>)));
     }
-    LABFM_LAUNCH_CHECK("fixed-point rhs kernel");
+    if (e != cudaSuccess) return cuda_error(e, "fixed-point rhs kernel");
     return LABFM_OK;
 }
 
@@ -291,7 +293,8 @@ int fixed_stage(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, cons
                 void* qout, void* xout, double dt, double bk, double ck, const labfm_phys& php, void* D,
                 cudaStream_t st) {
     if (n_hi <= n_lo) return LABFM_OK;
-    const int g = lanes_for(group), passes = passes_for(n_hi - n_lo, g), grid = grid_of(n_hi - n_lo, g, passes);
+    const int g = lanes_for(group), passes = passes_for(n_hi - n_lo, g);
+    const int grid = grid_of(n_hi - n_lo, g, passes);
     const PlanView<double> v = view_of(p, n_lo, n_hi);
     auto launch = [&](auto* kernel) {
         return launch_pdl(p, kernel, grid, 32 * kFixedWarps, st, v, static_cast<const Packed<double>*>(xin),
@@ -312,7 +315,8 @@ int fixed_stage(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, cons
 }
 
 int fixed_coeffs(const labfm_plan* p, const void* X, void* D, cudaStream_t st) {
-    const int g = lanes_for(p->group), passes = passes_for(p->N, g), grid = grid_of(p->N, g, passes);
+    const int g = lanes_for(p->group), passes = passes_for(p->N, g);
+    const int grid = grid_of(p->N, g, passes);
     cudaError_t e = cudaSuccess;
     LABFM_FIXED_DISPATCH(g, (e = launch_pdl(p, k_fixed_coeffs<G>, grid, 32 * kFixedWarps, st, view<double>(p),
                                             static_cast<const Packed<double>*>(X), static_cast<D8<double>*>(D), passes)));
@@ -323,7 +327,8 @@ int fixed_coeffs(const labfm_plan* p, const void* X, void* D, cudaStream_t st) {
 int fixed_filter(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, const void* in, void* out, void* soa,
                  cudaStream_t st) {
     if (n_hi <= n_lo) return LABFM_OK;
-    const int g = filter_lanes_for(group), passes = passes_for(n_hi - n_lo, g), grid = grid_of(n_hi - n_lo, g, passes);
+    const int g = filter_lanes_for(group), passes = passes_for(n_hi - n_lo, g);
+    const int grid = grid_of(n_hi - n_lo, g, passes);
     const PlanView<double> v = view_of(p, n_lo, n_hi);
     cudaError_t e = cudaSuccess;
     LABFM_FIXED_DISPATCH(g, (e = launch_pdl(p, k_fixed_filter<G>, grid, 32 * kFixedWarps, st, v, static_cast<const Packed<double>*>(in),
@@ -334,10 +339,13 @@ int fixed_filter(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, con
 
 int fixed_filter_soa(const labfm_plan* p, const void* in, void* out, cudaStream_t st) {
     const double* f = static_cast<const double*>(in);
-    const SoA<double> src{f, f + p->N, f + 2 * p->N};
-    const int g = filter_lanes_for(p->group), passes = passes_for(p->N, g), grid = grid_of(p->N, g, passes);
-    LABFM_FIXED_DISPATCH(g, (k_fixed_filter_soa<G><<<grid, 32 * kFixedWarps, 0, st>>>(view<double>(p), src, static_cast<double*>(out), passes)));
-    LABFM_LAUNCH_CHECK("fixed-point filter kernel");
+    const Fields src{f, f + p->N, f + 2 * p->N};
+    const int g = filter_lanes_for(p->group), passes = passes_for(p->N, g);
+    const int grid = grid_of(p->N, g, passes);
+    cudaError_t e = cudaSuccess;
+    LABFM_FIXED_DISPATCH(g, (e = launch_pdl(p, k_fixed_filter_soa<G>, grid, 32 * kFixedWarps, st, view<double>(p), src,
+                                            static_cast<double*>(out), passes)));
+    if (e != cudaSuccess) return cuda_error(e, "fixed-point filter kernel");
     return LABFM_OK;
 }
 

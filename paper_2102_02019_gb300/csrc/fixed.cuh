@@ -137,11 +137,19 @@ __device__ __forceinline__ void load_cols(const double* w, int64_t off, uint32_t
     c[3] = uint32_t(v.w);
 }
 
-// A packed state that the launch before may write.  Plain loads: read-only ones (__ldg) the
-// compiler may move above the wait for that launch.
+// States that the launch before may write, packed or as three arrays.  Plain loads: read-only
+// ones (__ldg) the compiler may move above the wait for that launch.
 struct State {
     const Packed<double>* p;
     __device__ __forceinline__ void get(int j, double& x, double& y, double& z) const { unpack_rw(p, j, x, y, z); }
+};
+struct Fields {
+    const double *a, *u, *v;
+    __device__ __forceinline__ void get(int j, double& x, double& y, double& z) const {
+        x = a[j];
+        y = u[j];
+        z = v[j];
+    }
 };
 
 // Where the values of one field lie: node j's at p[j * stride].
@@ -150,7 +158,7 @@ struct Column {
     int stride;
     __device__ __forceinline__ double operator[](int j) const { return p[int64_t(j) * stride]; }
 };
-__device__ __forceinline__ Column column(const SoA<double>& f, int k) { return {k == 0 ? f.a : (k == 1 ? f.u : f.v), 1}; }
+__device__ __forceinline__ Column column(const Fields& f, int k) { return {k == 0 ? f.a : (k == 1 ? f.u : f.v), 1}; }
 __device__ __forceinline__ Column column(const State& f, int k) {
     return {reinterpret_cast<const double*>(f.p) + k, 4};
 }
@@ -393,6 +401,7 @@ __device__ __forceinline__ void fixed_nodes(const PlanView<double>& P, const F& 
         if (node - lane / G >= P.n_hi) break;
         const int i = int(node < P.n_hi ? node : P.n_hi - 1);
         const int e0 = P.row_ptr[i], e1 = node < P.n_hi ? P.row_ptr[i + 1] : e0;
+        if (p == 0) pdl_wait();  // nothing before it is written by a launch
         long long hi[LK], lo[LK];
         int T[LT];
         bool cold;
