@@ -257,8 +257,10 @@ def _field_dtype(t: torch.Tensor, name: str, rows: int = 3) -> int:
 
 
 def _stream(stream=None) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    # the raw handle of torch.cuda.current_stream() without its Stream object: 0.3 us for 2.9
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 @dataclass
