@@ -747,8 +747,8 @@ int labfm_conserved_vjp(const void* c, const void* qbar, void* cbar, int64_t N,
 
 /*
  * Domain kinetic energy KE = sum_i 1/2 rho_i |u_i|^2 s_i^2 (node volume s_i^2)
- * of a state q = (ln rho, u, v), summed in FP64 in a fixed order by one block
- * (the same result on every call), into one device double; and
+ * of a state q = (ln rho, u, v), summed in FP64 in a fixed order by one cluster
+ * of blocks (the same result on every call), into one device double; and
  * grad_out = scale * dKE/dq.
  */
 int labfm_kinetic_energy(const void* q, const double* s, int64_t N, labfm_dtype dtype,
@@ -759,8 +759,8 @@ int labfm_kinetic_energy_grad(const void* q, const double* s, int64_t N, labfm_d
 /*
  * Probe-weighted momentum J = sum_i rho_i (px_i u_i + py_i v_i) of a state
  * q = (ln rho, u, v) (px, py: device, N doubles of probe weights, e.g. a smooth
- * bump around a sensor), summed in FP64 in a fixed order by one block into one
- * device double; and grad_out = scale * dJ/dq (the flow objective alternative to
+ * bump around a sensor), summed in FP64 in a fixed order by one cluster of blocks
+ * into one device double; and grad_out = scale * dJ/dq (the flow objective alternative to
  * the kinetic energy for the adjoint; the paper itself has no adjoint).
  */
 int labfm_probe_momentum(const void* q, const double* px, const double* py, int64_t N,

@@ -137,3 +137,28 @@ def test_uniform_fields_give_exact_zeros(lb):
     assert torch.equal(lb.filter(plan, q), q)
     assert not lb.rhs(plan, q, lb.Phys(100.0, 0.1)).any()
     plan.close()
+
+
+@pytest.mark.parametrize("N", [70, 1073, 20000])
+def test_launches_without_a_gap_read_what_came_before(lb, N):
+    # right-hand sides and filters, launched to start as the launch before ends, between
+    # kernels that write their inputs: the same bits as with a synchronisation after each
+    rng = np.random.default_rng(N)
+    rp, col, w, kappa = _operator(N, np.full(N, 24), 1.0, N)
+    plan = _plan(lb, rp, col, w, 1e-3 * kappa)
+    q0 = torch.tensor(rng.standard_normal((3, N)), device="cuda")
+    phys = lb.Phys(1.0, 0.01)
+    out = []
+    for wait, programmatic in ((False, True), (True, True), (False, False)):
+        plan.set_programmatic_launch(programmatic)
+        q = q0.clone()
+        for _ in range(20):
+            r = lb.rhs(plan, q, phys)
+            q = lb.filter(plan, torch.tanh(q + 1e-3 * r))
+            q = lb.filter(plan, q)
+            if wait:
+                torch.cuda.synchronize()
+        out.append(q)
+    assert torch.isfinite(out[0]).all()
+    assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
+    plan.close()
