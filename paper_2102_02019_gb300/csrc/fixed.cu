@@ -230,10 +230,11 @@ __global__ void k_pack_fixed(int64_t N, int64_t nnz, int64_t off, const int32_t*
 // that an instance's sums are the same alone and in a batch.
 int lanes_for(int group) { return std::min(group, 16); }
 
-// The filter gives a lane whole chunks where the right-hand side gives a chunk to two
-// lanes: half the lanes take as many chunks at a time and idle less at the rows' ends
-// (262,144 nodes, order 8: 207 -> 192 us).
-int filter_lanes_for(int group) { return std::max(2, lanes_for(group) / 2); }
+// The filter's lanes likewise.  Half of them, a whole chunk a lane where the right-hand side
+// gives a chunk to two, would idle less at the rows' ends (262,144 nodes, order 8: 188 us for
+// 203), but doubles the serial chain that bounds small plans (4,096 nodes, order 8: 20.6 us
+// for 12.9; 1,600, order 6: 13.8 for 9.5).
+int filter_lanes_for(int group) { return lanes_for(group); }
 
 // Passes per warp: all the lanes' worth (32 nodes a warp, so that the work after the sums
 // runs on 32 lanes: 262,144 nodes of order 8, one pass 463 us, two 411, four 384) where
