@@ -27,7 +27,8 @@
 // 2^+-400, and plans of 2^30 nodes or more, keep the FP64 weights and kernels
 // (plan.wexp == nullptr).  A row whose differences are not finite or beyond 2^+-500 is
 // summed in FP64 from the decoded weights, so that infinities and NaN come out as they
-// would.  Differences below 2^-1022 count as zero.
+// would; so is a row whose differences of a field all lie below 2^-499 and are not all
+// zero.  Beside larger ones, differences below 2^-1022 count as zero.
 #pragma once
 
 #include "gather.cuh"
@@ -38,7 +39,7 @@ namespace {
 constexpr uint32_t kColMask = 0x3fffffffu;  // the column word: s_j in the two bits above
 constexpr int kFixedWarps = 2;  // warps a block
 constexpr int kOne20 = 1 << 20;
-constexpr int kFloorT = 65 << 20;           // T below: no difference but zero seen
+constexpr int kFloorT = 65 << 20;           // T of a field until a difference above it turns up
 constexpr int kLeastT = 524 << 20;          // smallest bound of the fixed-point sums
 constexpr uint32_t kMostT = 1500u << 20;
 
@@ -89,6 +90,15 @@ __device__ __forceinline__ void mac(long long& hi, long long& mid, int w1, int w
     mad_wide(mid, w1, d0);
     mad_wide(mid, w0, d1);
 }
+
+// Non-zero when d is (-0 is zero).
+__device__ __forceinline__ uint32_t not_zero(double d) {
+    return (uint32_t(__double2hiint(d)) << 1) | uint32_t(__double2loint(d));
+}
+
+// Whether a row's sums of a field with bound T need FP64: infinities and NaN aside, those
+// whose differences all lie below the range of the fixed-point sums without being all zero.
+__device__ __forceinline__ bool too_small(int T, uint32_t seen) { return T == kFloorT ? seen != 0 : T < kLeastT; }
 
 // Largest v over the lanes of the group that lie a multiple of STEP apart.
 template <int STEP, int G>
@@ -178,6 +188,7 @@ __device__ __forceinline__ void filter_row(const PlanView<double>& P, const F& f
         hi[f] = mid[f] = 0;
         T[f] = kFloorT;
     }
+    uint32_t seen[3] = {0, 0, 0};  // a difference other than zero
     cold = false;
     int e = e0 + 4 * gl;
 #pragma unroll 1
@@ -199,6 +210,7 @@ __device__ __forceinline__ void filter_row(const PlanView<double>& P, const F& f
 #pragma unroll
             for (int f = 0; f < 3; ++f) {
                 d[f][k] = v[f] - own[f];
+                seen[f] |= not_zero(d[f][k]);
                 t[f][k] = T[f] - exponent20(d[f][k]) - s20[k];
                 low |= t[f][k];
             }
@@ -226,7 +238,8 @@ __device__ __forceinline__ void filter_row(const PlanView<double>& P, const F& f
     }
     fold(hi, mid);
 #pragma unroll
-    for (int f = 0; f < 3; ++f) cold = cold || (T[f] > kFloorT && T[f] < kLeastT);
+    for (int f = 0; f < 3; ++f) cold = cold || too_small(T[f], seen[f]);
+    cold = group_max<1, G>(uint32_t(cold)) != 0;
 }
 
 // The twelve derivative sums of one row over the lanes of its group, two lanes to a chunk:
@@ -244,6 +257,7 @@ __device__ __forceinline__ void rhs_row(const PlanView<double>& P, const F& fld,
 #pragma unroll
     for (int k = 0; k < 7; ++k) hi[k] = mid[k] = 0;
     T[0] = T[1] = kFloorT;
+    uint32_t seen[2] = {0, 0};  // a difference other than zero
     cold = false;
     const char* rec = reinterpret_cast<const char*>(P.w);
     int e = e0 + 4 * (gl >> 1);
@@ -280,12 +294,14 @@ __device__ __forceinline__ void rhs_row(const PlanView<double>& P, const F& fld,
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             d[k] = g[k] - of;
+            seen[1] |= not_zero(d[k]);
             t[k] = T[1] - exponent20(d[k]) - int((cj[k] >> 30) << 20);
             low |= t[k];
         }
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             da[k] = g[4 + k] - oa;
+            seen[0] |= not_zero(da[k]);
             ta[k] = T[0] - exponent20(da[k]) - int(((odd ? cj[k + 2] : cj[k]) >> 30) << 20);
             low |= ta[k];
         }
@@ -328,7 +344,7 @@ __device__ __forceinline__ void rhs_row(const PlanView<double>& P, const F& fld,
     }
     fold(hi, mid);
 #pragma unroll
-    for (int f = 0; f < 2; ++f) cold = cold || (T[f] > kFloorT && T[f] < kLeastT);
+    for (int f = 0; f < 2; ++f) cold = cold || too_small(T[f], seen[f]);
     cold = group_max<1, G>(uint32_t(cold)) != 0;
 }
 

@@ -162,3 +162,28 @@ def test_launches_without_a_gap_read_what_came_before(lb, N):
     assert torch.isfinite(out[0]).all()
     assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
     plan.close()
+
+
+@pytest.mark.parametrize("scale", [2.0 ** -940, 2.0 ** -958, 2.0 ** -963, 2.0 ** -990, 2.0 ** -1012])
+def test_fields_with_tiny_differences_only(lb, scale):
+    # rows whose differences are all below the fixed-point range: the tail of a pulse in
+    # fluid at rest.  FP64's own error: n 2^-53 sum |w d|, and half of 2^-1074 per product
+    rng = np.random.default_rng(11)
+    N = 260
+    rp, col, w, kappa = _operator(N, rng.integers(1, 70, N), 1.0, 12)
+    q = scale * rng.uniform(1.0, 3.0, (3, N))
+    plan = _plan(lb, rp, col, w, kappa)
+    got = lb.filter(plan, torch.tensor(q, device="cuda")).cpu().numpy()
+    r = lb.rhs(plan, torch.tensor(np.stack([0.0 * q[0], q[1], q[2]]), device="cuda"), lb.Phys(0.0, 0.0)).cpu().numpy()
+    for i in range(N):
+        s = slice(rp[i], rp[i + 1])
+        d = (q[:, col[s]] - q[:, i:i + 1]).astype(np.longdouble)
+        n, tiny = rp[i + 1] - rp[i], 2.0 ** -1074
+        wf = (kappa[i] * w[5, s]).astype(np.longdouble)
+        ref, mag = d @ wf, np.abs(d) @ np.abs(wf)
+        assert np.all(np.abs(got[:, i] - (q[:, i] + ref)) <= (n + 2) * (2.0 ** -53 * (mag + np.abs(q[:, i])) + tiny)), i
+        # R of ln rho with ln rho = 0: -(u_x + v_y)
+        ref = -(w[0, s].astype(np.longdouble) @ d[1] + w[1, s].astype(np.longdouble) @ d[2])
+        mag = np.abs(w[0, s]) @ np.abs(d[1]) + np.abs(w[1, s]) @ np.abs(d[2])
+        assert abs(r[0, i] - ref) <= (n + 3) * (2.0 ** -53 * mag + 2 * tiny), i
+    plan.close()
