@@ -105,7 +105,7 @@ __device__ __forceinline__ int entry_shift(int below) {
     return below >= -748983 ? 3 : (below >= -2246949 ? 2 : (below >= -3744915 ? 1 : 0));
 }
 
-// Warp per row: the row's exponents, then its records (columns with s_j, digits).
+// Warp per row: the row's exponents, then its records (columns with s_j, weight words).
 __global__ void k_pack_fixed(int64_t N, int64_t nnz, int64_t off, const int32_t* __restrict__ row_ptr,
                              const int32_t* __restrict__ col, const double* __restrict__ w,
                              const double* __restrict__ kappa, const int32_t* __restrict__ prow,
@@ -138,11 +138,12 @@ __global__ void k_pack_fixed(int64_t N, int64_t nnz, int64_t off, const int32_t*
                 if (top[o] > 0) below = max(below, h[o] - top[o]);
             return entry_shift(below);
         };
-        int exps[6];
+        int exps[6], least[6];  // of |w| 2^-s: the largest and the smallest but zero
         float sum[6];
 #pragma unroll
         for (int o = 0; o < 6; ++o) {
             exps[o] = -2000;
+            least[o] = 4000;
             sum[o] = 0.0f;
         }
         for (int e = lane; e < len; e += 32) {
@@ -158,6 +159,7 @@ __global__ void k_pack_fixed(int64_t N, int64_t nnz, int64_t off, const int32_t*
             for (int o = 0; o < 6; ++o) {
                 const int s = o < 5 ? sr : sf;
                 exps[o] = max(exps[o], (h[o] >> 20) - s - 1022);
+                if (h[o] > 0) least[o] = min(least[o], (h[o] >> 20) - s - 1022);
                 // |w| 2^-s over the power of two above the row's largest |w|
                 const int ex = (h[o] >> 20) - (top[o] >> 20) - s + 126;
                 if (h[o] > 0 && ex > 0) sum[o] += __int_as_float((ex << 23) | ((h[o] & 0xfffff) << 3));
@@ -176,6 +178,7 @@ __global__ void k_pack_fixed(int64_t N, int64_t nnz, int64_t off, const int32_t*
                     a *= 0.5f;
                     ++exps[o];
                 }
+                odd |= exps[o] + 2 - least[o] > kMostAlign;
             }
         }
         odd = __any_sync(0xffffffffu, odd);
@@ -192,9 +195,7 @@ __global__ void k_pack_fixed(int64_t N, int64_t nnz, int64_t off, const int32_t*
         for (int e = lane; e < plen; e += 32) {
             const int64_t dst = int64_t(p0) + entry_slot(e, plen);
             uint32_t c = uint32_t(i), sr = 0, sf = 0;
-            int W1[6], W0[6];
-#pragma unroll
-            for (int o = 0; o < 6; ++o) W1[o] = W0[o] = 0;
+            long long word[6] = {0, 0, 0, 0, 0, 0};
             if (e < len) {
                 const int64_t src = int64_t(r0) + e;
                 c = uint32_t(off + col[src]);
@@ -208,18 +209,12 @@ __global__ void k_pack_fixed(int64_t N, int64_t nnz, int64_t off, const int32_t*
                 sr = uint32_t(shift_of(h, 0, 5));
                 sf = uint32_t(shift_of(h, 5, 6));
 #pragma unroll
-                for (int o = 0; o < 6; ++o) {
-                    const long long W = __double2ll_rn(v[o] * pow2(56 - exps[o] - int(o < 5 ? sr : sf)));
-                    W1[o] = int((W + (1ll << 27)) >> 28);
-                    W0[o] = int(W - ((long long)W1[o] << 28));
-                }
+                for (int o = 0; o < 6; ++o) word[o] = weight_word(v[o], exps[o], int(o < 5 ? sr : sf));
             }
             *reinterpret_cast<uint32_t*>(rb + Rec<double>::col_e(dst)) = c | (sr << 30);
             *reinterpret_cast<uint32_t*>(fb + Rec<double>::fcol_e(dst)) = c | (sf << 30);
 #pragma unroll
-            for (int o = 0; o < 6; ++o) {
-                *reinterpret_cast<int2*>((o < 5 ? rb : fb) + fixed_at(dst, o)) = make_int2(W1[o], W0[o]);
-            }
+            for (int o = 0; o < 6; ++o) *reinterpret_cast<long long*>((o < 5 ? rb : fb) + fixed_at(dst, o)) = word[o];
         }
     }
 }

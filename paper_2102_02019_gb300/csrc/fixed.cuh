@@ -7,12 +7,16 @@
 // differences d = phi_j - phi_i are taken in FP64 (as before, rounded once); the products
 // and sums run on integers:
 //
-//   weights, once when the plan is packed:  w_ji 2^-s_j ~ (w1 2^28 + w0) 2^(E_w - 56),
-//     w1 2^28 + w0 = rint(.), |w0| <= 2^27, E_w per row and operator;
-//   differences, per entry:  |d| 2^s_j ~ (d1 2^28 + d0) 2^(E_d - 57), truncated,
-//     0 <= d0 < 2^28, E_d per row and field, raised as larger differences turn up;
+//   weights:  w_ji 2^-s_j ~ (w1 2^28 + w0) 2^(E_w - 56), rounded, 0 <= w0 < 2^28,
+//     E_w per row and operator;
+//   differences:  |d| 2^s_j ~ (d1 2^28 + d0) 2^(E_d - 57), truncated, |d0| <= 2^27,
+//     E_d per row and field, raised as larger differences turn up;
 //   sum_j w_ji d_j ~ 2^(E_w + E_d - 113 + 28) (2^28 sum w1 d1 + sum (w1 d0 + w0 d1)),
-//     two exact 64-bit sums; w0 d0 (below 2^-57 of the bounds) is dropped.
+//     two exact 64-bit sums; w0 d0 (below 2^-57 of the bounds, and of either sign) is dropped.
+//
+// The plan keeps the FP64 weights themselves, bit for bit, in the form that gives these
+// digits with five instructions (weight_word): their 53 bits and the shift that aligns
+// them to E_w.  The FP64 fallback and the adjoint read them back exactly.
 //
 // The shift s_j (0 to 3, two bits of the column word) is the same for an entry's weights
 // and its difference and cancels: it moves the large weights near the node, where the
@@ -22,11 +26,11 @@
 // 0.93 at most.
 //
 // No overflow: E_w is raised until sum_j |w_ji| 2^-s_j <= 32 2^E_w, so |sum w1 d1| <=
-// 2^(5 + 28 + 29) over a whole row; |sum (w1 d0 + w0 d1)| <= 2^61 + n 2^56 over n entries,
-// whose carries a lane moves up after every 64.  Weights that are not finite or beyond
-// 2^+-400, and plans of 2^30 nodes or more, keep the FP64 weights and kernels
+// 2^(5 + 28 + 29) over a whole row; |sum (w1 d0 + w0 d1)| <= 2^60 + n 2^57 over n entries,
+// whose carries a lane moves up after every 32.  Weights that are not finite, beyond
+// 2^+-400 or below 2^-500 of their row's largest, and plans of 2^30 nodes or more, keep the FP64 weights and kernels
 // (plan.wexp == nullptr).  A row whose differences are not finite or beyond 2^+-500 is
-// summed in FP64 from the decoded weights, so that infinities and NaN come out as they
+// summed in FP64, so that infinities and NaN come out as they
 // would; so is a row whose differences of a field all lie below 2^-499 and are not all
 // zero.  Beside larger ones, differences below 2^-1022 count as zero.
 #pragma once
@@ -58,7 +62,8 @@ __device__ __forceinline__ int exponent20(double d) { return __double2hiint(d) &
 
 // Digits of d for t = T - exponent20(d) - s 2^20 >= 0, T = (E_d - 1) 2^20 (biased): the 53
 // significant bits, leading bit at 60, shifted down by t / 2^20; shifts of 64 and more
-// give zero, so a zero difference (exponent field 0) does.
+// give zero, so a zero difference (exponent field 0) does.  The high digit is rounded, the
+// low one signed, so that the dropped products w0 d0 have no mean.
 __device__ __forceinline__ void digits(double d, int t, int& d1, int& d0) {
     const int h = __double2hiint(d), l = __double2loint(d);
     const uint32_t sh = uint32_t(t) >> 20;
@@ -69,8 +74,42 @@ __device__ __forceinline__ void digits(double d, int t, int& d1, int& d0) {
     asm("shr.u32 %0, %1, %2;" : "=r"(top) : "r"(x1), "r"(sh));
     asm("shr.u64 %0, %1, %2;" : "=l"(low) : "l"(x), "r"(sh));
     const int sign = (h >> 31) | 1;
-    d1 = int(top) * sign;
-    d0 = int(uint32_t(low) >> 4) * sign;
+    d1 = int(top + (uint32_t(low) >> 31)) * sign;
+    d0 = (int(uint32_t(low)) >> 4) * sign;
+}
+
+// A weight w = M 2^(ex - 52), |M| in [2^52, 2^53), in a row and operator of bound E and at
+// an entry of shift s.  With the alignment t = 1 + E + s - ex (2 for the largest weights,
+// kMostAlign at most) in the low nine bits of the word and M above them, the digits are
+// bits t + 32 and up and bits t + 4 to t + 31 of the word: what lies below is rounded by
+// adding its half beforehand, at bit t + 3 (nothing is lost by t < 6).  From kNoDigits on
+// the digits are zero: the word is M + 2^53, not negative, which the shifts clear.
+constexpr int kNoDigits = 59;
+constexpr int kMostAlign = 511;
+__device__ __forceinline__ long long weight_word(double w, int E, int s) {
+    const long long b = __double_as_longlong(w);
+    if ((b << 1) == 0) return 0;
+    const int t = 1 + E + s - (int((b >> 52) & 0x7ff) - 1023);
+    const long long mag = (b & 0xfffffffffffffll) | (1ll << 52);
+    const long long M = b < 0 ? -mag : mag;
+    if (t >= kNoDigits) return ((M + (1ll << 53)) << 9) | t;
+    return (M * 512 + (t >= 6 ? 1ll << (t + 3) : 0)) | t;
+}
+__device__ __forceinline__ double word_weight(long long word, int E, int s) {
+    const int t = int(word) & 511;
+    const long long M = t < kNoDigits ? (word - (t >= 6 ? 1ll << (t + 3) : 0)) >> 9 : (word >> 9) - (1ll << 53);
+    if (M == 0) return 0.0;
+    const long long mag = M < 0 ? -M : M;
+    return __longlong_as_double((M < 0 ? 1ll << 63 : 0) | ((long long)(1 + E + s - t + 1023) << 52) |
+                                (mag & 0xfffffffffffffll));
+}
+// The digits of the word (lo, hi).
+__device__ __forceinline__ void weight_digits(int lo, int hi, int& w1, int& w0) {
+    const int t = lo & 511;
+    long long low;
+    asm("shr.s32 %0, %1, %2;" : "=r"(w1) : "r"(hi), "r"(t));
+    asm("shr.s64 %0, %1, %2;" : "=l"(low) : "l"((static_cast<long long>(hi) << 32) | uint32_t(lo)), "r"(t));
+    w0 = int(uint32_t(low) >> 4);
 }
 
 // s += a b, 32 x 32 + 64 bits.  As a carry pair, which the assembler makes one wide
@@ -227,13 +266,16 @@ __device__ __forceinline__ void filter_row(const PlanView<double>& P, const F& f
             }
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
+        for (int k = 0; k < 4; ++k) {
+            int w1, w0;
+            weight_digits(w[2 * k], w[2 * k + 1], w1, w0);
 #pragma unroll
             for (int f = 0; f < 3; ++f) {
                 int d1, d0;
                 digits(d[f][k], t[f][k], d1, d0);
-                mac(hi[f], mid[f], w[2 * k], w[2 * k + 1], d1, d0);
+                mac(hi[f], mid[f], w1, w0, d1, d0);
             }
+        }
         if (it % kFold == kFold - 1) fold(hi, mid);
     }
     fold(hi, mid);
@@ -319,7 +361,7 @@ __device__ __forceinline__ void rhs_row(const PlanView<double>& P, const F& fld,
 #pragma unroll
             for (int k = 0; k < 2; ++k) ta[k] += T[0] - T0;
         }
-        int last[8];  // the fifth operator's digits of the four entries
+        int last[8];  // the fifth operator's words of the four entries
         ld8i(rec + Rec<double>::w(c, 4), last);
 #pragma unroll
         for (int k = 0; k < 2; ++k) {  // entries k and k + 2
@@ -328,11 +370,19 @@ __device__ __forceinline__ void rhs_row(const PlanView<double>& P, const F& fld,
             ld8i(rec + Rec<double>::w(c, k + 2), w[1]);
 #pragma unroll
             for (int z = 0; z < 2; ++z) {
-                int d1, d0;
+                int d1, d0, w1, w0;
                 digits(d[k + 2 * z], t[k + 2 * z], d1, d0);
 #pragma unroll
-                for (int o = 0; o < 4; ++o) mac(hi[2 + o], mid[2 + o], w[z][2 * o], w[z][2 * o + 1], d1, d0);
-                mac(hi[6], mid[6], last[2 * (k + 2 * z)], last[2 * (k + 2 * z) + 1], d1, d0);
+                for (int o = 0; o < 4; ++o) {
+                    weight_digits(w[z][2 * o], w[z][2 * o + 1], w1, w0);
+                    mac(hi[2 + o], mid[2 + o], w1, w0, d1, d0);
+                    if (o < 2) {  // for ln rho
+                        w[z][2 * o] = w1;
+                        w[z][2 * o + 1] = w0;
+                    }
+                }
+                weight_digits(last[2 * (k + 2 * z)], last[2 * (k + 2 * z) + 1], w1, w0);
+                mac(hi[6], mid[6], w1, w0, d1, d0);
             }
             int a1, a0;
             digits(da[k], ta[k], a1, a0);
@@ -348,7 +398,7 @@ __device__ __forceinline__ void rhs_row(const PlanView<double>& P, const F& fld,
     cold = group_max<1, G>(uint32_t(cold)) != 0;
 }
 
-// Byte offset of the digits (w1, w0) of operator o (5: the filter's kappa w^hyp) at entry e
+// Byte offset of the weight word of operator o (5: the filter's kappa w^hyp) at entry e
 // in the RHS (o < 5) or filter records.  The five 32-byte segments of a chunk hold its four
 // entries' first four operators, entry by entry, then the fifth operator of all four, so
 // that a lane needs one entry's words at a time (operator by operator, as the FP64 records
@@ -367,12 +417,11 @@ __device__ __forceinline__ uint32_t fixed_col_word(const PlanView<double>& P, in
 // Weight of operator o at entry e of row i of a fixed-point plan.
 __device__ __forceinline__ double fixed_weight(const PlanView<double>& P, int i, int e, int o) {
     const char* rec = o == 5 ? reinterpret_cast<const char*>(P.wf) : reinterpret_cast<const char*>(P.w);
-    const int2 v = *reinterpret_cast<const int2*>(rec + fixed_at(e, o));
-    const long long W = ((long long)v.x << 28) + v.y;
-    return double(W) * pow2(P.wexp[int64_t(i) * 8 + o] - 56 + int(fixed_col_word(P, e, o == 5) >> 30));
+    return word_weight(*reinterpret_cast<const long long*>(rec + fixed_at(e, o)), P.wexp[int64_t(i) * 8 + o],
+                       int(fixed_col_word(P, e, o == 5) >> 30));
 }
 
-// Row i in FP64 from its decoded weights, by one lane.
+// Row i in FP64, by one lane.
 template <bool FILTER, int K, class F>
 __device__ __noinline__ void cold_row(const PlanView<double>& P, const F& fld, int i, double (&sum)[K]) {
     constexpr int KA = FILTER ? 1 : 2, KV = FILTER ? 1 : 5;

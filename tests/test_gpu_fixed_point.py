@@ -187,3 +187,40 @@ def test_fields_with_tiny_differences_only(lb, scale):
         mag = np.abs(w[0, s]) @ np.abs(d[1]) + np.abs(w[1, s]) @ np.abs(d[2])
         assert abs(r[0, i] - ref) <= (n + 3) * (2.0 ** -53 * mag + 2 * tiny), i
     plan.close()
+
+
+@pytest.mark.parametrize("spread", [5, 15, 40, 140])
+def test_weights_are_held_bit_for_bit(lb, spread):
+    # weights over `spread` decades within a row, read back one by one: a field that is zero
+    # but at one node gives the weights on that node times a power of two (2^-700: below the
+    # fixed-point range, so in FP64), and the adjoint of one output gives its row
+    rng = np.random.default_rng(spread)
+    N = 90
+    lengths = rng.integers(1, 80, N)
+    rp, col, w, kappa = _operator(N, lengths, 1.0, 13)
+    w *= 10.0 ** rng.uniform(5 - spread, 0, w.shape)
+    col = np.concatenate([np.sort(rng.choice([j for j in range(N) if j != i], n, replace=False))
+                          for i, n in enumerate(lengths)]).astype(np.int32)
+    plan = _plan(lb, rp, col, w, kappa)
+    lb.enable_adjoint(plan)
+    row = np.repeat(np.arange(N), lengths)
+    zero = np.zeros((3, N))
+    for j in range(0, N, 7):
+        on = col == j
+        rows = row[on]
+        q = zero.copy()
+        q[1, j] = 2.0 ** -700
+        out = lb.filter(plan, torch.tensor(q, device="cuda")).cpu().numpy()
+        assert np.array_equal(out[1, rows], kappa[rows] * w[5, on] * 2.0 ** -700)
+        out = lb.rhs(plan, torch.tensor(q, device="cuda"), lb.Phys(0.0, 0.0)).cpu().numpy()
+        assert np.array_equal(out[0, rows], -w[0, on] * 2.0 ** -700)
+        # R_a = -(u_x + v_y), R_u = -c^2 a_x at rest
+        lam = zero.copy()
+        lam[0, j] = 1.0
+        g = lb.rhs_adjoint(plan, torch.tensor(zero, device="cuda"), torch.tensor(lam, device="cuda"),
+                           lb.Phys(1.0, 0.0)).cpu().numpy()
+        on = row == j
+        assert np.array_equal(g[1, col[on]], -w[0, on]) and np.array_equal(g[2, col[on]], -w[1, on])
+        g = lb.filter_adjoint(plan, torch.tensor(lam, device="cuda")).cpu().numpy()
+        assert np.array_equal(g[0, col[on]], kappa[j] * w[5, on])
+    plan.close()
