@@ -12,12 +12,13 @@
 namespace labfm {
 namespace {
 
-// Resident warps per SM that the registers allow for (96 and 64 registers).
+// Resident warps per SM that the registers allow for (96 registers; the filter spills 240
+// bytes in 72, and 262,144 nodes of order 8 take 230 us with 28 warps and 225 with 20).
 #ifndef LABFM_FIXED_RHS_WARPS
 #define LABFM_FIXED_RHS_WARPS 20
 #endif
 #ifndef LABFM_FIXED_FILTER_WARPS
-#define LABFM_FIXED_FILTER_WARPS 28
+#define LABFM_FIXED_FILTER_WARPS 20
 #endif
 #define LABFM_FIXED_BOUNDS __launch_bounds__(32 * kFixedWarps, LABFM_FIXED_RHS_WARPS / kFixedWarps)
 #define LABFM_FIXED_FILTER_BOUNDS __launch_bounds__(32 * kFixedWarps, LABFM_FIXED_FILTER_WARPS / kFixedWarps)
@@ -189,7 +190,9 @@ __global__ void k_pack_fixed(int64_t N, int64_t nnz, int64_t off, const int32_t*
             v.x = (exps[0] & 0xffff) | (exps[1] << 16);
             v.y = (exps[2] & 0xffff) | (exps[3] << 16);
             v.z = (exps[4] & 0xffff) | (exps[5] << 16);
-            v.w = 0;
+            v.w = 0;  // the operators that are zero throughout the row
+#pragma unroll
+            for (int o = 0; o < 6; ++o) v.w |= top[o] == 0 ? 1 << o : 0;
             reinterpret_cast<int4*>(wexp)[i] = v;
         }
         for (int e = lane; e < plen; e += 32) {
@@ -237,7 +240,7 @@ int filter_lanes_for(int group) { return lanes_for(group); }
 // over the chip (40,000 nodes of order 6: one pass 69 us, two 58, four 78).
 int passes_for(int64_t nodes, int g) {
     int passes = g;
-    while (passes > 1 && nodes * g / (32 * passes) < int64_t(152) * LABFM_FIXED_RHS_WARPS / 2) passes /= 2;
+    while (passes > 1 && nodes * g / (32 * passes) < int64_t(152) * 10) passes /= 2;
     return passes;
 }
 

@@ -20,19 +20,31 @@
 //
 // The shift s_j (0 to 3, two bits of the column word) is the same for an entry's weights
 // and its difference and cancels: it moves the large weights near the node, where the
-// differences are small, down and those differences up, which gains two bits.  Against
-// exact sums, on jittered lattices of orders 4 to 10 (120 rows each, every operator and
-// field), the error of these sums is 0.12-0.69 of the FP64 sums' it replaces on average,
-// 0.93 at most.
+// differences are small, down and those differences up, which gains two bits.
+//
+// The error of such a sum over n entries is at most (24 + n) 2^-56 2^(E_w + E_d): relative
+// to the bounds, where FP64's is relative to sum |w d|.  So the lanes add up the leading bits
+// of |w1| |d1| (four entries an instruction) as they go, and a row where that lower bound of
+// sum |w d| is below 1/8 of 2^(E_w + E_d) for any operator and field is summed in FP64
+// instead.  What is left is within (24 + n) 2^-53 sum |w d|, FP64's own a priori bound,
+// whatever the fields.  Against exact sums on jittered lattices of orders 4 to 10 (100 rows
+// each, every operator and field), in units of 2^-53 sum |w d|: smooth fields 0.03-0.05 on
+// average and 0.36 at most (FP64 0.24-0.32, 2.2), white noise 0.04-0.06 and 0.6 (0.36-0.44,
+// 2.5), and of the rows that pass in log-normal fields, fronts, pulses and impulses 0.04-0.37
+// and 1.7 (0.24-1.2, 5.9).  Smooth fields pass on all rows but one in a thousand, noise on
+// all but 3 % at order 4 and all from order 6 on; fronts and pulses on a fifth to two fifths,
+// the rest of which costs as much again as FP64 kernels would.  The sizes take the
+// right-hand side of 262,144 nodes of order 8 from 403 to 434 us (490 as a high product of
+// every entry).
 //
 // No overflow: E_w is raised until sum_j |w_ji| 2^-s_j <= 32 2^E_w, so |sum w1 d1| <=
 // 2^(5 + 28 + 29) over a whole row; |sum (w1 d0 + w0 d1)| <= 2^60 + n 2^57 over n entries,
 // whose carries a lane moves up after every 32.  Weights that are not finite, beyond
-// 2^+-400 or below 2^-500 of their row's largest, and plans of 2^30 nodes or more, keep the FP64 weights and kernels
-// (plan.wexp == nullptr).  A row whose differences are not finite or beyond 2^+-500 is
-// summed in FP64, so that infinities and NaN come out as they
-// would; so is a row whose differences of a field all lie below 2^-499 and are not all
-// zero.  Beside larger ones, differences below 2^-1022 count as zero.
+// 2^+-400 or below 2^-500 of their row's largest, and plans of 2^30 nodes or more, keep the
+// FP64 weights and kernels (plan.wexp == nullptr).  A row whose differences are not finite
+// or beyond 2^477 is summed in FP64 too, so that infinities and NaN come out as they would,
+// and one whose differences of a field all lie below 2^-499 without being all zero.  Beside
+// larger ones, differences below 2^-1022 count as zero.
 #pragma once
 
 #include "gather.cuh"
@@ -42,10 +54,10 @@ namespace {
 
 constexpr uint32_t kColMask = 0x3fffffffu;  // the column word: s_j in the two bits above
 constexpr int kFixedWarps = 2;  // warps a block
-constexpr int kOne20 = 1 << 20;
 constexpr int kFloorT = 65 << 20;           // T of a field until a difference above it turns up
 constexpr int kLeastT = 524 << 20;          // smallest bound of the fixed-point sums
 constexpr uint32_t kMostT = 1500u << 20;
+constexpr uint32_t kLeastSize = 64;         // 1/8 of the bounds' product, in units of 2^-9 of it
 
 __device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
 
@@ -64,7 +76,7 @@ __device__ __forceinline__ int exponent20(double d) { return __double2hiint(d) &
 // significant bits, leading bit at 60, shifted down by t / 2^20; shifts of 64 and more
 // give zero, so a zero difference (exponent field 0) does.  The high digit is rounded, the
 // low one signed, so that the dropped products w0 d0 have no mean.
-__device__ __forceinline__ void digits(double d, int t, int& d1, int& d0) {
+__device__ __forceinline__ void digits(double d, int t, int& d1, int& d0, uint32_t& size) {
     const int h = __double2hiint(d), l = __double2loint(d);
     const uint32_t sh = uint32_t(t) >> 20;
     const uint32_t x1 = (__funnelshift_l(uint32_t(l), uint32_t(h), 8) & 0x1fffffffu) | 0x10000000u;
@@ -74,7 +86,8 @@ __device__ __forceinline__ void digits(double d, int t, int& d1, int& d0) {
     asm("shr.u32 %0, %1, %2;" : "=r"(top) : "r"(x1), "r"(sh));
     asm("shr.u64 %0, %1, %2;" : "=l"(low) : "l"(x), "r"(sh));
     const int sign = (h >> 31) | 1;
-    d1 = int(top + (uint32_t(low) >> 31)) * sign;
+    size = top + (uint32_t(low) >> 31);  // |d1|
+    d1 = int(size) * sign;
     d0 = (int(uint32_t(low)) >> 4) * sign;
 }
 
@@ -130,14 +143,43 @@ __device__ __forceinline__ void mac(long long& hi, long long& mid, int w1, int w
     mad_wide(mid, w0, d1);
 }
 
+// Bytes of x and y (prmt: 0-3 of x, 4-7 of y, + 8 its sign throughout).
+template <int SEL>
+__device__ __forceinline__ uint32_t bytes_of(uint32_t x, uint32_t y) {
+    uint32_t v;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(v) : "r"(x), "r"(y), "n"(SEL));
+    return v;
+}
+// The leading bytes of four digits: 0 to 16 of a weight's magnitude (|w1| <= 2^28, rounded
+// down), 0 to 32 of a difference's.
+__device__ __forceinline__ uint32_t leading(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    return bytes_of<0x5410>(bytes_of<0x73>(a, b), bytes_of<0x73>(c, d));
+}
+__device__ __forceinline__ uint32_t magnitudes(uint32_t v) { return v ^ bytes_of<0xba98>(v, v); }
+
 // Non-zero when d is (-0 is zero).
 __device__ __forceinline__ uint32_t not_zero(double d) {
     return (uint32_t(__double2hiint(d)) << 1) | uint32_t(__double2loint(d));
 }
 
-// Whether a row's sums of a field with bound T need FP64: infinities and NaN aside, those
-// whose differences all lie below the range of the fixed-point sums without being all zero.
-__device__ __forceinline__ bool too_small(int T, uint32_t seen) { return T == kFloorT ? seen != 0 : T < kLeastT; }
+// Whether a row needs FP64 for the sums of a field with bound T over K operators, the first
+// of them `first`: its differences lie below the range of the fixed-point sums without being
+// all zero, or span too many bits for an operator that is not zero throughout the row.
+template <int K>
+__device__ __forceinline__ bool out_of_range(int T, uint32_t seen, const uint32_t* size, int first, int zero_ops) {
+    if (T == kFloorT) return seen != 0;
+    bool out = T < kLeastT;
+#pragma unroll
+    for (int k = 0; k < K; ++k) out |= size[k] < kLeastSize && !(zero_ops >> (first + k) & 1);
+    return out;
+}
+
+template <int STEP, int G>
+__device__ __forceinline__ uint32_t group_add(uint32_t v) {
+#pragma unroll
+    for (int off = G / 2; off >= STEP; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    return v;
+}
 
 // Largest v over the lanes of the group that lie a multiple of STEP apart.
 template <int STEP, int G>
@@ -151,18 +193,20 @@ __device__ __forceinline__ uint32_t group_max(uint32_t v) {
 // exponent m (over the group) exceeds it (and only then: other rows of the warp do not
 // change a row's sums), shifting the K sums taken so far.
 template <int K>
-__device__ __forceinline__ void raise_bound(uint32_t m, int& T, long long* hi, long long* mid, bool& cold) {
+__device__ __forceinline__ void raise_bound(uint32_t m, int& T, long long* hi, long long* mid, uint32_t* size,
+                                            bool& cold) {
     if (m <= uint32_t(T)) return;
     if (m >= kMostT) {
         cold = true;
         return;
     }
-    const int by = min((int(m) + kOne20 - T) >> 20, 63);
-    T = int(m) + kOne20;
+    const int by = min((int(m) - T) >> 20, 63);
+    T = int(m);
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         hi[k] >>= by;
         mid[k] >>= by;
+        size[k] >>= min(by, 31);
     }
 }
 
@@ -213,12 +257,13 @@ __device__ __forceinline__ Column column(const State& f, int k) {
 }
 
 // The filter's sums of one row over the lanes of its group, kappa w^hyp on three fields.
-// hi, mid: this lane's sums; T: the three bounds; cold (the same in the whole group): the
-// row needs FP64.  Every lane of the warp takes the same number of iterations (a lane
+// hi, mid: this lane's sums; T: the three bounds; zero_ops: the operators (bits) that are zero
+// throughout the row; cold (the same in the whole group): the row needs FP64.  Every lane of the warp takes the same number of iterations (a lane
 // without a chunk adds zeros).
 template <int G, class F>
 __device__ __forceinline__ void filter_row(const PlanView<double>& P, const F& fld, int i, int e0, int e1, int gl,
-                                           long long (&hi)[3], long long (&mid)[3], int (&T)[3], bool& cold) {
+                                           int zero_ops, long long (&hi)[3], long long (&mid)[3], int (&T)[3],
+                                           bool& cold) {
     const int trips = __reduce_max_sync(0xffffffffu, (e1 - e0 + 4 * G - 1) / (4 * G));
     double own[3];
     fld.get(i, own[0], own[1], own[2]);
@@ -228,6 +273,7 @@ __device__ __forceinline__ void filter_row(const PlanView<double>& P, const F& f
         T[f] = kFloorT;
     }
     uint32_t seen[3] = {0, 0, 0};  // a difference other than zero
+    uint32_t size[3] = {0, 0, 0};  // sum |w1 d1|
     cold = false;
     int e = e0 + 4 * gl;
 #pragma unroll 1
@@ -260,27 +306,33 @@ __device__ __forceinline__ void filter_row(const PlanView<double>& P, const F& f
                 uint32_t m = 0;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) m = max(m, uint32_t(exponent20(d[f][k])) + uint32_t(s20[k]));
-                raise_bound<1>(group_max<1, G>(m), T[f], hi + f, mid + f, cold);
+                raise_bound<1>(group_max<1, G>(m), T[f], hi + f, mid + f, size + f, cold);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) t[f][k] = T[f] - exponent20(d[f][k]) - s20[k];
             }
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            int w1, w0;
-            weight_digits(w[2 * k], w[2 * k + 1], w1, w0);
+        for (int k = 0; k < 4; ++k) weight_digits(w[2 * k], w[2 * k + 1], w[2 * k], w[2 * k + 1]);
+        const uint32_t wm = magnitudes(leading(w[0], w[2], w[4], w[6]));
 #pragma unroll
-            for (int f = 0; f < 3; ++f) {
+        for (int f = 0; f < 3; ++f) {
+            uint32_t u1[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
                 int d1, d0;
-                digits(d[f][k], t[f][k], d1, d0);
-                mac(hi[f], mid[f], w1, w0, d1, d0);
+                digits(d[f][k], t[f][k], d1, d0, u1[k]);
+                mac(hi[f], mid[f], w[2 * k], w[2 * k + 1], d1, d0);
             }
+            size[f] = __dp4a(wm, leading(u1[0], u1[1], u1[2], u1[3]), size[f]);
         }
         if (it % kFold == kFold - 1) fold(hi, mid);
     }
     fold(hi, mid);
 #pragma unroll
-    for (int f = 0; f < 3; ++f) cold = cold || too_small(T[f], seen[f]);
+    for (int f = 0; f < 3; ++f) {
+        const uint32_t all = group_add<1, G>(size[f]);
+        cold |= out_of_range<1>(T[f], seen[f], &all, 5, zero_ops);
+    }
     cold = group_max<1, G>(uint32_t(cold)) != 0;
 }
 
@@ -291,13 +343,15 @@ __device__ __forceinline__ void filter_row(const PlanView<double>& P, const F& f
 // bounds of ln rho and of the lane's own field.
 template <int G, class F>
 __device__ __forceinline__ void rhs_row(const PlanView<double>& P, const F& fld, int i, int e0, int e1, int gl,
-                                        long long (&hi)[7], long long (&mid)[7], int (&T)[2], bool& cold) {
+                                        int zero_ops, long long (&hi)[7], long long (&mid)[7], int (&T)[2],
+                                        bool& cold) {
     const int trips = __reduce_max_sync(0xffffffffu, (e1 - e0 + 2 * G - 1) / (2 * G));
     const bool odd = gl & 1;
     const Column fa = column(fld, 0), ff = column(fld, odd ? 2 : 1);
     const double oa = fa[i], of = ff[i];
 #pragma unroll
     for (int k = 0; k < 7; ++k) hi[k] = mid[k] = 0;
+    uint32_t size[7] = {0, 0, 0, 0, 0, 0, 0};  // sum |w1 d1|
     T[0] = T[1] = kFloorT;
     uint32_t seen[2] = {0, 0};  // a difference other than zero
     cold = false;
@@ -354,47 +408,72 @@ __device__ __forceinline__ void rhs_row(const PlanView<double>& P, const F& fld,
             for (int k = 0; k < 4; ++k) m = max(m, uint32_t(T1) - uint32_t(t[k]));
 #pragma unroll
             for (int k = 0; k < 2; ++k) ma = max(ma, uint32_t(T0) - uint32_t(ta[k]));
-            raise_bound<2>(group_max<1, G>(ma), T[0], hi, mid, cold);
-            raise_bound<5>(group_max<2, G>(m), T[1], hi + 2, mid + 2, cold);
+            raise_bound<2>(group_max<1, G>(ma), T[0], hi, mid, size, cold);
+            raise_bound<5>(group_max<2, G>(m), T[1], hi + 2, mid + 2, size + 2, cold);
 #pragma unroll
             for (int k = 0; k < 4; ++k) t[k] += T[1] - T1;
 #pragma unroll
             for (int k = 0; k < 2; ++k) ta[k] += T[0] - T0;
         }
-        int last[8];  // the fifth operator's words of the four entries
-        ld8i(rec + Rec<double>::w(c, 4), last);
+        // digits of the differences (entries 0, 2, 1, 3), and their leading bytes for the sizes
+        int d1[4], d0[4], a1[2], a0[2];
+        uint32_t um, am;
+        {
+            uint32_t u[4], v[2];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int q = 2 * (k & 1) + (k >> 1);
+                digits(d[q], t[q], d1[k], d0[k], u[k]);
+            }
+#pragma unroll
+            for (int k = 0; k < 2; ++k) digits(da[k], ta[k], a1[k], a0[k], v[k]);
+            um = leading(u[0], u[1], u[2], u[3]);
+            am = bytes_of<0x7733>(v[0], v[1]) & (odd ? 0xff00ff00u : 0x00ff00ffu);
+        }
+        uint32_t wm[5];
 #pragma unroll
         for (int k = 0; k < 2; ++k) {  // entries k and k + 2
             int w[2][8];
             ld8i(rec + Rec<double>::w(c, k), w[0]);
             ld8i(rec + Rec<double>::w(c, k + 2), w[1]);
 #pragma unroll
-            for (int z = 0; z < 2; ++z) {
-                int d1, d0, w1, w0;
-                digits(d[k + 2 * z], t[k + 2 * z], d1, d0);
+            for (int o = 0; o < 4; ++o) {
 #pragma unroll
-                for (int o = 0; o < 4; ++o) {
-                    weight_digits(w[z][2 * o], w[z][2 * o + 1], w1, w0);
-                    mac(hi[2 + o], mid[2 + o], w1, w0, d1, d0);
-                    if (o < 2) {  // for ln rho
-                        w[z][2 * o] = w1;
-                        w[z][2 * o + 1] = w0;
-                    }
+                for (int z = 0; z < 2; ++z) {
+                    weight_digits(w[z][2 * o], w[z][2 * o + 1], w[z][2 * o], w[z][2 * o + 1]);
+                    mac(hi[2 + o], mid[2 + o], w[z][2 * o], w[z][2 * o + 1], d1[2 * k + z], d0[2 * k + z]);
                 }
-                weight_digits(last[2 * (k + 2 * z)], last[2 * (k + 2 * z) + 1], w1, w0);
-                mac(hi[6], mid[6], w1, w0, d1, d0);
+                const uint32_t m = bytes_of<0x73>(w[0][2 * o], w[1][2 * o]);
+                wm[o] = k == 0 ? m : bytes_of<0x5410>(wm[o], m);
             }
-            int a1, a0;
-            digits(da[k], ta[k], a1, a0);
 #pragma unroll
             for (int o = 0; o < 2; ++o)
-                mac(hi[o], mid[o], odd ? w[1][2 * o] : w[0][2 * o], odd ? w[1][2 * o + 1] : w[0][2 * o + 1], a1, a0);
+                mac(hi[o], mid[o], odd ? w[1][2 * o] : w[0][2 * o], odd ? w[1][2 * o + 1] : w[0][2 * o + 1], a1[k], a0[k]);
+        }
+        {
+            int w[8];  // the fifth operator's words of the four entries
+            ld8i(rec + Rec<double>::w(c, 4), w);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int q = 2 * (2 * (k & 1) + (k >> 1));
+                weight_digits(w[q], w[q + 1], w[q], w[q + 1]);
+                mac(hi[6], mid[6], w[q], w[q + 1], d1[k], d0[k]);
+            }
+            wm[4] = leading(w[0], w[4], w[2], w[6]);
+        }
+#pragma unroll
+        for (int o = 0; o < 5; ++o) {
+            wm[o] = magnitudes(wm[o]);
+            size[2 + o] = __dp4a(wm[o], um, size[2 + o]);
+            if (o < 2) size[o] = __dp4a(wm[o], am, size[o]);
         }
         if (it % kFold == kFold - 1) fold(hi, mid);
     }
     fold(hi, mid);
 #pragma unroll
-    for (int f = 0; f < 2; ++f) cold = cold || too_small(T[f], seen[f]);
+    for (int k = 0; k < 7; ++k) size[k] = k < 2 ? group_add<1, G>(size[k]) : group_add<2, G>(size[k]);
+    cold |= out_of_range<2>(T[0], seen[0], size, 0, zero_ops);
+    cold |= out_of_range<5>(T[1], seen[1], size + 2, 0, zero_ops);
     cold = group_max<1, G>(uint32_t(cold)) != 0;
 }
 
@@ -421,29 +500,59 @@ __device__ __forceinline__ double fixed_weight(const PlanView<double>& P, int i,
                        int(fixed_col_word(P, e, o == 5) >> 30));
 }
 
-// Row i in FP64, by one lane.
-template <bool FILTER, int K, class F>
-__device__ __noinline__ void cold_row(const PlanView<double>& P, const F& fld, int i, double (&sum)[K]) {
-    constexpr int KA = FILTER ? 1 : 2, KV = FILTER ? 1 : 5;
-    double ai, ui, vi;
-    fld.get(i, ai, ui, vi);
+// The rows that need FP64, by as many lanes as the fixed-point sums: in the order of the
+// FP64 kernels (a lane takes every G-th chunk, then the lanes' sums), 32 / G rows of the warp
+// at a time.  slots: the rows, as bits (fixed_nodes); out[k][slot]: the sums' bit patterns.
+template <int G, bool FILTER, int K, class F>
+__device__ __noinline__ void cold_rows(const int32_t* row_ptr, const char* rec, const int16_t* wexp, F fld,
+                                       int64_t first, uint32_t slots, long long (*out)[32]) {
+    constexpr int KA = FILTER ? 1 : 2, KV = FILTER ? 1 : 5, R = 32 / G;
+    const int lane = threadIdx.x & 31, gl = lane % G;
+    while (slots) {
+        uint32_t left = slots;
+        for (int k = 0; k < lane / G; ++k) left &= left - 1;
+        const int slot = __ffs(left) - 1;  // this group's row, or -1
+        double sum[K];
 #pragma unroll
-    for (int k = 0; k < K; ++k) sum[k] = 0.0;
-    const int e1 = P.row_ptr[i + 1];
-    for (int e = P.row_ptr[i]; e < e1; ++e) {
-        double a, u, v;
-        fld.get(int(fixed_col_word(P, e, FILTER) & kColMask), a, u, v);
-        a -= ai;
-        u -= ui;
-        v -= vi;
+        for (int k = 0; k < K; ++k) sum[k] = 0.0;
+        if (slot >= 0) {
+            const int i = int(first + (slot / R) * (kFixedWarps * R) + slot % R);
+            double ai, ui, vi;
+            fld.get(i, ai, ui, vi);
+            const int4 ev = *reinterpret_cast<const int4*>(wexp + int64_t(i) * 8);
+            const int E[6] = {int16_t(ev.x), ev.x >> 16, int16_t(ev.y), ev.y >> 16, int16_t(ev.z), ev.z >> 16};
+            const int e1 = row_ptr[i + 1];
+#pragma unroll 1
+            for (int e = row_ptr[i] + 4 * gl; e < e1; e += 4 * G) {
+#pragma unroll 1
+                for (int k = 0; k < 4; ++k) {
+                    const uint32_t cw = *reinterpret_cast<const uint32_t*>(
+                        rec + (FILTER ? Rec<double>::fcol_e(e + k) : Rec<double>::col_e(e + k)));
+                    const int s = int(cw >> 30);
+                    double a, u, v;
+                    fld.get(int(cw & kColMask), a, u, v);
+                    a -= ai;
+                    u -= ui;
+                    v -= vi;
 #pragma unroll
-        for (int o = 0; o < KV; ++o) {
-            const double w = fixed_weight(P, i, e, FILTER ? 5 : o);
-            if (o < KA) sum[o] = fma(a, w, sum[o]);
-            sum[KA + o] = fma(u, w, sum[KA + o]);
-            sum[KA + KV + o] = fma(v, w, sum[KA + KV + o]);
+                    for (int o = 0; o < KV; ++o) {
+                        const int op = FILTER ? 5 : o;
+                        const double w = word_weight(*reinterpret_cast<const long long*>(rec + fixed_at(e + k, op)), E[op], s);
+                        if (o < KA) sum[o] = fma(a, w, sum[o]);
+                        sum[KA + o] = fma(u, w, sum[KA + o]);
+                        sum[KA + KV + o] = fma(v, w, sum[KA + KV + o]);
+                    }
+                }
+            }
         }
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            sum[k] = group_sum<G>(sum[k]);
+            if (slot >= 0 && gl == 0) out[k][slot] = __double_as_longlong(sum[k]);
+        }
+        for (int k = 0; k < R; ++k) slots &= slots - 1;
     }
+    __syncwarp();
 }
 
 // The sums of the block's nodes, epi(node, a, u, v, sums) for each.  A pass takes 32/G nodes
@@ -466,12 +575,13 @@ __device__ __forceinline__ void fixed_nodes(const PlanView<double>& P, const F& 
         if (node - lane / G >= P.n_hi) break;
         const int i = int(node < P.n_hi ? node : P.n_hi - 1);
         const int e0 = P.row_ptr[i], e1 = node < P.n_hi ? P.row_ptr[i + 1] : e0;
+        const int zero_ops = P.wexp[int64_t(i) * 8 + 6];
         if (p == 0) pdl_wait();  // nothing before it is written by a launch
         long long hi[LK], lo[LK];
         int T[LT];
         bool cold;
-        if constexpr (FILTER) filter_row<G>(P, fld, i, e0, e1, gl, hi, lo, T, cold);
-        else rhs_row<G>(P, fld, i, e0, e1, gl, hi, lo, T, cold);
+        if constexpr (FILTER) filter_row<G>(P, fld, i, e0, e1, gl, zero_ops, hi, lo, T, cold);
+        else rhs_row<G>(P, fld, i, e0, e1, gl, zero_ops, hi, lo, T, cold);
         // over the lanes that share a sum: all of them (filter, ln rho), or every second one
 #pragma unroll
         for (int k = 0; k < LK; ++k) {
@@ -505,10 +615,14 @@ __device__ __forceinline__ void fixed_nodes(const PlanView<double>& P, const F& 
                 if (groups >> (n * G) & 1) cold_slots |= 1u << (p * R + n);
     }
     __syncwarp();
+    if (cold_slots)
+        cold_rows<G, FILTER, K>(P.row_ptr, reinterpret_cast<const char*>(FILTER ? P.wf : P.w), P.wexp, fld, first,
+                                cold_slots, s_hi[warp]);
     const int64_t node = first + (lane / R) * (kFixedWarps * R) + lane % R;
     const bool mine = lane < passes * R && node < P.n_hi;
     double sum[K];
     if (mine) {
+        const bool cold = cold_slots >> lane & 1;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const int f = FILTER ? k : (k < 2 ? 0 : (k < 7 ? 1 : 2));
@@ -516,11 +630,8 @@ __device__ __forceinline__ void fixed_nodes(const PlanView<double>& P, const F& 
             // E_w + E_d - 113 + 28, E_d = T / 2^20 + 1 - 1023
             const double S = pow2(max(P.wexp[node * 8 + o] + (s_T[warp][f][lane] >> 20) - 1107, -1000));
             sum[k] = fma(double(s_hi[warp][k][lane]), S * 268435456.0, double(s_lo[warp][k][lane]) * S);
+            if (cold) sum[k] = __longlong_as_double(s_hi[warp][k][lane]);
         }
-    }
-    if (cold_slots) {
-        // one lane per row in FP64: rare, and no other lane's business
-        if (mine && (cold_slots >> lane & 1)) cold_row<FILTER, K>(P, fld, int(node), sum);
     }
     if (mine) {
         double a, u, v;

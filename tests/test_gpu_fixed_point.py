@@ -4,6 +4,8 @@ FP64 weights; infinities and NaN; exact zeros."""
 import numpy as np
 import pytest
 
+import labfm_inputs as li
+
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
@@ -223,4 +225,61 @@ def test_weights_are_held_bit_for_bit(lb, spread):
         assert np.array_equal(g[1, col[on]], -w[0, on]) and np.array_equal(g[2, col[on]], -w[1, on])
         g = lb.filter_adjoint(plan, torch.tensor(lam, device="cuda")).cpu().numpy()
         assert np.array_equal(g[0, col[on]], kappa[j] * w[5, on])
+    plan.close()
+
+
+def _wide_field(kind, ns, rng):
+    x, y = ns.xy.T
+    s = ns.s[0]
+    if kind == "front":
+        return np.stack([0.3 * np.tanh((x - 0.5) / (k * s)) for k in (0.2, 0.5, 2.0)])
+    if kind == "pulse":
+        return np.stack([np.exp(-((x - 0.5) ** 2 + (y - 0.5) ** 2) / (2 * (k * s) ** 2)) for k in (2, 5, 10)])
+    if kind == "impulses":
+        return (rng.random((3, ns.N)) < 1 / 60) * rng.standard_normal((3, ns.N))
+    if kind == "jump":  # small differences beside a unit one
+        return 1e-9 * rng.standard_normal((3, ns.N)) + (x > 0.5)
+    return 1e-6 * np.exp(5 * rng.standard_normal((3, ns.N))).clip(max=1e6)  # log-normal
+
+
+@pytest.mark.parametrize("m", [4, 6, 8, 10])
+@pytest.mark.parametrize("kind", ["front", "pulse", "impulses", "jump", "lognormal"])
+def test_fields_of_a_wide_span_within_a_stencil(lb, kind, m):
+    # every sum within (24 + n) 2^-53 sum |w d| of the exact one (FP64's own bound for n
+    # terms and the lanes' sums), for each operator and field: the bounds of the sums that
+    # enter an output, with its coefficients, and a few roundings of its terms
+    ns = li.tgv_lattice(30, 28, m=m, jitter=0.3 if m != 4 else 0.05, seed=m)
+    xy, h, sp = (torch.tensor(a, device="cuda") for a in (ns.xy, ns.h, ns.s))
+    rpd, cold = lb.build_stencils(xy, h, ns.Lx, ns.Ly)
+    wb = lb.build_weights(xy, h, sp, ns.Lx, ns.Ly, rpd, cold, m, residual=False)
+    plan = lb.Plan(rpd, cold, wb["w"], wb["kappa"], sp, dtype=torch.float64)
+    rp, col, w, kappa = (t.cpu().numpy() for t in (rpd, cold, wb["w"], wb["kappa"]))
+    q = _wide_field(kind, ns, np.random.default_rng(m))
+    Q = torch.tensor(q, device="cuda")
+    ph = lb.Phys(3.0, 0.7)
+    R, filt = lb.rhs(plan, Q, ph).cpu().numpy(), lb.filter(plan, Q).cpu().numpy()
+    L, u = np.longdouble, 2.0 ** -53
+    S, B = np.zeros((6, 3, ns.N), L), np.zeros((6, 3, ns.N))
+    for i in range(ns.N):
+        s = slice(rp[i], rp[i + 1])
+        d = (q[:, col[s]] - q[:, i:i + 1]).astype(L)
+        wi = w[:, s].copy()
+        wi[5] *= kappa[i]
+        S[:, :, i] = wi.astype(L) @ d.T
+        B[:, :, i] = (24 + rp[i + 1] - rp[i]) * u * (np.abs(wi) @ np.abs(d).T.astype(float))
+    a, uu, vv = q
+    nu = 0.7 * np.exp(-a.astype(L))
+    third = L(1) / 3
+
+    def out(terms):  # [(coefficient, operator, field)]: value and bound
+        val = sum(c * S[o, f] for c, o, f in terms)
+        tol = sum(np.abs(c) * (B[o, f] + 12 * u * np.abs(S[o, f])) for c, o, f in terms)
+        return val, tol
+    for k, terms in enumerate([[(-uu, 0, 0), (-vv, 1, 0), (-1, 0, 1), (-1, 1, 2)],
+                               [(-uu, 0, 1), (-vv, 1, 1), (-3, 0, 0), (4 * third * nu, 2, 1), (nu, 4, 1), (third * nu, 3, 2)],
+                               [(-uu, 0, 2), (-vv, 1, 2), (-3, 1, 0), (4 * third * nu, 4, 2), (nu, 2, 2), (third * nu, 3, 1)]]):
+        val, tol = out(terms)
+        assert np.all(np.abs(R[k] - val) <= tol), k
+    for f in range(3):
+        assert np.all(np.abs(filt[f] - (q[f] + S[5, f])) <= B[5, f] + 2 * u * np.abs(filt[f])), f
     plan.close()
