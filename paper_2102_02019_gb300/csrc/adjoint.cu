@@ -159,7 +159,7 @@ __device__ __forceinline__ void fused_pass_a(const PlanView<T>& P, const FusedA<
     node_adjoints_m<T, SCALED>(P, k, a, u, v, c, ma, mu, mv, fa.g, fa.o, fa.ph);
 }
 
-// Pass A with the derivatives gathered at X (the single right-hand-side adjoint).
+// Pass A with the derivatives gathered at X (the single right-hand-side adjoint, F32).
 template <typename T, int G, bool KAHAN, bool SCALED>
 __global__ void k_adj_pointwise(PlanView<T> P, const Packed<T>* X, const Packed<T>* M,
                                 G8<T>* __restrict__ gout, Packed<T>* __restrict__ oout, Phys<T> ph) {
@@ -357,15 +357,17 @@ __device__ __forceinline__ int entry_col(const PlanView<float>& P, int e) {
 }
 __device__ __forceinline__ int entry_col(const PlanView<double>& P, int e) {
     const uint32_t c = fixed_col_word(P, e, false);
-    return int(P.wexp ? c & kColMask : c);
+    return int(c & col_mask(P.N));
 }
 template <typename T>
 __device__ __forceinline__ double entry_weight(const PlanView<T>& P, int i, int e, int o) {
-    if constexpr (std::is_same<T, double>::value)
-        if (P.wexp) return fixed_weight(P, i, e, o);
-    const char* at = o < 5 ? reinterpret_cast<const char*>(P.w) + Rec<T>::w_e(e, o)
-                           : reinterpret_cast<const char*>(P.wf) + Rec<T>::fw_e(e);
-    return double(*reinterpret_cast<const T*>(at));
+    if constexpr (std::is_same<T, double>::value) {
+        return fixed_weight(P, i, e, o);
+    } else {
+        const char* at = o < 5 ? reinterpret_cast<const char*>(P.w) + Rec<T>::w_e(e, o)
+                               : reinterpret_cast<const char*>(P.wf) + Rec<T>::fw_e(e);
+        return double(*reinterpret_cast<const T*>(at));
+    }
 }
 
 // Warp per forward row i: count the in-degree of every column k (pads, which
@@ -649,14 +651,12 @@ int rhs_adjoint_t(const labfm_plan* p, const void* fields, const void* lambda, v
     if ((rc = pack_fields(p, fields, w.X[0], st))) return rc;
     if ((rc = pack_fields(p, lambda, w.Fb, st))) return rc;
     if constexpr (std::is_same<T, double>::value) {
-        if (p->wexp) {
-            if ((rc = fixed_coeffs(p, w.X[0], w.D, st))) return rc;
-            k_adj_pointwise_d8<<<unsigned((p->N + 127) / 128), 128, 0, st>>>(view<T>(p), w.X[0], w.D, w.Fb, w.g, w.Ob, ph);
-            LABFM_LAUNCH_CHECK("adjoint pointwise kernel");
-        }
-    }
-    if (!p->wexp)
+        if ((rc = fixed_coeffs(p, w.X[0], w.D, st))) return rc;
+        k_adj_pointwise_d8<<<unsigned((p->N + 127) / 128), 128, 0, st>>>(view<T>(p), w.X[0], w.D, w.Fb, w.g, w.Ob, ph);
+        LABFM_LAUNCH_CHECK("adjoint pointwise kernel");
+    } else {
         if ((rc = pass_a<T>(p, w.X[0], w.Fb, w.g, w.Ob, ph, st))) return rc;
+    }
     const FusedA<T> none{nullptr, nullptr, nullptr, nullptr, ph};
     if ((rc = pass_b<T>(p, 0, w.g, w.Ob, w.Lam, nullptr, nullptr, 0.0, 0.0, 0.0, none, st))) return rc;
     return unpack_fields(p, w.Lam, grad, st);

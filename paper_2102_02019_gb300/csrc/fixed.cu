@@ -1,4 +1,4 @@
-// Kernels of F64 plans whose weights are stored in fixed point (fixed.cuh): the right-hand
+// Kernels of F64 plans, whose sums run in fixed point (fixed.cuh): the right-hand
 // side, the RK stage (recording or not), the derivative combinations of the adjoint and the
 // filter, and the packing of the rows.
 #include <cuda_runtime.h>
@@ -110,8 +110,7 @@ __device__ __forceinline__ int entry_shift(int below) {
 __global__ void k_pack_fixed(int64_t N, int64_t nnz, int64_t off, const int32_t* __restrict__ row_ptr,
                              const int32_t* __restrict__ col, const double* __restrict__ w,
                              const double* __restrict__ kappa, const int32_t* __restrict__ prow,
-                             char* __restrict__ rb, char* __restrict__ fb, int16_t* __restrict__ wexp,
-                             int* __restrict__ unfit) {
+                             char* __restrict__ rb, char* __restrict__ fb, int16_t* __restrict__ wexp, bool shifts) {
     const int lane = threadIdx.x & 31;
     const int64_t warps = int64_t(gridDim.x) * (blockDim.x >> 5);
     for (int64_t il = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5; il < N; il += warps) {
@@ -134,6 +133,7 @@ __global__ void k_pack_fixed(int64_t N, int64_t nnz, int64_t off, const int32_t*
             odd |= top[o] >= (1023 + 400) << 20 || (top[o] < (1023 - 400) << 20 && top[o] > 0);
         }
         auto shift_of = [&](const int (&h)[6], int o0, int o1) {
+            if (!shifts) return 0;
             int below = -0x7fffffff;
             for (int o = o0; o < o1; ++o)
                 if (top[o] > 0) below = max(below, h[o] - top[o]);
@@ -182,9 +182,7 @@ __global__ void k_pack_fixed(int64_t N, int64_t nnz, int64_t off, const int32_t*
                 odd |= exps[o] + 2 - least[o] > kMostAlign;
             }
         }
-        odd = __any_sync(0xffffffffu, odd);
-        if (odd && lane == 0) atomicOr(unfit, 1);
-        if (odd) continue;
+        const bool raw = __any_sync(0xffffffffu, odd);
         if (lane == 0) {
             int4 v;
             v.x = (exps[0] & 0xffff) | (exps[1] << 16);
@@ -193,6 +191,7 @@ __global__ void k_pack_fixed(int64_t N, int64_t nnz, int64_t off, const int32_t*
             v.w = 0;  // the operators that are zero throughout the row
 #pragma unroll
             for (int o = 0; o < 6; ++o) v.w |= top[o] == 0 ? 1 << o : 0;
+            if (raw) v.w = kRawRow;
             reinterpret_cast<int4*>(wexp)[i] = v;
         }
         for (int e = lane; e < plen; e += 32) {
@@ -209,10 +208,13 @@ __global__ void k_pack_fixed(int64_t N, int64_t nnz, int64_t off, const int32_t*
                     v[o] = weight(src, o);
                     h[o] = __double2hiint(v[o]) & 0x7fffffff;
                 }
-                sr = uint32_t(shift_of(h, 0, 5));
-                sf = uint32_t(shift_of(h, 5, 6));
+                if (!raw) {
+                    sr = uint32_t(shift_of(h, 0, 5));
+                    sf = uint32_t(shift_of(h, 5, 6));
+                }
 #pragma unroll
-                for (int o = 0; o < 6; ++o) word[o] = weight_word(v[o], exps[o], int(o < 5 ? sr : sf));
+                for (int o = 0; o < 6; ++o)
+                    word[o] = raw ? __double_as_longlong(v[o]) : weight_word(v[o], exps[o], int(o < 5 ? sr : sf));
             }
             *reinterpret_cast<uint32_t*>(rb + Rec<double>::col_e(dst)) = c | (sr << 30);
             *reinterpret_cast<uint32_t*>(fb + Rec<double>::fcol_e(dst)) = c | (sf << 30);
@@ -348,10 +350,11 @@ int fixed_filter_soa(const labfm_plan* p, const void* in, void* out, cudaStream_
     return LABFM_OK;
 }
 
-int fixed_pack(const PlanInput& in, int64_t off, labfm_plan* p, int* unfit, cudaStream_t st) {
+int fixed_pack(const PlanInput& in, int64_t off, labfm_plan* p, cudaStream_t st) {
     const int gw = int(std::min<int64_t>((in.N * 32 + 255) / 256, 1 << 20));
     k_pack_fixed<<<gw, 256, 0, st>>>(in.N, in.nnz, off, in.row_ptr, in.col, in.w, in.kappa, p->row_ptr,
-                                     static_cast<char*>(p->w), static_cast<char*>(p->wf), p->wexp, unfit);
+                                     static_cast<char*>(p->w), static_cast<char*>(p->wf), p->wexp,
+                                     col_mask(p->N) < 0x7fffffffu);
     LABFM_LAUNCH_CHECK("fixed-point pack kernel");
     return LABFM_OK;
 }

@@ -39,12 +39,14 @@
 //
 // No overflow: E_w is raised until sum_j |w_ji| 2^-s_j <= 32 2^E_w, so |sum w1 d1| <=
 // 2^(5 + 28 + 29) over a whole row; |sum (w1 d0 + w0 d1)| <= 2^60 + n 2^57 over n entries,
-// whose carries a lane moves up after every 32.  Weights that are not finite, beyond
-// 2^+-400 or below 2^-500 of their row's largest, and plans of 2^30 nodes or more, keep the
-// FP64 weights and kernels (plan.wexp == nullptr).  A row whose differences are not finite
-// or beyond 2^477 is summed in FP64 too, so that infinities and NaN come out as they would,
-// and one whose differences of a field all lie below 2^-499 without being all zero.  Beside
-// larger ones, differences below 2^-1022 count as zero.
+// whose carries a lane moves up after every 32.  Rows with a weight that is not finite,
+// beyond 2^+-400 at their largest, subnormal or below 2^-500 of their row's largest hold
+// plain FP64 weights and are summed in FP64 (kRawRow), each by itself, so that a failed node
+// changes no other row.  A row whose differences are not finite or beyond 2^477 is summed in
+// FP64 too, so that infinities and NaN come out as they would, and one whose differences of
+// a field all lie below 2^-499 without being all zero.  Beside larger ones, differences below
+// 2^-1022 count as zero.  Plans of 2^30 nodes or more need the two bits for their columns:
+// there every s_j is 0.
 #pragma once
 
 #include "gather.cuh"
@@ -52,7 +54,9 @@
 namespace labfm {
 namespace {
 
-constexpr uint32_t kColMask = 0x3fffffffu;  // the column word: s_j in the two bits above
+// The column word: the column, and s_j in the bits above it.
+__host__ __device__ __forceinline__ uint32_t col_mask(int64_t N) { return N < (int64_t(1) << 30) ? 0x3fffffffu : 0x7fffffffu; }
+constexpr int kRawRow = 64;  // with the zero operators' bits in wexp[8 i + 6]: the row holds FP64 weights
 constexpr int kFixedWarps = 2;  // warps a block
 constexpr int kFloorT = 65 << 20;           // T of a field until a difference above it turns up
 constexpr int kLeastT = 524 << 20;          // smallest bound of the fixed-point sums
@@ -265,6 +269,7 @@ __device__ __forceinline__ void filter_row(const PlanView<double>& P, const F& f
                                            int zero_ops, long long (&hi)[3], long long (&mid)[3], int (&T)[3],
                                            bool& cold) {
     const int trips = __reduce_max_sync(0xffffffffu, (e1 - e0 + 4 * G - 1) / (4 * G));
+    const uint32_t mask = col_mask(P.N);
     double own[3];
     fld.get(i, own[0], own[1], own[2]);
 #pragma unroll
@@ -290,8 +295,8 @@ __device__ __forceinline__ void filter_row(const PlanView<double>& P, const F& f
         for (int k = 0; k < 4; ++k) {
             const uint32_t cw = on ? cj[k] : uint32_t(i);
             double v[3];
-            fld.get(int(cw & kColMask), v[0], v[1], v[2]);
-            s20[k] = int((cw >> 30) << 20);
+            fld.get(int(cw & mask), v[0], v[1], v[2]);
+            s20[k] = int((cw & ~mask) >> 10);
 #pragma unroll
             for (int f = 0; f < 3; ++f) {
                 d[f][k] = v[f] - own[f];
@@ -346,6 +351,7 @@ __device__ __forceinline__ void rhs_row(const PlanView<double>& P, const F& fld,
                                         int zero_ops, long long (&hi)[7], long long (&mid)[7], int (&T)[2],
                                         bool& cold) {
     const int trips = __reduce_max_sync(0xffffffffu, (e1 - e0 + 2 * G - 1) / (2 * G));
+    const uint32_t mask = col_mask(P.N);
     const bool odd = gl & 1;
     const Column fa = column(fld, 0), ff = column(fld, odd ? 2 : 1);
     const double oa = fa[i], of = ff[i];
@@ -365,9 +371,9 @@ __device__ __forceinline__ void rhs_row(const PlanView<double>& P, const F& fld,
     };
     auto values = [&](const uint32_t (&cj)[4], double (&g)[6]) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) g[k] = ff[int(cj[k] & kColMask)];
-        g[4] = fa[int((odd ? cj[2] : cj[0]) & kColMask)];
-        g[5] = fa[int((odd ? cj[3] : cj[1]) & kColMask)];
+        for (int k = 0; k < 4; ++k) g[k] = ff[int(cj[k] & mask)];
+        g[4] = fa[int((odd ? cj[2] : cj[0]) & mask)];
+        g[5] = fa[int((odd ? cj[3] : cj[1]) & mask)];
     };
     uint32_t cj[4];
     double g[6];
@@ -391,14 +397,14 @@ __device__ __forceinline__ void rhs_row(const PlanView<double>& P, const F& fld,
         for (int k = 0; k < 4; ++k) {
             d[k] = g[k] - of;
             seen[1] |= not_zero(d[k]);
-            t[k] = T[1] - exponent20(d[k]) - int((cj[k] >> 30) << 20);
+            t[k] = T[1] - exponent20(d[k]) - int((cj[k] & ~mask) >> 10);
             low |= t[k];
         }
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             da[k] = g[4 + k] - oa;
             seen[0] |= not_zero(da[k]);
-            ta[k] = T[0] - exponent20(da[k]) - int(((odd ? cj[k + 2] : cj[k]) >> 30) << 20);
+            ta[k] = T[0] - exponent20(da[k]) - int(((odd ? cj[k + 2] : cj[k]) & ~mask) >> 10);
             low |= ta[k];
         }
         if (__any_sync(0xffffffffu, low < 0)) {
@@ -493,11 +499,12 @@ __device__ __forceinline__ uint32_t fixed_col_word(const PlanView<double>& P, in
     return *reinterpret_cast<const uint32_t*>(at);
 }
 
-// Weight of operator o at entry e of row i of a fixed-point plan.
+// Weight of operator o at entry e of row i of an F64 plan.
 __device__ __forceinline__ double fixed_weight(const PlanView<double>& P, int i, int e, int o) {
     const char* rec = o == 5 ? reinterpret_cast<const char*>(P.wf) : reinterpret_cast<const char*>(P.w);
-    return word_weight(*reinterpret_cast<const long long*>(rec + fixed_at(e, o)), P.wexp[int64_t(i) * 8 + o],
-                       int(fixed_col_word(P, e, o == 5) >> 30));
+    const long long word = *reinterpret_cast<const long long*>(rec + fixed_at(e, o));
+    if (P.wexp[int64_t(i) * 8 + 6] & kRawRow) return __longlong_as_double(word);
+    return word_weight(word, P.wexp[int64_t(i) * 8 + o], int((fixed_col_word(P, e, o == 5) & ~col_mask(P.N)) >> 30));
 }
 
 // The rows that need FP64, by as many lanes as the fixed-point sums: in the order of the
@@ -505,7 +512,7 @@ __device__ __forceinline__ double fixed_weight(const PlanView<double>& P, int i,
 // at a time.  slots: the rows, as bits (fixed_nodes); out[k][slot]: the sums' bit patterns.
 template <int G, bool FILTER, int K, class F>
 __device__ __noinline__ void cold_rows(const int32_t* row_ptr, const char* rec, const int16_t* wexp, F fld,
-                                       int64_t first, uint32_t slots, long long (*out)[32]) {
+                                       uint32_t mask, int64_t first, uint32_t slots, long long (*out)[32]) {
     constexpr int KA = FILTER ? 1 : 2, KV = FILTER ? 1 : 5, R = 32 / G;
     const int lane = threadIdx.x & 31, gl = lane % G;
     while (slots) {
@@ -521,6 +528,7 @@ __device__ __noinline__ void cold_rows(const int32_t* row_ptr, const char* rec, 
             fld.get(i, ai, ui, vi);
             const int4 ev = *reinterpret_cast<const int4*>(wexp + int64_t(i) * 8);
             const int E[6] = {int16_t(ev.x), ev.x >> 16, int16_t(ev.y), ev.y >> 16, int16_t(ev.z), ev.z >> 16};
+            const bool raw = ev.w & kRawRow;
             const int e1 = row_ptr[i + 1];
 #pragma unroll 1
             for (int e = row_ptr[i] + 4 * gl; e < e1; e += 4 * G) {
@@ -528,16 +536,17 @@ __device__ __noinline__ void cold_rows(const int32_t* row_ptr, const char* rec, 
                 for (int k = 0; k < 4; ++k) {
                     const uint32_t cw = *reinterpret_cast<const uint32_t*>(
                         rec + (FILTER ? Rec<double>::fcol_e(e + k) : Rec<double>::col_e(e + k)));
-                    const int s = int(cw >> 30);
+                    const int s = int((cw & ~mask) >> 30);
                     double a, u, v;
-                    fld.get(int(cw & kColMask), a, u, v);
+                    fld.get(int(cw & mask), a, u, v);
                     a -= ai;
                     u -= ui;
                     v -= vi;
 #pragma unroll
                     for (int o = 0; o < KV; ++o) {
                         const int op = FILTER ? 5 : o;
-                        const double w = word_weight(*reinterpret_cast<const long long*>(rec + fixed_at(e + k, op)), E[op], s);
+                        const long long word = *reinterpret_cast<const long long*>(rec + fixed_at(e + k, op));
+                        const double w = raw ? __longlong_as_double(word) : word_weight(word, E[op], s);
                         if (o < KA) sum[o] = fma(a, w, sum[o]);
                         sum[KA + o] = fma(u, w, sum[KA + o]);
                         sum[KA + KV + o] = fma(v, w, sum[KA + KV + o]);
@@ -574,8 +583,9 @@ __device__ __forceinline__ void fixed_nodes(const PlanView<double>& P, const F& 
         const int64_t node = first + p * (kFixedWarps * R) + lane / G;
         if (node - lane / G >= P.n_hi) break;
         const int i = int(node < P.n_hi ? node : P.n_hi - 1);
-        const int e0 = P.row_ptr[i], e1 = node < P.n_hi ? P.row_ptr[i + 1] : e0;
         const int zero_ops = P.wexp[int64_t(i) * 8 + 6];
+        const bool raw = node < P.n_hi && (zero_ops & kRawRow);
+        const int e0 = P.row_ptr[i], e1 = node < P.n_hi && !raw ? P.row_ptr[i + 1] : e0;
         if (p == 0) pdl_wait();  // nothing before it is written by a launch
         long long hi[LK], lo[LK];
         int T[LT];
@@ -609,15 +619,15 @@ __device__ __forceinline__ void fixed_nodes(const PlanView<double>& P, const F& 
                 s_T[warp][1 + gl][slot] = T[1];
             }
         }
-        const uint32_t groups = __ballot_sync(0xffffffffu, cold && gl == 0);
+        const uint32_t groups = __ballot_sync(0xffffffffu, (cold || raw) && gl == 0);
         if (groups)
             for (int n = 0; n < R; ++n)
                 if (groups >> (n * G) & 1) cold_slots |= 1u << (p * R + n);
     }
     __syncwarp();
     if (cold_slots)
-        cold_rows<G, FILTER, K>(P.row_ptr, reinterpret_cast<const char*>(FILTER ? P.wf : P.w), P.wexp, fld, first,
-                                cold_slots, s_hi[warp]);
+        cold_rows<G, FILTER, K>(P.row_ptr, reinterpret_cast<const char*>(FILTER ? P.wf : P.w), P.wexp, fld, col_mask(P.N),
+                                first, cold_slots, s_hi[warp]);
     const int64_t node = first + (lane / R) * (kFixedWarps * R) + lane % R;
     const bool mine = lane < passes * R && node < P.n_hi;
     double sum[K];

@@ -323,7 +323,7 @@ struct PlanView {
     const int32_t* bnd_kind;   // per slot: LABFM_WALL, LABFM_INFLOW, LABFM_OUTFLOW (null: all walls)
     const T* bnd_target;       // per slot: (u_xi,IN, u_eta,IN) of an inflow, p_inf (first) of an outflow
     T sigma, Lb, mach, rho0;   // relaxation coefficient, length, Mach number, reference density
-    const int16_t* wexp;       // F64 plans in fixed point (fixed.cuh): per row the operators' exponents, 8 values
+    const int16_t* wexp;       // F64 plans (fixed.cuh): per row the operators' exponents and its flags, 8 values
 };
 
 // Operator loads of one 4-entry chunk starting at entry e (a multiple of 4).

@@ -85,8 +85,8 @@ struct labfm_plan {
     void* w = nullptr;           // 5 x nnz_pad RHS weights, operator-major (dtype)
     void* wf = nullptr;          // nnz_pad filter weights kappa_i w^hyp_ji (dtype)
     void* inv_s = nullptr;       // N values 1/s_i (dtype), used by the F32 kernels
-    // F64 plans whose weights are stored in fixed point (fixed.cuh): per row the
-    // exponents of the six operators (8 int16); null: FP64 weights
+    // F64 plans (fixed.cuh): per row the exponents of the six operators, the operators that
+    // are zero throughout it and whether it holds plain FP64 weights (8 int16)
     int16_t* wexp = nullptr;
     int64_t device_bytes = 0;
     // instances of a batched plan (one instance for labfm_plan_create): node
@@ -197,7 +197,7 @@ int ahead_stage(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, cons
 int ahead_filter(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, const void* in, void* out, void* soa,
                  cudaStream_t st);
 
-// The gathers of F64 plans in fixed point (fixed.cu), on `group` lanes per node or more.
+// The gathers of F64 plans in fixed point (fixed.cu), on `group` lanes per node, 16 at most.
 // Packed states, D8 records and SoA fields as in step.cu; nodes [n_lo, n_hi).
 int fixed_rhs(const labfm_plan* p, const void* fields, void* rhs, const labfm_phys& ph, int group, cudaStream_t st);
 int fixed_stage(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, const void* xin, const void* qin,
@@ -207,9 +207,8 @@ int fixed_coeffs(const labfm_plan* p, const void* X, void* D, cudaStream_t st);
 int fixed_filter(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, const void* in, void* out, void* soa,
                  cudaStream_t st);
 int fixed_filter_soa(const labfm_plan* p, const void* in, void* out, cudaStream_t st);
-// Packs one instance's rows (nodes off .. off + N of the plan) in fixed point; sets
-// *unfit on the device where a row cannot be.
-int fixed_pack(const PlanInput& in, int64_t off, labfm_plan* p, int* unfit, cudaStream_t st);
+// Packs one instance's rows (nodes off .. off + N of the plan).
+int fixed_pack(const PlanInput& in, int64_t off, labfm_plan* p, cudaStream_t st);
 
 // Plan packing (step.cu): concatenates the instances block-diagonally.
 int pack_plan(labfm_plan* p, const PlanInput* in, int n_inst, cudaStream_t st);

@@ -591,14 +591,18 @@ int rhs_launch_g(const labfm_plan* p, const void* fields, void* rhs, const Phys<
 template <typename T>
 int rhs_launch(const labfm_plan* p, const void* fields, void* rhs, const labfm_phys* php, int group,
                int block, cudaStream_t st) {
-    if (p->wexp) return fixed_rhs(p, fields, rhs, *php, group, st);
-    const Phys<T> ph{T(php->c2), T(php->mu), T(php->gx), T(php->gy)};
-    switch (group) {
-        case 2: return rhs_launch_g<T, 2>(p, fields, rhs, ph, block, st);
-        case 4: return rhs_launch_g<T, 4>(p, fields, rhs, ph, block, st);
-        case 8: return rhs_launch_g<T, 8>(p, fields, rhs, ph, block, st);
-        case 16: return rhs_launch_g<T, 16>(p, fields, rhs, ph, block, st);
-        case 32: return rhs_launch_g<T, 32>(p, fields, rhs, ph, block, st);
+    if constexpr (std::is_same<T, double>::value) {
+        (void)block;
+        return fixed_rhs(p, fields, rhs, *php, group, st);
+    } else {
+        const Phys<T> ph{T(php->c2), T(php->mu), T(php->gx), T(php->gy)};
+        switch (group) {
+            case 2: return rhs_launch_g<T, 2>(p, fields, rhs, ph, block, st);
+            case 4: return rhs_launch_g<T, 4>(p, fields, rhs, ph, block, st);
+            case 8: return rhs_launch_g<T, 8>(p, fields, rhs, ph, block, st);
+            case 16: return rhs_launch_g<T, 16>(p, fields, rhs, ph, block, st);
+            case 32: return rhs_launch_g<T, 32>(p, fields, rhs, ph, block, st);
+        }
     }
     return set_error(LABFM_EINVAL, "unsupported group size");
 }
@@ -686,21 +690,23 @@ template <typename T>
 int stage_launch(const labfm_plan* p, const Packed<T>* xin, const Packed<T>* qin, Packed<T>* qout,
                  Packed<T>* xout, double dt, double bk, double ck, const Phys<T>& ph, int* counter,
                  cudaStream_t st) {
-    if (p->wexp) return fixed_stage(p, 0, p->N, p->group, xin, qin, qout, xout, dt, bk, ck, as_phys(ph), nullptr, st);
-    if constexpr (std::is_same<T, float>::value) {
+    if constexpr (std::is_same<T, double>::value) {
+        (void)counter;
+        return fixed_stage(p, 0, p->N, p->group, xin, qin, qout, xout, dt, bk, ck, as_phys(ph), nullptr, st);
+    } else {
         if (!staged(p) && !p->persistent && ahead_serves(p->N, p->group))
             return ahead_stage(p, 0, p->N, p->group, xin, qin, qout, xout, dt, bk, ck, as_phys(ph), nullptr, st);
         if (staged(p)) {
             if (p->group == 32) return stage_bulk_launch_s<32>(p, xin, qin, qout, xout, dt, bk, ck, ph, st);
             return stage_bulk_launch_s<16>(p, xin, qin, qout, xout, dt, bk, ck, ph, st);
         }
-    }
-    switch (p->group) {
-        case 2: return stage_launch_g<T, 2>(p, xin, qin, qout, xout, dt, bk, ck, ph, counter, st);
-        case 4: return stage_launch_g<T, 4>(p, xin, qin, qout, xout, dt, bk, ck, ph, counter, st);
-        case 8: return stage_launch_g<T, 8>(p, xin, qin, qout, xout, dt, bk, ck, ph, counter, st);
-        case 16: return stage_launch_g<T, 16>(p, xin, qin, qout, xout, dt, bk, ck, ph, counter, st);
-        case 32: return stage_launch_g<T, 32>(p, xin, qin, qout, xout, dt, bk, ck, ph, counter, st);
+        switch (p->group) {
+            case 2: return stage_launch_g<T, 2>(p, xin, qin, qout, xout, dt, bk, ck, ph, counter, st);
+            case 4: return stage_launch_g<T, 4>(p, xin, qin, qout, xout, dt, bk, ck, ph, counter, st);
+            case 8: return stage_launch_g<T, 8>(p, xin, qin, qout, xout, dt, bk, ck, ph, counter, st);
+            case 16: return stage_launch_g<T, 16>(p, xin, qin, qout, xout, dt, bk, ck, ph, counter, st);
+            case 32: return stage_launch_g<T, 32>(p, xin, qin, qout, xout, dt, bk, ck, ph, counter, st);
+        }
     }
     return set_error(LABFM_EINVAL, "unsupported group size");
 }
@@ -743,24 +749,20 @@ int stage_ranges(const labfm_plan* p, const Packed<T>* xin, const Packed<T>* qin
                  Packed<T>* xout, double dt, double bk, double ck, const Phys<T>& ph, cudaStream_t st) {
     for (int r = 0; r < p->n_ranges; ++r) {
         int rc = LABFM_EINVAL;
-        if (p->wexp) {
-            if ((rc = fixed_stage(p, p->range_begin[r], p->range_begin[r + 1], p->range_group[r], xin, qin, qout, xout,
-                                  dt, bk, ck, as_phys(ph), nullptr, st)))
-                return rc;
-            continue;
-        }
-        if (std::is_same<T, float>::value && ahead_serves(p->range_begin[r + 1] - p->range_begin[r], p->range_group[r])) {
-            if ((rc = ahead_stage(p, p->range_begin[r], p->range_begin[r + 1], p->range_group[r], xin, qin,
-                                  qout, xout, dt, bk, ck, as_phys(ph), nullptr, st)))
-                return rc;
-            continue;
-        }
-        switch (p->range_group[r]) {
-            case 2: rc = stage_range_launch_g<T, 2>(p, r, xin, qin, qout, xout, dt, bk, ck, ph, st); break;
-            case 4: rc = stage_range_launch_g<T, 4>(p, r, xin, qin, qout, xout, dt, bk, ck, ph, st); break;
-            case 8: rc = stage_range_launch_g<T, 8>(p, r, xin, qin, qout, xout, dt, bk, ck, ph, st); break;
-            case 16: rc = stage_range_launch_g<T, 16>(p, r, xin, qin, qout, xout, dt, bk, ck, ph, st); break;
-            case 32: rc = stage_range_launch_g<T, 32>(p, r, xin, qin, qout, xout, dt, bk, ck, ph, st); break;
+        if constexpr (std::is_same<T, double>::value) {
+            rc = fixed_stage(p, p->range_begin[r], p->range_begin[r + 1], p->range_group[r], xin, qin, qout, xout, dt, bk,
+                             ck, as_phys(ph), nullptr, st);
+        } else if (ahead_serves(p->range_begin[r + 1] - p->range_begin[r], p->range_group[r])) {
+            rc = ahead_stage(p, p->range_begin[r], p->range_begin[r + 1], p->range_group[r], xin, qin, qout, xout, dt, bk,
+                             ck, as_phys(ph), nullptr, st);
+        } else {
+            switch (p->range_group[r]) {
+                case 2: rc = stage_range_launch_g<T, 2>(p, r, xin, qin, qout, xout, dt, bk, ck, ph, st); break;
+                case 4: rc = stage_range_launch_g<T, 4>(p, r, xin, qin, qout, xout, dt, bk, ck, ph, st); break;
+                case 8: rc = stage_range_launch_g<T, 8>(p, r, xin, qin, qout, xout, dt, bk, ck, ph, st); break;
+                case 16: rc = stage_range_launch_g<T, 16>(p, r, xin, qin, qout, xout, dt, bk, ck, ph, st); break;
+                case 32: rc = stage_range_launch_g<T, 32>(p, r, xin, qin, qout, xout, dt, bk, ck, ph, st); break;
+            }
         }
         if (rc) return rc;
     }
@@ -771,22 +773,18 @@ template <typename T>
 int filter_ranges(const labfm_plan* p, const Packed<T>* in, Packed<T>* out, cudaStream_t st, T* soa = nullptr) {
     for (int r = 0; r < p->n_ranges; ++r) {
         int rc = LABFM_EINVAL;
-        if (p->wexp) {
-            if ((rc = fixed_filter(p, p->range_begin[r], p->range_begin[r + 1], p->range_group[r], in, out, soa, st)))
-                return rc;
-            continue;
-        }
-        if (std::is_same<T, float>::value && ahead_serves(p->range_begin[r + 1] - p->range_begin[r], p->range_group[r])) {
-            if ((rc = ahead_filter(p, p->range_begin[r], p->range_begin[r + 1], p->range_group[r], in, out, soa, st)))
-                return rc;
-            continue;
-        }
-        switch (p->range_group[r]) {
-            case 2: rc = filter_range_launch_g<T, 2>(p, r, in, out, soa, st); break;
-            case 4: rc = filter_range_launch_g<T, 4>(p, r, in, out, soa, st); break;
-            case 8: rc = filter_range_launch_g<T, 8>(p, r, in, out, soa, st); break;
-            case 16: rc = filter_range_launch_g<T, 16>(p, r, in, out, soa, st); break;
-            case 32: rc = filter_range_launch_g<T, 32>(p, r, in, out, soa, st); break;
+        if constexpr (std::is_same<T, double>::value) {
+            rc = fixed_filter(p, p->range_begin[r], p->range_begin[r + 1], p->range_group[r], in, out, soa, st);
+        } else if (ahead_serves(p->range_begin[r + 1] - p->range_begin[r], p->range_group[r])) {
+            rc = ahead_filter(p, p->range_begin[r], p->range_begin[r + 1], p->range_group[r], in, out, soa, st);
+        } else {
+            switch (p->range_group[r]) {
+                case 2: rc = filter_range_launch_g<T, 2>(p, r, in, out, soa, st); break;
+                case 4: rc = filter_range_launch_g<T, 4>(p, r, in, out, soa, st); break;
+                case 8: rc = filter_range_launch_g<T, 8>(p, r, in, out, soa, st); break;
+                case 16: rc = filter_range_launch_g<T, 16>(p, r, in, out, soa, st); break;
+                case 32: rc = filter_range_launch_g<T, 32>(p, r, in, out, soa, st); break;
+            }
         }
         if (rc) return rc;
     }
@@ -795,15 +793,18 @@ int filter_ranges(const labfm_plan* p, const Packed<T>* in, Packed<T>* out, cuda
 
 template <typename T>
 int filter_aos(const labfm_plan* p, const Packed<T>* in, Packed<T>* out, cudaStream_t st, T* soa = nullptr) {
-    if (p->wexp) return fixed_filter(p, 0, p->N, filter_lanes(p), in, out, soa, st);
-    if (std::is_same<T, float>::value && !p->filter_persistent && ahead_serves(p->N, filter_lanes(p)))
-        return ahead_filter(p, 0, p->N, filter_lanes(p), in, out, soa, st);
-    switch (filter_lanes(p)) {
-        case 2: return filter_aos_g<T, 2>(p, in, out, soa, st);
-        case 4: return filter_aos_g<T, 4>(p, in, out, soa, st);
-        case 8: return filter_aos_g<T, 8>(p, in, out, soa, st);
-        case 16: return filter_aos_g<T, 16>(p, in, out, soa, st);
-        case 32: return filter_aos_g<T, 32>(p, in, out, soa, st);
+    if constexpr (std::is_same<T, double>::value) {
+        return fixed_filter(p, 0, p->N, filter_lanes(p), in, out, soa, st);
+    } else {
+        if (!p->filter_persistent && ahead_serves(p->N, filter_lanes(p)))
+            return ahead_filter(p, 0, p->N, filter_lanes(p), in, out, soa, st);
+        switch (filter_lanes(p)) {
+            case 2: return filter_aos_g<T, 2>(p, in, out, soa, st);
+            case 4: return filter_aos_g<T, 4>(p, in, out, soa, st);
+            case 8: return filter_aos_g<T, 8>(p, in, out, soa, st);
+            case 16: return filter_aos_g<T, 16>(p, in, out, soa, st);
+            case 32: return filter_aos_g<T, 32>(p, in, out, soa, st);
+        }
     }
     return set_error(LABFM_EINVAL, "unsupported group size");
 }
@@ -821,13 +822,16 @@ int filter_soa_g(const labfm_plan* p, const void* in, void* out, cudaStream_t st
 
 template <typename T>
 int filter_soa(const labfm_plan* p, const void* in, void* out, cudaStream_t st) {
-    if (p->wexp) return fixed_filter_soa(p, in, out, st);
-    switch (p->group) {
-        case 2: return filter_soa_g<T, 2>(p, in, out, st);
-        case 4: return filter_soa_g<T, 4>(p, in, out, st);
-        case 8: return filter_soa_g<T, 8>(p, in, out, st);
-        case 16: return filter_soa_g<T, 16>(p, in, out, st);
-        case 32: return filter_soa_g<T, 32>(p, in, out, st);
+    if constexpr (std::is_same<T, double>::value) {
+        return fixed_filter_soa(p, in, out, st);
+    } else {
+        switch (p->group) {
+            case 2: return filter_soa_g<T, 2>(p, in, out, st);
+            case 4: return filter_soa_g<T, 4>(p, in, out, st);
+            case 8: return filter_soa_g<T, 8>(p, in, out, st);
+            case 16: return filter_soa_g<T, 16>(p, in, out, st);
+            case 32: return filter_soa_g<T, 32>(p, in, out, st);
+        }
     }
     return set_error(LABFM_EINVAL, "unsupported group size");
 }
@@ -849,7 +853,7 @@ int rk_one_step_t(const labfm_plan* p, void* work, double dt, const labfm_phys* 
     Packed<T>* X = P + p->N;
     Packed<T>* Y = X + p->N;
     int* tickets = reinterpret_cast<int*>(Y + p->N);
-    if (p->persistent && !p->wexp) LABFM_CUDA_TRY(cudaMemsetAsync(tickets, 0, 4 * sizeof(int), st));
+    if (p->persistent && p->dtype == LABFM_F32) LABFM_CUDA_TRY(cudaMemsetAsync(tickets, 0, 4 * sizeof(int), st));
     int rc;
     labfm_plan* pm = const_cast<labfm_plan*>(p);  // only the launch-timing record changes
     const Packed<T>* xin[4] = {X, Y, X, Y};
@@ -915,15 +919,18 @@ template <typename T>
 int stage_rec_launch(const labfm_plan* p, const Packed<T>* xin, const Packed<T>* qin, Packed<T>* qout,
                      Packed<T>* xout, double dt, double bk, double ck, const Phys<T>& ph, D8<T>* D,
                      cudaStream_t st) {
-    if (p->wexp) return fixed_stage(p, 0, p->N, p->group, xin, qin, qout, xout, dt, bk, ck, as_phys(ph), D, st);
-    if (std::is_same<T, float>::value && !p->wall_slot && ahead_serves(p->N, p->group))
-        return ahead_stage(p, 0, p->N, p->group, xin, qin, qout, xout, dt, bk, ck, as_phys(ph), D, st);
-    switch (p->group) {
-        case 2: return stage_rec_launch_g<T, 2>(p, xin, qin, qout, xout, dt, bk, ck, ph, D, st);
-        case 4: return stage_rec_launch_g<T, 4>(p, xin, qin, qout, xout, dt, bk, ck, ph, D, st);
-        case 8: return stage_rec_launch_g<T, 8>(p, xin, qin, qout, xout, dt, bk, ck, ph, D, st);
-        case 16: return stage_rec_launch_g<T, 16>(p, xin, qin, qout, xout, dt, bk, ck, ph, D, st);
-        case 32: return stage_rec_launch_g<T, 32>(p, xin, qin, qout, xout, dt, bk, ck, ph, D, st);
+    if constexpr (std::is_same<T, double>::value) {
+        return fixed_stage(p, 0, p->N, p->group, xin, qin, qout, xout, dt, bk, ck, as_phys(ph), D, st);
+    } else {
+        if (!p->wall_slot && ahead_serves(p->N, p->group))
+            return ahead_stage(p, 0, p->N, p->group, xin, qin, qout, xout, dt, bk, ck, as_phys(ph), D, st);
+        switch (p->group) {
+            case 2: return stage_rec_launch_g<T, 2>(p, xin, qin, qout, xout, dt, bk, ck, ph, D, st);
+            case 4: return stage_rec_launch_g<T, 4>(p, xin, qin, qout, xout, dt, bk, ck, ph, D, st);
+            case 8: return stage_rec_launch_g<T, 8>(p, xin, qin, qout, xout, dt, bk, ck, ph, D, st);
+            case 16: return stage_rec_launch_g<T, 16>(p, xin, qin, qout, xout, dt, bk, ck, ph, D, st);
+            case 32: return stage_rec_launch_g<T, 32>(p, xin, qin, qout, xout, dt, bk, ck, ph, D, st);
+        }
     }
     return set_error(LABFM_EINVAL, "unsupported group size");
 }
@@ -1095,30 +1102,19 @@ int launch_rk_steps(const labfm_plan* p, void* Q, void* work, double dt, int nst
 }
 
 int filter_persistent_grid(const labfm_plan* p) {
+    if (p->dtype != LABFM_F32) return 0;  // F64 plans run one grid (fixed.cu)
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaError_t e = cudaErrorInvalidValue;
-#define LABFM_FOCC(T, G)                                                                            \
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(                                              \
-        &per_sm, k_filter_aos<T, G, std::is_same<T, float>::value, true>, p->block, 0)
-    const int g = filter_lanes(p);
-    if (p->dtype == LABFM_F32) {
-        switch (g) {
-            case 2: LABFM_FOCC(float, 2); break;
-            case 4: LABFM_FOCC(float, 4); break;
-            case 8: LABFM_FOCC(float, 8); break;
-            case 16: LABFM_FOCC(float, 16); break;
-            case 32: LABFM_FOCC(float, 32); break;
-        }
-    } else {
-        switch (g) {
-            case 2: LABFM_FOCC(double, 2); break;
-            case 4: LABFM_FOCC(double, 4); break;
-            case 8: LABFM_FOCC(double, 8); break;
-            case 16: LABFM_FOCC(double, 16); break;
-            case 32: LABFM_FOCC(double, 32); break;
-        }
+#define LABFM_FOCC(G) \
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_filter_aos<float, G, true, true>, p->block, 0)
+    switch (filter_lanes(p)) {
+        case 2: LABFM_FOCC(2); break;
+        case 4: LABFM_FOCC(4); break;
+        case 8: LABFM_FOCC(8); break;
+        case 16: LABFM_FOCC(16); break;
+        case 32: LABFM_FOCC(32); break;
     }
 #undef LABFM_FOCC
     if (e != cudaSuccess || per_sm < 1) per_sm = 1;
@@ -1126,31 +1122,19 @@ int filter_persistent_grid(const labfm_plan* p) {
 }
 
 int persistent_grid(const labfm_plan* p) {
+    if (p->dtype != LABFM_F32) return 0;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaError_t e = cudaErrorInvalidValue;
-#define LABFM_OCC(T, G)                                                                      \
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(                                       \
-        &per_sm, k_stage<T, G, std::is_same<T, float>::value, std::is_same<T, float>::value, \
-                         true>,                                                             \
-        kGatherBlock, 0)
-    if (p->dtype == LABFM_F32) {
-        switch (p->group) {
-            case 2: LABFM_OCC(float, 2); break;
-            case 4: LABFM_OCC(float, 4); break;
-            case 8: LABFM_OCC(float, 8); break;
-            case 16: LABFM_OCC(float, 16); break;
-            case 32: LABFM_OCC(float, 32); break;
-        }
-    } else {
-        switch (p->group) {
-            case 2: LABFM_OCC(double, 2); break;
-            case 4: LABFM_OCC(double, 4); break;
-            case 8: LABFM_OCC(double, 8); break;
-            case 16: LABFM_OCC(double, 16); break;
-            case 32: LABFM_OCC(double, 32); break;
-        }
+#define LABFM_OCC(G) \
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stage<float, G, true, true, true>, kGatherBlock, 0)
+    switch (p->group) {
+        case 2: LABFM_OCC(2); break;
+        case 4: LABFM_OCC(4); break;
+        case 8: LABFM_OCC(8); break;
+        case 16: LABFM_OCC(16); break;
+        case 32: LABFM_OCC(32); break;
     }
 #undef LABFM_OCC
     if (e != cudaSuccess || per_sm < 1) per_sm = 1;
@@ -1231,39 +1215,21 @@ int pack_plan(labfm_plan* p, const PlanInput* in, int n_inst, cudaStream_t st) {
         LABFM_CUDA_TRY(cudaMalloc(&p->inv_s, size_t(N) * es));
         p->device_bytes += N * es;
     }
-    // F64: in fixed point (fixed.cuh) where every row can be, else FP64 weights
-    if (p->dtype == LABFM_F64 && N < (int64_t(1) << 30)) {
+    if (p->dtype == LABFM_F64) {
         LABFM_CUDA_TRY(cudaMalloc(reinterpret_cast<void**>(&p->wexp), size_t(N) * 8 * sizeof(int16_t)));
-        int* unfit_dev = nullptr;
-        int unfit = 0;
-        LABFM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&unfit_dev), sizeof(int), st));
-        cudaError_t e = cudaMemsetAsync(unfit_dev, 0, sizeof(int), st);
-        for (int k = 0; k < n_inst && e == cudaSuccess && rc == LABFM_OK; ++k)
-            rc = fixed_pack(in[k], p->inst_off_host[k], p, unfit_dev, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&unfit, unfit_dev, sizeof(int), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        cudaFreeAsync(unfit_dev, st);
-        if (rc) return rc;
-        if (e != cudaSuccess) return cuda_error(e, "packing in fixed point");
-        if (!unfit) {
-            p->device_bytes += int64_t(N) * 8 * sizeof(int16_t);
-            return LABFM_OK;
-        }
-        cudaFree(p->wexp);
-        p->wexp = nullptr;
+        p->device_bytes += int64_t(N) * 8 * sizeof(int16_t);
     }
     for (int k = 0; k < n_inst; ++k) {
         const PlanInput& I = in[k];
         const int64_t off = p->inst_off_host[k];
+        if (p->dtype == LABFM_F64) {
+            if ((rc = fixed_pack(I, off, p, st))) return rc;
+            continue;
+        }
         const int gw = int(std::min<int64_t>((I.N * 32 + 255) / 256, 1 << 20));
-        if (p->dtype == LABFM_F32)
-            k_pack_rows<float, true><<<gw, 256, 0, st>>>(
-                I.N, I.nnz, nnz_pad, off, I.row_ptr, I.col, I.w, I.kappa, I.s, p->row_ptr, p->col,
-                static_cast<float*>(p->w), static_cast<float*>(p->wf), static_cast<float*>(p->inv_s));
-        else
-            k_pack_rows<double, false><<<gw, 256, 0, st>>>(
-                I.N, I.nnz, nnz_pad, off, I.row_ptr, I.col, I.w, I.kappa, I.s, p->row_ptr, p->col,
-                static_cast<double*>(p->w), static_cast<double*>(p->wf), nullptr);
+        k_pack_rows<float, true><<<gw, 256, 0, st>>>(I.N, I.nnz, nnz_pad, off, I.row_ptr, I.col, I.w, I.kappa, I.s,
+                                                     p->row_ptr, p->col, static_cast<float*>(p->w),
+                                                     static_cast<float*>(p->wf), static_cast<float*>(p->inv_s));
         LABFM_LAUNCH_CHECK("plan pack kernel");
     }
     LABFM_CUDA_TRY(cudaStreamSynchronize(st));

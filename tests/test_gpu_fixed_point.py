@@ -283,3 +283,101 @@ def test_fields_of_a_wide_span_within_a_stencil(lb, kind, m):
     for f in range(3):
         assert np.all(np.abs(filt[f] - (q[f] + S[5, f])) <= B[5, f] + 2 * u * np.abs(filt[f])), f
     plan.close()
+
+
+def _lattice_operator(lb, nx, ny, m, seed):
+    ns = li.tgv_lattice(nx, ny, m=m, jitter=0.05, seed=seed)
+    xy, h, s = (torch.tensor(a, device="cuda") for a in (ns.xy, ns.h, ns.s))
+    rp, col = lb.build_stencils(xy, h, ns.Lx, ns.Ly)
+    wb = lb.build_weights(xy, h, s, ns.Lx, ns.Ly, rp, col, m, residual=False)
+    return ns, {"row_ptr": rp, "col": col, "w": wb["w"], "kappa": wb["kappa"], "s": s}
+
+
+@pytest.mark.parametrize("weight", [np.nan, np.inf, 1e130, 1e-310])
+def test_a_row_out_of_the_fixed_range_changes_no_other_instance(lb, weight):
+    # an instance's bits alone and beside one with such a weight in one row (a failed node)
+    ns, a = _lattice_operator(lb, 22, 20, 4, 1)
+    nb, b = _lattice_operator(lb, 17, 19, 6, 2)
+    b["w"] = b["w"].clone()
+    b["w"][5, 40] = weight
+    alone = lb.Plan.batched([a], dtype=torch.float64)
+    both = lb.Plan.batched([b, a], dtype=torch.float64)
+    q = torch.tensor(li.tgv_fields(ns.xy, 10.0), device="cuda")
+    Q = torch.cat([torch.tensor(li.tgv_fields(nb.xy, 10.0), device="cuda"), q], dim=1).contiguous()
+    ph, part = lb.Phys(100.0, 0.005), slice(nb.N, None)
+    assert torch.equal(lb.rhs(both, Q, ph)[:, part], lb.rhs(alone, q, ph))
+    assert torch.equal(lb.filter(both, Q)[:, part], lb.filter(alone, q))
+    dt = float(lb.stable_dt(alone, q, a["s"], 10.0, 0.005).item())
+    assert torch.equal(lb.rk_step(both, Q, dt, 3, ph)[:, part], lb.rk_step(alone, q, dt, 3, ph))
+    alone.close()
+    both.close()
+
+
+def _plain_rows(op):
+    """The operator with one more entry in every row, on a node that is not in it (a column
+    stands in a row once), whose weights are subnormal (1e-310): rows that hold plain FP64
+    weights, with the same sums."""
+    rp, col, w = (op[k].cpu().numpy() for k in ("row_ptr", "col", "w"))
+    at = rp[1:]
+    N = len(at)
+    dev = lambda a: torch.tensor(np.ascontiguousarray(a), device="cuda")  # noqa: E731
+    return {**op, "row_ptr": dev((rp + np.arange(N + 1)).astype(np.int32)),
+            "col": dev(np.insert(col, at, (np.arange(N) + N // 2) % N).astype(np.int32)),
+            "w": dev(np.insert(w, at, 1e-310, axis=1))}
+
+
+def _close(a, b):
+    return bool((torch.linalg.vector_norm(a - b, dim=-1) <= 1e-12 * torch.linalg.vector_norm(b, dim=-1)).all())
+
+
+@pytest.mark.parametrize("group", [2, 4, 8, 16, 32])
+def test_plain_fp64_rows_through_every_call(lb, group):
+    # right-hand side, filter, steps, recorded steps, ranges and adjoints of a plan whose rows
+    # all hold FP64 weights, against the same operator in fixed point: the package's FP64 bar
+    ns, op = _lattice_operator(lb, 26, 25, 6, 3)
+    ph = lb.Phys(100.0, 0.005)
+    q = torch.tensor(li.tgv_fields(ns.xy, 10.0), device="cuda")
+    q[0] += 0.01 * torch.sin(torch.arange(ns.N, device="cuda"))
+    out = []
+    for o in (op, _plain_rows(op)):
+        plan = lb.Plan(o["row_ptr"], o["col"], o["w"], o["kappa"], o["s"], dtype=torch.float64)
+        plan.set_launch(group, 128)
+        lb.enable_adjoint(plan)
+        dt = float(lb.stable_dt(plan, q, o["s"], 10.0, 0.005).item())
+        r = [lb.rhs(plan, q, ph), lb.filter(plan, q), lb.rk_step(plan, q.clone(), dt, 3, ph)]
+        r.append(lb.rhs_adjoint(plan, q, r[0], ph))
+        r.append(lb.filter_adjoint(plan, r[0]))
+        q0 = q.clone().requires_grad_(True)
+        z = lb.rollout(plan, q0, dt, 4, ph, checkpoint_every=2)
+        lb.domain_kinetic_energy(z, o["s"]).backward()
+        r += [z.detach(), q0.grad]
+        plan.set_launch_ranges([0, 300, ns.N], [group, 4], [0, 0])
+        r.append(lb.rk_step(plan, q.clone(), dt, 2, ph))
+        out.append(r)
+        plan.close()
+    for a, b in zip(*out):
+        assert torch.isfinite(b).all() and _close(b, a)
+
+
+def test_plain_fp64_rows_beside_walls(lb):
+    ns = li.channel(24, 20, m=6, jitter=0.1, seed=4)
+    cols, normals = li.channel_walls(ns)
+    dev = lambda a, t=torch.float64: torch.tensor(np.ascontiguousarray(a), dtype=t, device="cuda")  # noqa: E731
+    xy, h, s = dev(ns.xy), dev(ns.h), dev(ns.s)
+    op = lb.build_wall_operator(xy, h, s, ns.Lx, ns.Ly, 6, 4, dev(cols, torch.int32), dev(normals), 1.7,
+                                periodic=(True, False), check=True)
+    op["s"] = s
+    ph = lb.Phys(400.0, ns.Ly / 10.0, 0.8, 0.0)
+    t = xy[:, 1] / ns.Ly
+    x = 2 * np.pi * xy[:, 0] / ns.Lx
+    q = torch.stack([0.01 * torch.sin(x), 4 * t * (1 - t), 0.01 * torch.sin(np.pi * t) * torch.cos(x)]).contiguous()
+    q[1:, dev(cols[:, 0], torch.int64)] = 0.0
+    out = []
+    for o in (op, _plain_rows(op)):
+        plan = lb.Plan(o["row_ptr"], o["col"], o["w"], o["kappa"], s, dtype=torch.float64)
+        plan.set_walls(dev(cols[:, 0], torch.int32), dev(normals))
+        dt = float(lb.stable_dt(plan, q, s, 20.0, ph.mu).item())
+        out.append([lb.rhs(plan, q, ph), lb.rk_step(plan, q.clone(), dt, 5, ph)])
+        plan.close()
+    for a, b in zip(*out):
+        assert torch.isfinite(b).all() and _close(b, a)
