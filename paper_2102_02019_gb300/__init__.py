@@ -279,20 +279,26 @@ def build_stencils(xy: torch.Tensor, h: torch.Tensor, Lx: float, Ly: float,
                    periodic=(True, True), stream=None):
     """CSR (row_ptr int32 [N+1], col int32 [nnz]) of |r_ji| <= 2 h_i (labfm_stencil_count, then
     labfm_stencil_fill over the cell list that the count left in its work buffer)."""
+    if stream is not None:
+        # a block of the current stream's pool may still be in use there: the buffers come
+        # from the search's own stream, and the results are marked as used on the current one
+        current = torch.cuda.current_stream()
+        own = stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(stream.cuda_stream)
+        with torch.cuda.stream(own):
+            row_ptr, col = build_stencils(xy, h, Lx, Ly, periodic)
+        row_ptr.record_stream(current)
+        col.record_stream(current)
+        return row_ptr, col
     N = _node_set(xy, h=h)
     mask = (1 if periodic[0] else 0) | (2 if periodic[1] else 0)
     row_ptr = torch.empty(N + 1, dtype=torch.int32, device=xy.device)
     work = torch.empty(int(lib.labfm_stencil_work_bytes(N)), dtype=torch.uint8, device=xy.device)
     nnz, longest = _I64(0), ctypes.c_int32(0)
-    st = _stream(stream)
+    st = _stream()
     args = (_ptr(xy), _ptr(h), N, Lx, Ly, mask, _ptr(row_ptr), _ptr(work), work.numel())
     _check(lib.labfm_stencil_count(*args, ctypes.byref(nnz), ctypes.byref(longest), st))
     col = torch.empty(max(nnz.value, 1), dtype=torch.int32, device=xy.device)
-    try:
-        _check(lib.labfm_stencil_fill(*args, nnz, longest, _ptr(col), col.numel(), st))
-    finally:
-        if stream is not None:  # the buffer is the current stream's: it outlives the search on the other
-            work.record_stream(stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(st))
+    _check(lib.labfm_stencil_fill(*args, nnz, longest, _ptr(col), col.numel(), st))
     return row_ptr, col[:nnz.value]
 
 

@@ -77,3 +77,24 @@ def test_search_on_another_stream(lb):
         rp2, col2 = lb.build_stencils(t, ht, 1.0, 1.0, stream=s)
         s.synchronize()
         assert torch.equal(rp, rp2) and torch.equal(col, col2)
+
+
+def test_search_on_another_stream_beside_work_on_freed_blocks(lb):
+    # blocks of the search's sizes, freed with a write of the current stream still to come: the
+    # search on the other stream takes none of them, for its cell list or for its results
+    rng = np.random.default_rng(4)
+    N = 5000
+    t, ht = torch.tensor(rng.uniform(size=(N, 2)), device="cuda"), torch.tensor(np.full(N, 0.03), device="cuda")
+    rp, col = lb.build_stencils(t, ht, 1.0, 1.0)
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for _ in range(3):
+        blocks = [torch.empty(n, dtype=torch.uint8, device="cuda")
+                  for n in (int(lb.lib.labfm_stencil_work_bytes(N)), 4 * (N + 1), 4 * len(col))]
+        torch.cuda._sleep(20_000_000)
+        for b in blocks:
+            b.fill_(255)
+        del b, blocks
+        rp2, col2 = lb.build_stencils(t, ht, 1.0, 1.0, stream=s)
+        torch.cuda.synchronize()
+        assert torch.equal(rp, rp2) and torch.equal(col, col2)
