@@ -246,19 +246,27 @@ template <int M>
 __device__ const AssemblyTables<M> d_tables{};
 
 // M_i[r][c] = 1/(a_r! b_r!) sum_{k,l} he_{a_c,k} he_{b_c,l} mu_{a_r+k, b_r+l} into
-// A (row stride LDA) and, when A0 is not null, a copy with stride n.  s_in:
-// AssemblyTables<M>::NI doubles of scratch.  Barriers inside, none at the end.
+// A (row stride LDA) and, when A0 is not null, a copy with stride n.  s_own: scratch for the
+// AssemblyTables<M>::NI inner sums (not used when OVERLAY).  Barriers inside, none at the end.
 //
 // The inner sums are formed once (729 at m = 8) instead of once per entry and k (8,300
 // products), and the index arithmetic is read from tables: it had cost more than the
 // sums.  Same operations on the same numbers in the same order as entry by entry, so the
-// matrix is the same bit for bit.  The whole weight build of 65,536 nodes, order 8: 16.83
-// -> 16.0 ms.
-template <int M, int LDA>
-__device__ void block_assemble(double* A, double* A0, const double* s_mu, const double* s_he, double* s_in) {
+// matrix is the same bit for bit.  OVERLAY: the sums lie in the last rows of A, whose entries
+// wait in registers (7 a thread at most) until all have been read.  That is for the kernels
+// from which an array of their own takes a block an SM (9 -> 8 at m = 8, 5 -> 4 at m = 10
+// without the residual); the others keep them where the weight polynomials' coefficients go
+// later.  The whole weight build of 65,536 nodes without the residual, entry by entry -> now:
+// order 4 3.41 -> 3.32 ms, 6 7.09 -> 6.74, 8 16.77 -> 15.80, 10 38.1 -> 35.7 (with an array
+// 38.4); with it, order 8 19.0 -> 18.2 (with an array 18.8).
+template <int M, int LDA, bool OVERLAY>
+__device__ void block_assemble(double* A, double* A0, const double* s_mu, const double* s_he, double* s_own) {
     using C = WCfg<M>;
     using Tab = AssemblyTables<M>;
     constexpr int n = C::n, NT = C::NT;
+    constexpr int R = OVERLAY ? (Tab::NI + LDA - 1) / LDA : 0, R0 = n - R;  // rows that hold the sums, rows before them
+    static_assert(R0 >= 0, "the inner sums fit in the matrix");
+    double* s_in = OVERLAY ? A + R0 * LDA : s_own;
     for (int idx = threadIdx.x; idx < Tab::NI; idx += NT) {
         const uint32_t t = d_tables<M>.inner[idx];
         const int bc = t & 255, br = (t >> 8) & 255, pp = t >> 16;
@@ -270,19 +278,39 @@ __device__ void block_assemble(double* A, double* A0, const double* s_mu, const 
         s_in[idx] = inner;
     }
     __syncthreads();
-    // column-major over the threads: the lanes of a warp share the column c, whose
-    // Hermite exponent fixes the trip count below (no divergence)
-    for (int idx = threadIdx.x; idx < n * n; idx += NT) {
-        const int c = idx / n, r = idx - c * n;
+    auto entry = [&](int r, int c) {
         const uint32_t er = d_tables<M>.ex[r], ec = d_tables<M>.ex[c];
         const int ar = er & 255, br = er >> 8, ac = ec & 255, bc = ec >> 8;
         const double* in = s_in + d_tables<M>.base[bc * (M + 1) + br] + ar;
         const double* he = s_he + ac * (M + 1);
         double sum = 0.0;
         for (int k = ac; k >= 0; k -= 2) sum = fma(he[k], in[k], sum);
-        const double v = sum * d_tables<M>.scale[r];
+        return sum * d_tables<M>.scale[r];
+    };
+    auto put = [&](int r, int c, double v) {
         A[r * LDA + c] = v;
         if (A0) A0[r * n + c] = v;
+    };
+    // column-major over the threads: the lanes of a warp share the column c, whose
+    // Hermite exponent fixes the trip count (no divergence)
+    for (int idx = threadIdx.x; idx < R0 * n; idx += NT) {
+        const int c = idx / R0, r = idx - c * R0;
+        put(r, c, entry(r, c));
+    }
+    if constexpr (OVERLAY) {
+        constexpr int PER = (R * n + NT - 1) / NT;
+        double v[PER];
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int idx = threadIdx.x + u * NT, c = idx / R;
+            if (idx < R * n) v[u] = entry(R0 + idx - c * R, c);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int idx = threadIdx.x + u * NT, c = idx / R;
+            if (idx < R * n) put(R0 + idx - c * R, c, v[u]);
+        }
     }
 }
 
@@ -424,9 +452,9 @@ __global__ void __launch_bounds__(WCfg<M>::NT)
     double* A0 = smem + n * LDA;   // [n][n] copy of M for the residual
     __shared__ double s_mu[C::NMOM];
     __shared__ double s_he[(M + 1) * (M + 1)];
-    // the assembly's inner sums, then the weight polynomials' coefficients
-    __shared__ double s_in[AssemblyTables<M>::NI > NC * 6 ? AssemblyTables<M>::NI : NC * 6];
-    double* s_cf = s_in;
+    constexpr bool kOverlay = M == 8 || (M == 10 && !RESID);
+    // the assembly's inner sums (unless they lie in A), then the weight polynomials' coefficients
+    __shared__ double s_cf[!kOverlay && AssemblyTables<M>::NI > NC * 6 ? AssemblyTables<M>::NI : NC * 6];
     __shared__ int s_piv;
     __shared__ int s_flag;
     __shared__ int s_nonfinite;
@@ -460,7 +488,7 @@ __global__ void __launch_bounds__(WCfg<M>::NT)
     if (t <= 2 * M) s_hp[t] = pow(g.hi, double(t - M));
     build_he<M>(s_he);
     block_moments<M>(xy, col, r0, r1, g, smem, smem + C::MCH * C::NPOW, s_mu);
-    block_assemble<M, LDA>(A, RESID ? A0 : nullptr, s_mu, s_he, s_in);
+    block_assemble<M, LDA, kOverlay>(A, RESID ? A0 : nullptr, s_mu, s_he, s_cf);
     for (int idx = t; idx < n * 6; idx += NT) {  // selectors C~^d
         const int q = idx / 6, d = idx - q * 6;
         int a, b;
@@ -792,10 +820,10 @@ __global__ void __launch_bounds__(WCfg<M>::NT, stencil_opt_min_blocks<M>())
     __shared__ double s_he[(M + 1) * (M + 1)];
     __shared__ double s_red[NT / 32];
     __shared__ double s_part[(NT / 32) * 3 * kNk];
+    constexpr bool kOverlay = M >= 8;
     constexpr int kCf3 = (M + 1) * (M + 2) / 2 * 3;
-    // the assembly's inner sums, then the weight polynomials' coefficients
-    __shared__ double s_in[AssemblyTables<M>::NI > kCf3 ? AssemblyTables<M>::NI : kCf3];
-    double* s_cf3 = s_in;
+    // the assembly's inner sums (unless they lie in A), then the weight polynomials' coefficients
+    __shared__ double s_cf3[!kOverlay && AssemblyTables<M>::NI > kCf3 ? AssemblyTables<M>::NI : kCf3];
     __shared__ double s_hp[M + 1];
     __shared__ double s_amax;
     __shared__ double s_rdiag[n];
@@ -831,7 +859,7 @@ __global__ void __launch_bounds__(WCfg<M>::NT, stencil_opt_min_blocks<M>())
         if (block_sum<NT>(cnt, s_red) < double(n)) break;
         // Section 4 steps 1-2: solve for x, y and L and test the Laplacian residual
         block_moments<M>(xy, col, r0, r1, g, smem, smem + C::MCH * C::NPOW, s_mu);
-        block_assemble<M, LDA>(A, A0, s_mu, s_he, s_in);
+        block_assemble<M, LDA, kOverlay>(A, A0, s_mu, s_he, s_cf3);
         for (int idx = t; idx < n * 3; idx += NT) {
             const int q = idx / 3, d = idx - q * 3;
             int a, b;
