@@ -470,7 +470,8 @@ int labfm_stable_dt_instances(const labfm_plan* plan, const void* fields, const 
  * takes tiles of consecutive nodes from a work-queue ticket (reset at every
  * step), which balances uneven stencils and mixed instances dynamically.  The
  * workspace grows by 64 bytes for the tickets (query labfm_rk_workspace_bytes
- * after changing this).
+ * after changing this).  F32 plans only: accepted for F64 plans, whose stages run
+ * one kernel whatever the setting.
  */
 int labfm_plan_set_persistent(labfm_plan* plan, int enable);
 
@@ -483,19 +484,23 @@ int labfm_plan_set_persistent(labfm_plan* plan, int enable);
  * Results do not change.  Rows of fewer than 48 padded entries are
  * never prefetched (measured faster for the rows of m = 6, 8 and 10, ~60-220
  * entries; a lower threshold slowed the ~35-entry rows of m = 4).  Plan creation sets 2 for F32 plans and 0 for F64
- * plans (whose kernels do not prefetch).  Host-only call.
+ * plans (whose kernels have a fixed prefetch of their own).  The F32 kernels of
+ * small launches (lanes per node x nodes up to 56 warps an SM: 68,096 nodes at 4
+ * lanes on 152 SMs), which keep whole chunks in flight instead, do not use it.
+ * Host-only call.
  */
 int labfm_plan_set_prefetch(labfm_plan* plan, int distance);
 
 /*
  * Programmatic dependent launches (enable = 1, the default) or plain launches
  * (enable = 0) for the plan's plain-grid stage, filter, recording-stage, adjoint,
- * pack and unpack kernels.  With them on, each such kernel is launched with
- * programmatic stream serialization: it may start while the previous kernel of the
- * stream finishes, reads only the plan's constant operator (row pointers, and an L2
- * prefetch of its rows' first record blocks) until griddepcontrol.wait has seen the
- * previous kernel complete, and only then reads or writes the state; results are
- * bit-identical either way.  No counterpart in the paper: a launch-scheduling
+ * pack and unpack kernels, and for labfm_rhs and labfm_filter of F64 plans.  With
+ * them on, each such kernel is launched with programmatic stream serialization: it
+ * may start while the previous kernel of the stream finishes, and until
+ * griddepcontrol.wait has seen the previous kernel complete it reads only what the
+ * plan's creation wrote (row pointers, node spacings, the rows' exponents, and its
+ * rows' first records, into registers or into L2); only then does it read or write
+ * the state, the time steps and the boundaries; results are bit-identical either way.  No counterpart in the paper: a launch-scheduling
  * setting (sm_90 and later).  EINVAL for another value of enable.  Host-only call.
  */
 int labfm_plan_set_programmatic_launch(labfm_plan* plan, int enable);
@@ -566,8 +571,10 @@ int labfm_plan_get_info(const labfm_plan* plan, labfm_plan_info* info);
  * Override the launch shape: `group` lanes per node (2, 4, 8, 16 or 32) in every
  * gather kernel, and `block` threads per block (a multiple of 32 and of group,
  * 64..1024) for the filter and filter-transpose kernels; the fused right-hand-side,
- * stage and adjoint gather kernels always run one-warp (32-thread) blocks.  Defaults: group 4, block 128;
- * labfm_plan_autotune picks the fastest group.
+ * stage and adjoint gather kernels of F32 plans always run one-warp (32-thread)
+ * blocks.  Of an F64 plan the right-hand-side, stage and filter kernels run two-warp
+ * blocks and at most 16 lanes per node (32 is accepted, and holds for the adjoint
+ * gathers).  Defaults: group 4, block 128; labfm_plan_autotune picks the fastest group.
  */
 int labfm_plan_set_launch(labfm_plan* plan, int group, int block);
 
@@ -594,14 +601,16 @@ int labfm_plan_set_launch_ranges(labfm_plan* plan, int n, const int64_t* begin, 
  * blocks) whose warps stride over the nodes, so that no partly filled last wave
  * of blocks leaves the GPU idle (0 = one group per node over a full grid).
  * The filtered state does not depend on `persistent`; with another lane count
- * the filter sums are added in another order (FP rounding only).  Host-only.
+ * the filter sums are added in another order (FP rounding only).  `persistent` is
+ * for F32 plans (accepted for F64 plans, without effect).  Host-only.
  * Errors: EINVAL (unsupported lanes per node).
  */
 int labfm_plan_set_filter_launch(labfm_plan* plan, int group, int persistent);
 
 /*
  * Time every supported group size on this plan with CUDA events (the RHS
- * kernel on `fields`, `reps` launches each) and keep the fastest.
+ * kernel on `fields`, `reps` launches each; 32 on F32 plans only) and keep the
+ * fastest.
  * Writes the chosen pair to *group_out / *block_out (host, may be NULL).
  * Synchronises `stream`.
  */

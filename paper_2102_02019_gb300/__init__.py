@@ -687,19 +687,24 @@ class Plan:
                   groups=(2, 4, 8, 16), staged=((16, 3), (32, 3), (32, 4)),
                   prefetch=(0, 2), filter_groups=(2, 4, 8, 16), filter_blocks=(64, 128)) -> dict:
         """Autotune the time step itself: time `steps` RK steps (CUDA events) for every
-        lanes-per-node group with the plain and the persistent stage kernel (F32: with
-        each L2 prefetch distance), and (F32) for the staged kernel at the given (lanes
-        per node, ring slots), keep the fastest; then, with that stage kernel, time the
-        filter's own lanes per node with its plain and persistent grids and the plan's
-        block size (which only the filter and filter-transpose kernels use; the stage and
-        adjoint gather kernels run one-warp blocks), and keep the fastest.  Q is not modified.  Returns the chosen configuration."""
+        lanes-per-node group (F32: with the plain and the persistent stage kernel and each
+        L2 prefetch distance, and for the staged kernel at the given (lanes per node, ring
+        slots)) and keep the fastest; then, with that stage kernel, time the filter's own
+        lanes per node (F32: with its plain and persistent grids and the plan's block size,
+        which only the filter and filter-transpose kernels use) and keep the fastest.  Q is
+        not modified.  Returns the chosen configuration."""
         _state(self, Q)
         info = self.info()
         block = info["block"]
-        pfs = tuple(prefetch) if self.dtype == torch.float32 else (info["prefetch"],)
-        configs = [(g, p, 0, pf) for pf in pfs for p in (False, True) for g in groups]
-        if self.dtype == torch.float32:
+        # F64 plans have one stage and one filter kernel, without a prefetch distance or a block size
+        f32 = self.dtype == torch.float32
+        grids = (False, True) if f32 else (False,)
+        pfs = tuple(prefetch) if f32 else (info["prefetch"],)
+        configs = [(g, p, 0, pf) for pf in pfs for p in grids for g in groups]
+        if f32:
             configs += [(g, False, k, 0) for g, k in staged]
+        else:
+            filter_blocks = (block,)
 
         def timed():
             work = workspace(self)
@@ -734,7 +739,7 @@ class Plan:
                 if fb % fg or fb % 32:
                     continue
                 self.set_launch(g, fb)
-                for fp in (False, True):
+                for fp in grids:
                     self.set_filter_launch(fg, fp)
                     ms = timed()
                     if ms < fbest[0]:

@@ -258,7 +258,7 @@ __device__ const AssemblyTables<M> d_tables{};
 // without the residual); the others keep them where the weight polynomials' coefficients go
 // later.  The whole weight build of 65,536 nodes without the residual, entry by entry -> now:
 // order 4 3.41 -> 3.32 ms, 6 7.09 -> 6.74, 8 16.77 -> 15.80, 10 38.1 -> 35.7 (with an array
-// 38.4); with it, order 8 19.0 -> 18.2 (with an array 18.8).
+// 38.4); with it, order 8 19.0 -> 18.2 to 18.5 (with an array 18.8).
 template <int M, int LDA, bool OVERLAY>
 __device__ void block_assemble(double* A, double* A0, const double* s_mu, const double* s_he, double* s_own) {
     using C = WCfg<M>;

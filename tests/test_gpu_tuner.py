@@ -57,3 +57,29 @@ def test_tuned_shape_is_applied_and_reproducible(lb, dtype):
     assert torch.equal(Q, Qr)
     plan.close()
     ref.close()
+
+
+def test_tuners_leave_out_settings_that_f64_plans_do_not_have(lb):
+    # 32 lanes run as 16, and there is no persistent grid: neither is picked, by noise or otherwise
+    ns = li.tgv_lattice(24, 22, m=4, jitter=0.1, seed=82, s=1.0 / 24)
+    xy, h, s = (torch.tensor(a, device="cuda") for a in (ns.xy, ns.h, ns.s))
+    rp, col = lb.build_stencils(xy, h, ns.Lx, ns.Ly)
+    wb = lb.build_weights(xy, h, s, ns.Lx, ns.Ly, rp, col, ns.m)
+    phys = lb.Phys(C * C, MU)
+    plan = lb.Plan(rp, col, wb["w"], wb["kappa"], s, dtype=torch.float64)
+    Q = torch.tensor(li.tgv_fields(ns.xy, C), device="cuda")
+    dt = float(lb.stable_dt(plan, Q, s, C, MU).item())
+    for _ in range(10):
+        plan.autotune(Q, phys, reps=1)
+        assert plan.info()["group"] in (2, 4, 8, 16)
+    for _ in range(5):
+        cfg = plan.tune_step(Q, phys, dt, steps=1)
+        assert not cfg["persistent"] and not cfg["filter_persistent"] and cfg["staging"] == 0
+    # accepted all the same, and without effect on the state
+    out = []
+    for on in (False, True):
+        plan.set_persistent(on)
+        plan.set_filter_launch(0, on)
+        out.append(lb.rk_step(plan, Q.clone(), dt, 3, phys))
+    assert torch.equal(out[0], out[1])
+    plan.close()
