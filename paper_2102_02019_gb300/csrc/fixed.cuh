@@ -215,8 +215,8 @@ __device__ __forceinline__ void raise_bound(uint32_t m, int& T, long long* hi, l
 }
 
 // Moves the carries of the low sums up, so that a lane can take rows of any length: due
-// every kFold chunks (64 entries).
-constexpr int kFold = 16;
+// every kFold chunks (32 entries).
+constexpr int kFold = 8;
 template <int K>
 __device__ __forceinline__ void fold(long long (&hi)[K], long long (&mid)[K]) {
 #pragma unroll

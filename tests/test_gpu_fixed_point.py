@@ -381,3 +381,23 @@ def test_plain_fp64_rows_beside_walls(lb):
         plan.close()
     for a, b in zip(*out):
         assert torch.isfinite(b).all() and _close(b, a)
+
+
+@pytest.mark.parametrize("n", [32, 64, 128, 256])
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_the_largest_low_sums_do_not_overflow(lb, n, sign):
+    # digits at their largest and all products of one sign: weights 1 - 2^-53, differences
+    # with a high digit of 2^29 - 1 and the largest low digit, rows of 64 entries a lane and more
+    N = n + 1
+    rp = np.concatenate([[0], np.full(N, n).cumsum()]).astype(np.int32)
+    col = np.concatenate([[j for j in range(N) if j != i] for i in range(N)]).astype(np.int32)
+    w = np.full((6, len(col)), sign * (1 - 2.0 ** -53))
+    q = np.full((3, N), 1 - 2.0 ** -30 - 2.0 ** -50)
+    q[0] = 0.0
+    q[1:, 0] = 0.0
+    plan = _plan(lb, rp, col, w, np.ones(N))
+    plan.set_launch(2, 128)
+    _check(lb, plan, rp, col, w, np.ones(N), q)
+    q[0] = q[1]
+    _check(lb, plan, rp, col, w, np.ones(N), q)
+    plan.close()
