@@ -12,28 +12,27 @@
 namespace labfm {
 namespace {
 
-// Resident warps per SM that the registers allow for (96 registers; the filter spills 240
-// bytes in 72, and 262,144 nodes of order 8 take 230 us with 28 warps and 225 with 20).
-#ifndef LABFM_FIXED_RHS_WARPS
-#define LABFM_FIXED_RHS_WARPS 20
-#endif
-#ifndef LABFM_FIXED_FILTER_WARPS
-#define LABFM_FIXED_FILTER_WARPS 20
-#endif
-#define LABFM_FIXED_BOUNDS __launch_bounds__(32 * kFixedWarps, LABFM_FIXED_RHS_WARPS / kFixedWarps)
-#define LABFM_FIXED_FILTER_BOUNDS __launch_bounds__(32 * kFixedWarps, LABFM_FIXED_FILTER_WARPS / kFixedWarps)
+// Resident warps per SM that the registers allow for.  The right-hand-side kernels come with
+// 96 registers (20 warps, a few spills), with 128 (16 warps, none) and, for launches that are
+// bound by the latency of one warp, with the next chunk's gathers in flight (157 registers,
+// 12 warps): see warps_for.  The filter has 96 (it spills 240 bytes in 72: 262,144 nodes of
+// order 8 230 us with 28 warps, 225 with 20).
+constexpr int kManyWarps = 20, kFewWarps = 16, kAheadWarps = 12, kFilterWarps = 20;
+#define LABFM_FIXED_BOUNDS __launch_bounds__(32 * kFixedWarps, W / kFixedWarps)
+#define LABFM_FIXED_FILTER_BOUNDS __launch_bounds__(32 * kFixedWarps, kFilterWarps / kFixedWarps)
 
 // Launched so that they may start when the launch before ends (launch_pdl), with the row
 // pointers read before the wait for it, but without an early griddepcontrol.launch_dependents:
 // the next launch's blocks, placed beside this one's, crowd some SMs' pipes while others
 // idle.  A step of 10,000 nodes of order 6 takes 173 us with it and 108 without, of 40,000
 // 268 and 243, a right-hand side of 4,096 nodes of order 4 23.3 and 11.6; a right-hand side
-// of 1,073 nodes 14.3 us launched plainly and 11.8 so.
+// of 1,073 nodes 14.3 us launched plainly and 11.8 so.  Where the next launch finds idle SMs
+// it gives nothing (576 nodes of order 4 55.9 us a step with it, 55.5 without).
 
-template <int G, bool WALL>
+template <int W, int G, bool WALL>
 __global__ void LABFM_FIXED_BOUNDS k_fixed_rhs(PlanView<double> P, Fields in, double* __restrict__ out,
                                                Phys<double> ph, int passes) {
-    fixed_nodes<G, false>(P, in, passes,
+    fixed_nodes<G, false, W == kAheadWarps>(P, in, passes,
                           [&](int i, double a, double u, double v, const double (&d)[12]) {
                               double Ra, Ru, Rv;
                               node_rhs<double, false, WALL>(P, i, d, a, u, v, 1.0, ph, Ra, Ru, Rv);
@@ -44,12 +43,12 @@ __global__ void LABFM_FIXED_BOUNDS k_fixed_rhs(PlanView<double> P, Fields in, do
 }
 
 // REC: also stores the node's derivative combinations (k_stage_rec).
-template <int G, bool WALL, bool REC>
+template <int W, int G, bool WALL, bool REC>
 __global__ void LABFM_FIXED_BOUNDS k_fixed_stage(PlanView<double> P, const Packed<double>* X_in,
                                                  const Packed<double>* Q_in, Packed<double>* Q_out,
                                                  Packed<double>* X_out, double dt, double bk, double ck,
                                                  Phys<double> ph, D8<double>* Dout, int passes) {
-    fixed_nodes<G, false>(P, State{X_in}, passes,
+    fixed_nodes<G, false, W == kAheadWarps>(P, State{X_in}, passes,
                           [&](int i, double a, double u, double v, const double (&d)[12]) {
                               stage_epilogue<double, false, WALL>(P, i, 0, d, a, u, v, X_in, Q_in, Q_out, X_out,
                                                                   dt, bk, ck, ph);
@@ -61,10 +60,10 @@ __global__ void LABFM_FIXED_BOUNDS k_fixed_stage(PlanView<double> P, const Packe
                           });
 }
 
-template <int G>
+template <int W, int G>
 __global__ void LABFM_FIXED_BOUNDS k_fixed_coeffs(PlanView<double> P, const Packed<double>* X, D8<double>* Dout,
                                                   int passes) {
-    fixed_nodes<G, false>(P, State{X}, passes,
+    fixed_nodes<G, false, W == kAheadWarps>(P, State{X}, passes,
                           [&](int i, double, double, double, const double (&d)[12]) {
                               double c[8];
                               own_coeffs<double, false>(d, 1.0, c);
@@ -75,7 +74,7 @@ __global__ void LABFM_FIXED_BOUNDS k_fixed_coeffs(PlanView<double> P, const Pack
 template <int G>
 __global__ void LABFM_FIXED_FILTER_BOUNDS k_fixed_filter(PlanView<double> P, const Packed<double>* in, Packed<double>* out,
                                                   double* soa, int passes) {
-    fixed_nodes<G, true>(P, State{in}, passes,
+    fixed_nodes<G, true, false>(P, State{in}, passes,
                          [&](int i, double a, double u, double v, const double (&s)[3]) {
                              store(out, i, a + s[0], u + s[1], v + s[2]);
                              if (soa) {
@@ -89,7 +88,7 @@ __global__ void LABFM_FIXED_FILTER_BOUNDS k_fixed_filter(PlanView<double> P, con
 template <int G>
 __global__ void LABFM_FIXED_FILTER_BOUNDS k_fixed_filter_soa(PlanView<double> P, Fields in, double* __restrict__ out,
                                                       int passes) {
-    fixed_nodes<G, true>(P, in, passes,
+    fixed_nodes<G, true, false>(P, in, passes,
                          [&](int i, double a, double u, double v, const double (&s)[3]) {
                              out[i] = a + s[0];
                              out[P.N + i] = u + s[1];
@@ -237,11 +236,15 @@ int lanes_for(int group) { return std::min(group, 16); }
 int filter_lanes_for(int group) { return lanes_for(group); }
 
 // Passes per warp: all the lanes' worth (32 nodes a warp, so that the work after the sums
-// runs on 32 lanes: 262,144 nodes of order 8, one pass 463 us, two 411, four 384) where
-// that still leaves every SM half its warps, else fewer, so that small node sets spread
-// over the chip (40,000 nodes of order 6: one pass 69 us, two 58, four 78).
-int passes_for(int64_t nodes, int g) {
-    int passes = g;
+// runs on 32 lanes: 262,144 nodes of order 8, one pass 511 us, two 465, four 459) where
+// that still leaves every SM ten warps, else fewer, so that small node sets spread
+// over the chip (40,000 nodes of order 6: one pass 69 us, two 58, four 78).  The filter, which
+// has little work after its sums, takes two at most, for the finer waves (122,500 nodes of
+// order 10 138 us, with four 164; 262,144 of order 8 221 and 225; 90,000 of order 6 52.5 and
+// 51.2).
+constexpr int kRhsPasses = 16, kFilterPasses = 2;
+int passes_for(int64_t nodes, int g, int most) {
+    int passes = std::min(g, most);
     while (passes > 1 && nodes * g / (32 * passes) < int64_t(152) * 10) passes /= 2;
     return passes;
 }
@@ -249,6 +252,21 @@ int passes_for(int64_t nodes, int g) {
 int grid_of(int64_t nodes, int g, int passes) {
     const int64_t per = int64_t(passes) * kFixedWarps * (32 / g);
     return int((nodes + per - 1) / per);
+}
+
+// Which of the right-hand-side kernels a grid takes.  Where all its warps fit at 12 an SM, a
+// launch takes as long as one warp does, and the one that gathers ahead is the fastest (us a
+// right-hand side, ahead and with 128 registers: 576 nodes of order 4 10.7 and 12.0, of order
+// 8 17.4 and 21.0; 4,096 of order 8 18.0 and 21.7; 25,600 of order 6 35.4 and 39.1; 28,900 of
+// order 8 56.3 and 62.8).  Else the one with 128
+// registers where it takes no more waves than that with 96 (62,500 nodes of order 8 126 and
+// 138; 65,536 of order 4 55 and 60; 122,500 of order 10 304 and 325), since it loses the wave
+// otherwise (40,000 of order 6 71 and 58; 90,000 153 and 109; 262,144 of order 8 459 and 433).
+// Ahead with 128 registers: 65,536 nodes of order 4 58.
+int warps_for(int grid) {
+    auto waves = [&](int warps) { return (grid - 1) / (152 * (warps / kFixedWarps)); };
+    if (waves(kAheadWarps) == 0) return kAheadWarps;
+    return waves(kFewWarps) == waves(kManyWarps) ? kFewWarps : kManyWarps;
 }
 
 #define LABFM_FIXED_DISPATCH(g, call)                         \
@@ -259,6 +277,17 @@ int grid_of(int64_t nodes, int g, int passes) {
         case 16: { constexpr int G = 16; call; break; }       \
         default: return set_error(LABFM_EINVAL, "unsupported group size"); \
     }
+// kernel<W, G, ...> for the grid's number of warps
+#define LABFM_FIXED_LAUNCH(g, grid, kernel, ...)                                               \
+    switch (warps_for(grid)) {                                                                 \
+        case kAheadWarps: { constexpr int W = kAheadWarps;                                     \
+            LABFM_FIXED_DISPATCH(g, (e = launch(kernel<W, G __VA_ARGS__>))); break; }          \
+        case kFewWarps: { constexpr int W = kFewWarps;                                         \
+            LABFM_FIXED_DISPATCH(g, (e = launch(kernel<W, G __VA_ARGS__>))); break; }          \
+        default: { constexpr int W = kManyWarps;                                               \
+            LABFM_FIXED_DISPATCH(g, (e = launch(kernel<W, G __VA_ARGS__>))); }                 \
+    }
+#define LABFM_COMMA ,
 
 Phys<double> phys_of(const labfm_phys& ph) { return Phys<double>{ph.c2, ph.mu, ph.gx, ph.gy}; }
 
@@ -274,7 +303,7 @@ PlanView<double> view_of(const labfm_plan* p, int64_t n_lo, int64_t n_hi) {
 int fixed_rhs(const labfm_plan* p, const void* fields, void* rhs, const labfm_phys& php, int group, cudaStream_t st) {
     const double* f = static_cast<const double*>(fields);
     const Fields in{f, f + p->N, f + 2 * p->N};
-    const int g = lanes_for(group), passes = passes_for(p->N, g);
+    const int g = lanes_for(group), passes = passes_for(p->N, g, kRhsPasses);
     const int grid = grid_of(p->N, g, passes);
     double* out = static_cast<double*>(rhs);
     auto launch = [&](auto* kernel) {
@@ -282,9 +311,9 @@ int fixed_rhs(const labfm_plan* p, const void* fields, void* rhs, const labfm_ph
     };
     cudaError_t e = cudaSuccess;
     if (p->wall_slot) {
-        LABFM_FIXED_DISPATCH(g, (e = launch(k_fixed_rhs<G, true>)));
+        LABFM_FIXED_LAUNCH(g, grid, k_fixed_rhs, LABFM_COMMA true);
     } else {
-        LABFM_FIXED_DISPATCH(g, (e = launch(k_fixed_rhs<G, false>)));
+        LABFM_FIXED_LAUNCH(g, grid, k_fixed_rhs, LABFM_COMMA false);
     }
     if (e != cudaSuccess) return cuda_error(e, "fixed-point rhs kernel");
     return LABFM_OK;
@@ -294,7 +323,7 @@ int fixed_stage(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, cons
                 void* qout, void* xout, double dt, double bk, double ck, const labfm_phys& php, void* D,
                 cudaStream_t st) {
     if (n_hi <= n_lo) return LABFM_OK;
-    const int g = lanes_for(group), passes = passes_for(n_hi - n_lo, g);
+    const int g = lanes_for(group), passes = passes_for(n_hi - n_lo, g, kRhsPasses);
     const int grid = grid_of(n_hi - n_lo, g, passes);
     const PlanView<double> v = view_of(p, n_lo, n_hi);
     auto launch = [&](auto* kernel) {
@@ -305,21 +334,21 @@ int fixed_stage(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, cons
     };
     cudaError_t e = cudaSuccess;
     if (D) {
-        LABFM_FIXED_DISPATCH(g, (e = launch(k_fixed_stage<G, false, true>)));
+        LABFM_FIXED_LAUNCH(g, grid, k_fixed_stage, LABFM_COMMA false LABFM_COMMA true);
     } else if (p->wall_slot) {
-        LABFM_FIXED_DISPATCH(g, (e = launch(k_fixed_stage<G, true, false>)));
+        LABFM_FIXED_LAUNCH(g, grid, k_fixed_stage, LABFM_COMMA true LABFM_COMMA false);
     } else {
-        LABFM_FIXED_DISPATCH(g, (e = launch(k_fixed_stage<G, false, false>)));
+        LABFM_FIXED_LAUNCH(g, grid, k_fixed_stage, LABFM_COMMA false LABFM_COMMA false);
     }
     if (e != cudaSuccess) return cuda_error(e, "fixed-point rk stage kernel");
     return LABFM_OK;
 }
 
 int fixed_coeffs(const labfm_plan* p, const void* X, void* D, cudaStream_t st) {
-    const int g = lanes_for(p->group), passes = passes_for(p->N, g);
+    const int g = lanes_for(p->group), passes = passes_for(p->N, g, kRhsPasses);
     const int grid = grid_of(p->N, g, passes);
     cudaError_t e = cudaSuccess;
-    LABFM_FIXED_DISPATCH(g, (e = launch_pdl(p, k_fixed_coeffs<G>, grid, 32 * kFixedWarps, st, view<double>(p),
+    LABFM_FIXED_DISPATCH(g, (e = launch_pdl(p, k_fixed_coeffs<kManyWarps, G>, grid, 32 * kFixedWarps, st, view<double>(p),
                                             static_cast<const Packed<double>*>(X), static_cast<D8<double>*>(D), passes)));
     if (e != cudaSuccess) return cuda_error(e, "fixed-point derivative kernel");
     return LABFM_OK;
@@ -328,7 +357,7 @@ int fixed_coeffs(const labfm_plan* p, const void* X, void* D, cudaStream_t st) {
 int fixed_filter(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, const void* in, void* out, void* soa,
                  cudaStream_t st) {
     if (n_hi <= n_lo) return LABFM_OK;
-    const int g = filter_lanes_for(group), passes = passes_for(n_hi - n_lo, g);
+    const int g = filter_lanes_for(group), passes = passes_for(n_hi - n_lo, g, kFilterPasses);
     const int grid = grid_of(n_hi - n_lo, g, passes);
     const PlanView<double> v = view_of(p, n_lo, n_hi);
     cudaError_t e = cudaSuccess;
@@ -341,7 +370,7 @@ int fixed_filter(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, con
 int fixed_filter_soa(const labfm_plan* p, const void* in, void* out, cudaStream_t st) {
     const double* f = static_cast<const double*>(in);
     const Fields src{f, f + p->N, f + 2 * p->N};
-    const int g = filter_lanes_for(p->group), passes = passes_for(p->N, g);
+    const int g = filter_lanes_for(p->group), passes = passes_for(p->N, g, kFilterPasses);
     const int grid = grid_of(p->N, g, passes);
     cudaError_t e = cudaSuccess;
     LABFM_FIXED_DISPATCH(g, (e = launch_pdl(p, k_fixed_filter_soa<G>, grid, 32 * kFixedWarps, st, view<double>(p), src,

@@ -262,8 +262,8 @@ __device__ __forceinline__ Column column(const State& f, int k) {
 
 // The filter's sums of one row over the lanes of its group, kappa w^hyp on three fields.
 // hi, mid: this lane's sums; T: the three bounds; zero_ops: the operators (bits) that are zero
-// throughout the row; cold (the same in the whole group): the row needs FP64.  Every lane of the warp takes the same number of iterations (a lane
-// without a chunk adds zeros).
+// throughout the row; cold (the same in the whole group): the row needs FP64.  Every lane of
+// the warp takes the same number of iterations (a lane without a chunk adds zeros).
 template <int G, class F>
 __device__ __forceinline__ void filter_row(const PlanView<double>& P, const F& fld, int i, int e0, int e1, int gl,
                                            int zero_ops, long long (&hi)[3], long long (&mid)[3], int (&T)[3],
@@ -344,9 +344,11 @@ __device__ __forceinline__ void filter_row(const PlanView<double>& P, const F& f
 // The twelve derivative sums of one row over the lanes of its group, two lanes to a chunk:
 // the even one sums x, y, xx, xy, yy of u, the odd one of v, and each x and y of ln rho
 // over two of the chunk's four entries.  One lane for all twelve sums needed 128 registers
-// (16 warps an SM) and waited for its gathers.  hi, mid: [ln rho x, y, then five]; T:
-// bounds of ln rho and of the lane's own field.
-template <int G, class F>
+// (16 warps an SM) and waited for its gathers.  AHEAD: the next chunk's columns and gathers
+// are loaded before the current chunk's sums (16 more registers; a launch that fills the chip
+// gains nothing).  hi, mid: [ln rho x, y, then five]; T: bounds of ln rho and of the lane's
+// own field.
+template <int G, bool AHEAD, class F>
 __device__ __forceinline__ void rhs_row(const PlanView<double>& P, const F& fld, int i, int e0, int e1, int gl,
                                         int zero_ops, long long (&hi)[7], long long (&mid)[7], int (&T)[2],
                                         bool& cold) {
@@ -377,6 +379,10 @@ __device__ __forceinline__ void rhs_row(const PlanView<double>& P, const F& fld,
     };
     uint32_t cj[4];
     double g[6];
+    if (AHEAD) {
+        columns(e, cj);
+        values(cj, g);
+    }
 #pragma unroll 1
     for (int it = 0; it < trips; ++it, e += 2 * G) {
         const int64_t c = e < e1 ? e >> 2 : 0;
@@ -389,8 +395,10 @@ __device__ __forceinline__ void rhs_row(const PlanView<double>& P, const F& fld,
                 if (l + (gl & (NR - 1)) < 6)
                     asm volatile("prefetch.global.L2 [%0];" ::"l"(ahead + (l + (gl & (NR - 1))) * 128));
         }
-        columns(e, cj);
-        values(cj, g);
+        if (!AHEAD) {
+            columns(e, cj);
+            values(cj, g);
+        }
         double d[4], da[2];
         int t[4], ta[2], low = 0;
 #pragma unroll
@@ -406,6 +414,10 @@ __device__ __forceinline__ void rhs_row(const PlanView<double>& P, const F& fld,
             seen[0] |= not_zero(da[k]);
             ta[k] = T[0] - exponent20(da[k]) - int(((odd ? cj[k + 2] : cj[k]) & ~mask) >> 10);
             low |= ta[k];
+        }
+        if (AHEAD) {
+            columns(e + 2 * G, cj);
+            values(cj, g);
         }
         if (__any_sync(0xffffffffu, low < 0)) {
             const int T0 = T[0], T1 = T[1];
@@ -569,7 +581,7 @@ __device__ __noinline__ void cold_rows(const int32_t* row_ptr, const char* rec, 
 // lane l of a warp finishes one node of the warp's: the FP64 work after the sums (about 130
 // instructions, which cost the pipe the same for one lane as for 32) runs on as many lanes
 // as the warp has had nodes.
-template <int G, bool FILTER, class F, class Epi>
+template <int G, bool FILTER, bool AHEAD, class F, class Epi>
 __device__ __forceinline__ void fixed_nodes(const PlanView<double>& P, const F& fld, int passes, const Epi& epi) {
     constexpr int K = FILTER ? 3 : 12, R = 32 / G, LK = FILTER ? 3 : 7, LT = FILTER ? 3 : 2;
     __shared__ long long s_hi[kFixedWarps][K][32];
@@ -591,7 +603,7 @@ __device__ __forceinline__ void fixed_nodes(const PlanView<double>& P, const F& 
         int T[LT];
         bool cold;
         if constexpr (FILTER) filter_row<G>(P, fld, i, e0, e1, gl, zero_ops, hi, lo, T, cold);
-        else rhs_row<G>(P, fld, i, e0, e1, gl, zero_ops, hi, lo, T, cold);
+        else rhs_row<G, AHEAD>(P, fld, i, e0, e1, gl, zero_ops, hi, lo, T, cold);
         // over the lanes that share a sum: all of them (filter, ln rho), or every second one
 #pragma unroll
         for (int k = 0; k < LK; ++k) {

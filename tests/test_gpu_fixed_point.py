@@ -401,3 +401,47 @@ def test_the_largest_low_sums_do_not_overflow(lb, n, sign):
     q[0] = q[1]
     _check(lb, plan, rp, col, w, np.ones(N), q)
     plan.close()
+
+
+@pytest.mark.parametrize("side", [140, 250])
+@pytest.mark.parametrize("walls", [False, True])
+def test_same_bits_from_every_form_of_the_kernels(lb, side, walls):
+    # a small instance alone (one wave, gathering ahead) and beside one that makes the launch
+    # take the 96- and the 128-register form
+    if walls:
+        ns = li.channel(24, 20, m=6, jitter=0.1, seed=4)
+        cols, normals = li.channel_walls(ns)
+        dev = lambda a, t=torch.float64: torch.tensor(np.ascontiguousarray(a), dtype=t, device="cuda")  # noqa: E731
+        s = dev(ns.s)
+        a = lb.build_wall_operator(dev(ns.xy), dev(ns.h), s, ns.Lx, ns.Ly, 6, 4, dev(cols, torch.int32), dev(normals),
+                                   1.7, periodic=(True, False), check=True)
+        a["s"] = s
+    else:
+        ns, a = _lattice_operator(lb, 24, 21, 6, 5)
+    big, b = _lattice_operator(lb, side, side, 4, 6)
+    alone = lb.Plan.batched([a], dtype=torch.float64)
+    both = lb.Plan.batched([a, b], dtype=torch.float64)
+    rng = np.random.default_rng(side)
+    q = torch.tensor(0.1 * rng.standard_normal((3, ns.N)), device="cuda")
+    if walls:
+        wn = dev(cols[:, 0], torch.int32)
+        q[1:, wn.long()] = 0.0
+        for p in (alone, both):
+            p.set_walls(wn, dev(normals))
+    Q = torch.cat([q, torch.tensor(li.tgv_fields(big.xy, 10.0), device="cuda")], dim=1).contiguous()
+    ph, part = lb.Phys(100.0, 0.005), slice(0, ns.N)
+    assert torch.equal(lb.rhs(both, Q, ph)[:, part], lb.rhs(alone, q, ph))
+    assert torch.equal(lb.filter(both, Q)[:, part], lb.filter(alone, q))
+    # stage and recording launches; steps short enough for both instances
+    assert torch.equal(lb.rk_step(both, Q.clone(), 1e-5, 3, ph)[:, part], lb.rk_step(alone, q.clone(), 1e-5, 3, ph))
+    if not walls:
+        rec = []
+        for p, x in ((both, Q), (alone, q)):
+            lb.enable_adjoint(p)
+            x = x.clone()
+            X = lb.stage_states(p)
+            lb.rk_step_record(p, x, X, 1e-5, ph)
+            rec.append((x[:, part], lb.rhs_adjoint(p, x, x, ph)[:, part]))
+        assert all(torch.equal(x, y) for x, y in zip(*rec))
+    alone.close()
+    both.close()
