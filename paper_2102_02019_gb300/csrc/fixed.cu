@@ -99,11 +99,9 @@ __global__ void LABFM_FIXED_FILTER_BOUNDS k_fixed_filter_soa(PlanView<double> P,
 // ---------------------------------------------------------------- packing
 
 // s_j from how far (in log2, 2^20 units of the high words) the entry's largest weight lies
-// below the row's largest of the same operator: 3, 2, 1 or 0, so that weights falling as
-// r^-1.4 meet differences growing as r.
-__device__ __forceinline__ int entry_shift(int below) {
-    return below >= -748983 ? 3 : (below >= -2246949 ? 2 : (below >= -3744915 ? 1 : 0));
-}
+// below the row's largest of the same operator: 15 within a factor of two, one less for every
+// factor of two more.
+__device__ __forceinline__ int entry_shift(int below) { return max(min(kMostShift + 1 + (below >> 20), kMostShift), 0); }
 
 // Warp per row: the row's exponents, then its records (columns with s_j, weight words).
 __global__ void k_pack_fixed(int64_t N, int64_t nnz, int64_t off, const int32_t* __restrict__ row_ptr,
@@ -215,8 +213,8 @@ __global__ void k_pack_fixed(int64_t N, int64_t nnz, int64_t off, const int32_t*
                 for (int o = 0; o < 6; ++o)
                     word[o] = raw ? __double_as_longlong(v[o]) : weight_word(v[o], exps[o], int(o < 5 ? sr : sf));
             }
-            *reinterpret_cast<uint32_t*>(rb + Rec<double>::col_e(dst)) = c | (sr << 30);
-            *reinterpret_cast<uint32_t*>(fb + Rec<double>::fcol_e(dst)) = c | (sf << 30);
+            *reinterpret_cast<uint32_t*>(rb + Rec<double>::col_e(dst)) = c | (sr << 28);
+            *reinterpret_cast<uint32_t*>(fb + Rec<double>::fcol_e(dst)) = c | (sf << 28);
 #pragma unroll
             for (int o = 0; o < 6; ++o) *reinterpret_cast<long long*>((o < 5 ? rb : fb) + fixed_at(dst, o)) = word[o];
         }

@@ -18,34 +18,40 @@
 // digits with five instructions (weight_word): their 53 bits and the shift that aligns
 // them to E_w.  The FP64 fallback and the adjoint read them back exactly.
 //
-// The shift s_j (0 to 3, two bits of the column word) is the same for an entry's weights
-// and its difference and cancels: it moves the large weights near the node, where the
-// differences are small, down and those differences up, which gains two bits.
+// The shift s_j (0 to 15, four bits of the column word) is the same for an entry's weights
+// and its difference and cancels.  It is the entry's size: that of its largest weight, against
+// the row's largest of the same operator.  So the weights of all entries come to the same
+// scale, and a difference counts with the weight that it meets: a large one at the edge of the
+// stencil, where the weights are small, takes no bits from the others.
 //
 // The error of such a sum over n entries is at most (24 + n) 2^-56 2^(E_w + E_d): relative
 // to the bounds, where FP64's is relative to sum |w d|.  So the lanes add up the leading bits
 // of |w1| |d1| (four entries an instruction) as they go, and a row where that lower bound of
-// sum |w d| is below 1/8 of 2^(E_w + E_d) for any operator and field is summed in FP64
-// instead.  What is left is within (24 + n) 2^-53 sum |w d|, FP64's own a priori bound,
-// whatever the fields.  Against exact sums on jittered lattices of orders 4 to 10 (100 rows
-// each, every operator and field), in units of 2^-53 sum |w d|: smooth fields 0.03-0.05 on
-// average and 0.36 at most (FP64 0.24-0.32, 2.2), white noise 0.04-0.06 and 0.6 (0.36-0.44,
-// 2.5), and of the rows that pass in log-normal fields, fronts, pulses and impulses 0.04-0.37
-// and 1.7 (0.24-1.2, 5.9).  Smooth fields pass on all rows but one in a thousand, noise on
-// all but 3 % at order 4 and all from order 6 on; fronts and pulses on a fifth to two fifths,
-// the rest of which costs as much again as FP64 kernels would.  The sizes take the
-// right-hand side of 262,144 nodes of order 8 from 403 to 434 us (490 as a high product of
-// every entry).
+// sum |w d| is below 1/16 of 2^(E_w + E_d) for any operator and field is summed in FP64
+// instead.  What is left is within (24 + n) 2^-52 sum |w d| whatever the fields; FP64's own a
+// priori bound is n 2^-53 sum |w d|.  Against exact sums on jittered lattices of orders 4 to
+// 10 (100 rows each, every operator and field), in units of 2^-53 sum |w d|: smooth fields
+// 0.04-0.07 on average and 0.65 at most (FP64 0.24-0.32, 2.2), white noise 0.07-0.12 and 0.9
+// (0.36-0.44, 2.5), pulses and fronts of a spacing's width 0.05-0.12 and 2.6 (0.28-0.45, 4.7),
+// single-node impulses 0.04-0.09 and 0.9 (0.38-0.43, 1.9), log-normal values of sigma 2 and 5
+// 0.13-0.53 and 4.7 (0.43-0.99, 6.6).  Smooth fields and noise pass on all rows, pulses on
+// nine tenths and more, fronts on half.  With shifts of 0 to 3 and 1/8, pulses had passed on a
+// fifth, and the Lamb-Oseen vortex, whose tails they are, on a fifth of its rows.  One
+// exception: differences that are tiny against the node's own value (rounding noise on a
+// uniform stream) are exact in the high digit, so that only the weights' rounding is left,
+// 2^-57 of the entry's size each, and such rows stay in fixed point.  A row that fails costs
+// as much again as FP64 kernels would.  The sizes take the right-hand side of 262,144 nodes of
+// order 8 from 403 to 434 us (490 as a high product of every entry).
 //
 // No overflow: E_w is raised until sum_j |w_ji| 2^-s_j <= 32 2^E_w, so |sum w1 d1| <=
 // 2^(5 + 28 + 29) over a whole row; |sum (w1 d0 + w0 d1)| <= 2^60 + n 2^57 over n entries,
 // whose carries a lane moves up after every 32.  Rows with a weight that is not finite,
 // beyond 2^+-400 at their largest, subnormal or below 2^-500 of their row's largest hold
 // plain FP64 weights and are summed in FP64 (kRawRow), each by itself, so that a failed node
-// changes no other row.  A row whose differences are not finite or beyond 2^477 is summed in
+// changes no other row.  A row whose differences are not finite or beyond 2^460 is summed in
 // FP64 too, so that infinities and NaN come out as they would, and one whose differences of
-// a field all lie below 2^-499 without being all zero.  Beside larger ones, differences below
-// 2^-1022 count as zero.  Plans of 2^30 nodes or more need the two bits for their columns:
+// a field, with their shifts, all lie below 2^-498 without being all zero.  Beside larger ones, differences below
+// 2^-1022 count as zero.  Plans of 2^28 nodes or more need the four bits for their columns:
 // there every s_j is 0.
 #pragma once
 
@@ -54,14 +60,15 @@
 namespace labfm {
 namespace {
 
-// The column word: the column, and s_j in the bits above it.
-__host__ __device__ __forceinline__ uint32_t col_mask(int64_t N) { return N < (int64_t(1) << 30) ? 0x3fffffffu : 0x7fffffffu; }
+// The column word: the column, and s_j in the four bits above it.
+__host__ __device__ __forceinline__ uint32_t col_mask(int64_t N) { return N < (int64_t(1) << 28) ? 0x0fffffffu : 0x7fffffffu; }
+constexpr int kMostShift = 15;
 constexpr int kRawRow = 64;  // with the zero operators' bits in wexp[8 i + 6]: the row holds FP64 weights
 constexpr int kFixedWarps = 2;  // warps a block
-constexpr int kFloorT = 65 << 20;           // T of a field until a difference above it turns up
+constexpr int kFloorT = 80 << 20;           // T of a field until a difference above it turns up
 constexpr int kLeastT = 524 << 20;          // smallest bound of the fixed-point sums
 constexpr uint32_t kMostT = 1500u << 20;
-constexpr uint32_t kLeastSize = 64;         // 1/8 of the bounds' product, in units of 2^-9 of it
+constexpr uint32_t kLeastSize = 32;         // 1/16 of the bounds' product, in units of 2^-9 of it
 
 __device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
 
@@ -168,11 +175,16 @@ __device__ __forceinline__ uint32_t not_zero(double d) {
 
 // Whether a row needs FP64 for the sums of a field with bound T over K operators, the first
 // of them `first`: its differences lie below the range of the fixed-point sums without being
-// all zero, or span too many bits for an operator that is not zero throughout the row.
+// all zero, or span too many bits for an operator that is not zero throughout the row.  Not
+// where they are below 2^-24 of the node's value (shifts included): then they are whole
+// multiples of the high digit's last bit.
 template <int K>
-__device__ __forceinline__ bool out_of_range(int T, uint32_t seen, const uint32_t* size, int first, int zero_ops) {
+__device__ __forceinline__ bool out_of_range(int T, uint32_t seen, double own, const uint32_t* size, int first,
+                                             int zero_ops) {
     if (T == kFloorT) return seen != 0;
-    bool out = T < kLeastT;
+    if (T < kLeastT) return true;
+    if (T + (25 << 20) <= exponent20(own)) return false;
+    bool out = false;
 #pragma unroll
     for (int k = 0; k < K; ++k) out |= size[k] < kLeastSize && !(zero_ops >> (first + k) & 1);
     return out;
@@ -296,7 +308,7 @@ __device__ __forceinline__ void filter_row(const PlanView<double>& P, const F& f
             const uint32_t cw = on ? cj[k] : uint32_t(i);
             double v[3];
             fld.get(int(cw & mask), v[0], v[1], v[2]);
-            s20[k] = int((cw & ~mask) >> 10);
+            s20[k] = int((cw & ~mask) >> 8);
 #pragma unroll
             for (int f = 0; f < 3; ++f) {
                 d[f][k] = v[f] - own[f];
@@ -336,7 +348,7 @@ __device__ __forceinline__ void filter_row(const PlanView<double>& P, const F& f
 #pragma unroll
     for (int f = 0; f < 3; ++f) {
         const uint32_t all = group_add<1, G>(size[f]);
-        cold |= out_of_range<1>(T[f], seen[f], &all, 5, zero_ops);
+        cold |= out_of_range<1>(T[f], seen[f], own[f], &all, 5, zero_ops);
     }
     cold = group_max<1, G>(uint32_t(cold)) != 0;
 }
@@ -405,14 +417,14 @@ __device__ __forceinline__ void rhs_row(const PlanView<double>& P, const F& fld,
         for (int k = 0; k < 4; ++k) {
             d[k] = g[k] - of;
             seen[1] |= not_zero(d[k]);
-            t[k] = T[1] - exponent20(d[k]) - int((cj[k] & ~mask) >> 10);
+            t[k] = T[1] - exponent20(d[k]) - int((cj[k] & ~mask) >> 8);
             low |= t[k];
         }
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             da[k] = g[4 + k] - oa;
             seen[0] |= not_zero(da[k]);
-            ta[k] = T[0] - exponent20(da[k]) - int(((odd ? cj[k + 2] : cj[k]) & ~mask) >> 10);
+            ta[k] = T[0] - exponent20(da[k]) - int(((odd ? cj[k + 2] : cj[k]) & ~mask) >> 8);
             low |= ta[k];
         }
         if (AHEAD) {
@@ -490,8 +502,8 @@ __device__ __forceinline__ void rhs_row(const PlanView<double>& P, const F& fld,
     fold(hi, mid);
 #pragma unroll
     for (int k = 0; k < 7; ++k) size[k] = k < 2 ? group_add<1, G>(size[k]) : group_add<2, G>(size[k]);
-    cold |= out_of_range<2>(T[0], seen[0], size, 0, zero_ops);
-    cold |= out_of_range<5>(T[1], seen[1], size + 2, 0, zero_ops);
+    cold |= out_of_range<2>(T[0], seen[0], oa, size, 0, zero_ops);
+    cold |= out_of_range<5>(T[1], seen[1], of, size + 2, 0, zero_ops);
     cold = group_max<1, G>(uint32_t(cold)) != 0;
 }
 
@@ -516,62 +528,95 @@ __device__ __forceinline__ double fixed_weight(const PlanView<double>& P, int i,
     const char* rec = o == 5 ? reinterpret_cast<const char*>(P.wf) : reinterpret_cast<const char*>(P.w);
     const long long word = *reinterpret_cast<const long long*>(rec + fixed_at(e, o));
     if (P.wexp[int64_t(i) * 8 + 6] & kRawRow) return __longlong_as_double(word);
-    return word_weight(word, P.wexp[int64_t(i) * 8 + o], int((fixed_col_word(P, e, o == 5) & ~col_mask(P.N)) >> 30));
+    return word_weight(word, P.wexp[int64_t(i) * 8 + o], int((fixed_col_word(P, e, o == 5) & ~col_mask(P.N)) >> 28));
 }
 
-// The rows that need FP64, by as many lanes as the fixed-point sums: in the order of the
-// FP64 kernels (a lane takes every G-th chunk, then the lanes' sums), 32 / G rows of the warp
-// at a time.  slots: the rows, as bits (fixed_nodes); out[k][slot]: the sums' bit patterns.
-template <int G, bool FILTER, int K, class F>
+// The rows that need FP64, by 8 lanes each, four at a time (whatever the lanes of the
+// fixed-point sums and however many rows of the warp need it: a row's sums are the same
+// beside any others).  slots: the rows, as bits (fixed_nodes, R of them a pass);
+// out[k][slot]: the sums' bit patterns.  Such rows come in clusters (all 16 of a warp, beside
+// a boundary), and a warp's chain through them is what the launch waits for: the next entry's
+// column, values and words are in flight while the current one's products are summed (the
+// Lamb-Oseen step of 40,000 nodes, 2.5 % of whose rows come here: 392 us, an entry at a time
+// 421, a chunk of four 423, without these rows 285; with 16 and 32 lanes a row, whose sums take
+// more of the FP64 pipe, 12 and 48 % more).
+template <bool FILTER, int R, int K, class F>
 __device__ __noinline__ void cold_rows(const int32_t* row_ptr, const char* rec, const int16_t* wexp, F fld,
                                        uint32_t mask, int64_t first, uint32_t slots, long long (*out)[32]) {
-    constexpr int KA = FILTER ? 1 : 2, KV = FILTER ? 1 : 5, R = 32 / G;
-    const int lane = threadIdx.x & 31, gl = lane % G;
+    constexpr int KA = FILTER ? 1 : 2, KV = FILTER ? 1 : 5, L = 8;
+    const int lane = threadIdx.x & 31, gl = lane % L;
+    auto column = [&](int e) {
+        return *reinterpret_cast<const uint32_t*>(rec + (FILTER ? Rec<double>::fcol_e(e) : Rec<double>::col_e(e)));
+    };
+#pragma unroll 1
     while (slots) {
         uint32_t left = slots;
-        for (int k = 0; k < lane / G; ++k) left &= left - 1;
+#pragma unroll 1
+        for (int k = 0; k < lane / L; ++k) left &= left - 1;
         const int slot = __ffs(left) - 1;  // this group's row, or -1
+        const int i = slot < 0 ? 0 : int(first + (slot / R) * (kFixedWarps * R) + slot % R);
         double sum[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) sum[k] = 0.0;
-        if (slot >= 0) {
-            const int i = int(first + (slot / R) * (kFixedWarps * R) + slot % R);
-            double ai, ui, vi;
-            fld.get(i, ai, ui, vi);
-            const int4 ev = *reinterpret_cast<const int4*>(wexp + int64_t(i) * 8);
-            const int E[6] = {int16_t(ev.x), ev.x >> 16, int16_t(ev.y), ev.y >> 16, int16_t(ev.z), ev.z >> 16};
-            const bool raw = ev.w & kRawRow;
-            const int e1 = row_ptr[i + 1];
-#pragma unroll 1
-            for (int e = row_ptr[i] + 4 * gl; e < e1; e += 4 * G) {
-#pragma unroll 1
-                for (int k = 0; k < 4; ++k) {
-                    const uint32_t cw = *reinterpret_cast<const uint32_t*>(
-                        rec + (FILTER ? Rec<double>::fcol_e(e + k) : Rec<double>::col_e(e + k)));
-                    const int s = int((cw & ~mask) >> 30);
-                    double a, u, v;
-                    fld.get(int(cw & mask), a, u, v);
-                    a -= ai;
-                    u -= ui;
-                    v -= vi;
+        double ai, ui, vi;
+        fld.get(i, ai, ui, vi);
+        const int4 ev = *reinterpret_cast<const int4*>(wexp + int64_t(i) * 8);
+        const int E[6] = {int16_t(ev.x), ev.x >> 16, int16_t(ev.y), ev.y >> 16, int16_t(ev.z), ev.z >> 16};
+        const bool raw = ev.w & kRawRow;
+        int e = row_ptr[i] + gl;
+        const int e1 = slot < 0 ? 0 : row_ptr[i + 1];
+        // the next entry's column, values and words are loaded before this one's products
+        uint32_t cw = 0, cn = 0;
+        double a = ai, u = ui, v = vi;
+        long long word[KV], more[KV];
+        auto words = [&](int q, long long (&to)[KV]) {
 #pragma unroll
-                    for (int o = 0; o < KV; ++o) {
-                        const int op = FILTER ? 5 : o;
-                        const long long word = *reinterpret_cast<const long long*>(rec + fixed_at(e + k, op));
-                        const double w = raw ? __longlong_as_double(word) : word_weight(word, E[op], s);
-                        if (o < KA) sum[o] = fma(a, w, sum[o]);
-                        sum[KA + o] = fma(u, w, sum[KA + o]);
-                        sum[KA + KV + o] = fma(v, w, sum[KA + KV + o]);
-                    }
-                }
+            for (int o = 0; o < KV; ++o) to[o] = *reinterpret_cast<const long long*>(rec + fixed_at(q, FILTER ? 5 : o));
+        };
+        if (e < e1) {
+            cw = column(e);
+            words(e, word);
+            if (e + L < e1) cn = column(e + L);
+            fld.get(int(cw & mask), a, u, v);
+        }
+#pragma unroll 1
+        for (; e < e1; e += L) {
+            double an = ai, un = ui, vn = vi;
+            uint32_t cm = 0;
+            if (e + L < e1) {
+                words(e + L, more);
+                fld.get(int(cn & mask), an, un, vn);
+                if (e + 2 * L < e1) cm = column(e + 2 * L);
             }
-        }
+            const int s = int((cw & ~mask) >> 28);
+            a -= ai;
+            u -= ui;
+            v -= vi;
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            sum[k] = group_sum<G>(sum[k]);
-            if (slot >= 0 && gl == 0) out[k][slot] = __double_as_longlong(sum[k]);
+            for (int o = 0; o < KV; ++o) {
+                const double w = raw ? __longlong_as_double(word[o]) : word_weight(word[o], E[FILTER ? 5 : o], s);
+                if (o < KA) sum[o] = fma(a, w, sum[o]);
+                sum[KA + o] = fma(u, w, sum[KA + o]);
+                sum[KA + KV + o] = fma(v, w, sum[KA + KV + o]);
+                word[o] = more[o];
+            }
+            cw = cn;
+            cn = cm;
+            a = an;
+            u = un;
+            v = vn;
         }
-        for (int k = 0; k < R; ++k) slots &= slots - 1;
+#pragma unroll 1
+        for (int off = L / 2; off > 0; off >>= 1) {
+#pragma unroll
+            for (int k = 0; k < K; ++k) sum[k] += __shfl_xor_sync(0xffffffffu, sum[k], off);
+        }
+        if (slot >= 0 && gl == 0) {
+#pragma unroll
+            for (int k = 0; k < K; ++k) out[k][slot] = __double_as_longlong(sum[k]);
+        }
+#pragma unroll 1
+        for (int k = 0; k < 32 / L; ++k) slots &= slots - 1;
     }
     __syncwarp();
 }
@@ -638,7 +683,7 @@ __device__ __forceinline__ void fixed_nodes(const PlanView<double>& P, const F& 
     }
     __syncwarp();
     if (cold_slots)
-        cold_rows<G, FILTER, K>(P.row_ptr, reinterpret_cast<const char*>(FILTER ? P.wf : P.w), P.wexp, fld, col_mask(P.N),
+        cold_rows<FILTER, R, K>(P.row_ptr, reinterpret_cast<const char*>(FILTER ? P.wf : P.w), P.wexp, fld, col_mask(P.N),
                                 first, cold_slots, s_hi[warp]);
     const int64_t node = first + (lane / R) * (kFixedWarps * R) + lane % R;
     const bool mine = lane < passes * R && node < P.n_hi;
