@@ -143,11 +143,7 @@ __global__ void __launch_bounds__(32)
         qu = ui;
         qv = vi;
     }
-    qa = fma(cb, Ra, qa);
-    qu = fma(cb, Ru, qu);
-    qv = fma(cb, Rv, qv);
-    store(Q_out, i, qa, qu, qv);
-    if (X_out) store(X_out, i, fma(cx, Ra, qa), fma(cx, Ru, qu), fma(cx, Rv, qv));
+    stage_store(i, cb, cx, Ra, Ru, Rv, qa, qu, qv, Q_out, X_out);
     if (REC) {
         float c[8];
         own_coeffs<float, true>(d, is, c);
@@ -261,13 +257,6 @@ cudaError_t filter_u(const labfm_plan* p, const PlanView<float>& v, const Packed
         default: return set_error(LABFM_EINVAL, "unsupported group size");          \
     }
 
-PlanView<float> view_of(const labfm_plan* p, int64_t n_lo, int64_t n_hi) {
-    PlanView<float> v = view<float>(p);
-    v.n_lo = n_lo;
-    v.n_hi = n_hi;
-    return v;
-}
-
 }  // namespace
 
 // Up to 56 warps an SM, 68,000 nodes at 4 lanes: there one chunk ahead takes 126.4 us a step
@@ -280,7 +269,7 @@ int ahead_stage(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, cons
                 cudaStream_t st) {
     if (n_hi <= n_lo) return LABFM_OK;
     const Phys<float> ph{float(php.c2), float(php.mu), float(php.gx), float(php.gy)};
-    const PlanView<float> v = view_of(p, n_lo, n_hi);
+    const PlanView<float> v = view<float>(p, n_lo, n_hi);
     const int u = chunks_ahead(n_hi - n_lo, group);
     cudaError_t e = cudaErrorInvalidValue;
     LABFM_AHEAD_DISPATCH((stage_u<G, U>(p, v, static_cast<const Packed<float>*>(xin), static_cast<const Packed<float>*>(qin),
@@ -293,7 +282,7 @@ int ahead_stage(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, cons
 int ahead_filter(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, const void* in, void* out, void* soa,
                  cudaStream_t st) {
     if (n_hi <= n_lo) return LABFM_OK;
-    const PlanView<float> v = view_of(p, n_lo, n_hi);
+    const PlanView<float> v = view<float>(p, n_lo, n_hi);
     const int u = chunks_ahead(n_hi - n_lo, group);
     cudaError_t e = cudaErrorInvalidValue;
     LABFM_AHEAD_DISPATCH((filter_u<G, U>(p, v, static_cast<const Packed<float>*>(in), static_cast<Packed<float>*>(out),

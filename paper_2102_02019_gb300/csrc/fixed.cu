@@ -289,13 +289,6 @@ int warps_for(int grid) {
 
 Phys<double> phys_of(const labfm_phys& ph) { return Phys<double>{ph.c2, ph.mu, ph.gx, ph.gy}; }
 
-PlanView<double> view_of(const labfm_plan* p, int64_t n_lo, int64_t n_hi) {
-    PlanView<double> v = view<double>(p);
-    v.n_lo = n_lo;
-    v.n_hi = n_hi;
-    return v;
-}
-
 }  // namespace
 
 int fixed_rhs(const labfm_plan* p, const void* fields, void* rhs, const labfm_phys& php, int group, cudaStream_t st) {
@@ -323,7 +316,7 @@ int fixed_stage(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, cons
     if (n_hi <= n_lo) return LABFM_OK;
     const int g = lanes_for(group), passes = passes_for(n_hi - n_lo, g, kRhsPasses);
     const int grid = grid_of(n_hi - n_lo, g, passes);
-    const PlanView<double> v = view_of(p, n_lo, n_hi);
+    const PlanView<double> v = view<double>(p, n_lo, n_hi);
     auto launch = [&](auto* kernel) {
         return launch_pdl(p, kernel, grid, 32 * kFixedWarps, st, v, static_cast<const Packed<double>*>(xin),
                           static_cast<const Packed<double>*>(qin), static_cast<Packed<double>*>(qout),
@@ -357,7 +350,7 @@ int fixed_filter(const labfm_plan* p, int64_t n_lo, int64_t n_hi, int group, con
     if (n_hi <= n_lo) return LABFM_OK;
     const int g = filter_lanes_for(group), passes = passes_for(n_hi - n_lo, g, kFilterPasses);
     const int grid = grid_of(n_hi - n_lo, g, passes);
-    const PlanView<double> v = view_of(p, n_lo, n_hi);
+    const PlanView<double> v = view<double>(p, n_lo, n_hi);
     cudaError_t e = cudaSuccess;
     LABFM_FIXED_DISPATCH(g, (e = launch_pdl(p, k_fixed_filter<G>, grid, 32 * kFixedWarps, st, v, static_cast<const Packed<double>*>(in),
                                             static_cast<Packed<double>*>(out), static_cast<double*>(soa), passes)));

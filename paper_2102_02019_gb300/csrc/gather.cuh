@@ -404,6 +404,15 @@ PlanView<T> view(const labfm_plan* p) {
                        T(p->nscbc.mach), T(p->nscbc.rho0), p->wexp};
 }
 
+// The same over nodes [n_lo, n_hi).
+template <typename T>
+PlanView<T> view(const labfm_plan* p, int64_t n_lo, int64_t n_hi) {
+    PlanView<T> v = view<T>(p);
+    v.n_lo = n_lo;
+    v.n_hi = n_hi;
+    return v;
+}
+
 // Chunk loaders for the gathers: from the plan's record stream in global memory,
 // or from a copy of a contiguous range of its blocks in shared memory.
 // Shortest row (padded entries) whose record stream the stage and filter kernels
@@ -868,6 +877,17 @@ __device__ __forceinline__ void node_rhs(const PlanView<T>& P, int i, const T (&
     pointwise_rhs<T, SCALED>(d, a, u, v, inv_s, ph.c2, ph.mu, ph.gx, ph.gy, Ra, Ru, Rv);
 }
 
+// Q_out = q + cb R; X_out = Q_out + cx R (skipped when X_out is null).
+template <typename T>
+__device__ __forceinline__ void stage_store(int i, T cb, T cx, T Ra, T Ru, T Rv, T qa, T qu, T qv, Packed<T>* Q_out,
+                                            Packed<T>* X_out) {
+    qa = fma(cb, Ra, qa);
+    qu = fma(cb, Ru, qu);
+    qv = fma(cb, Rv, qv);
+    store(Q_out, i, qa, qu, qv);
+    if (X_out) store(X_out, i, fma(cx, Ra, qa), fma(cx, Ru, qu), fma(cx, Rv, qv));
+}
+
 // The RK stage update at node i from its 12 derivatives: F = R(X_in);
 // Q_out = Q_in + dt_i b_k F; X_out = Q_out + dt_i (a - b) F (skipped when X_out
 // is null).  Q_in may equal Q_out, and Q_in may equal X_in (first stage, where
@@ -893,11 +913,7 @@ __device__ __forceinline__ void stage_epilogue(const PlanView<T>& P, int i, int 
         } else {
             unpack_rw(Q_in, i, qa, qu, qv);
         }
-        qa = fma(cb, Ra, qa);
-        qu = fma(cb, Ru, qu);
-        qv = fma(cb, Rv, qv);
-        store(Q_out, i, qa, qu, qv);
-        if (X_out) store(X_out, i, fma(cx, Ra, qa), fma(cx, Ru, qu), fma(cx, Rv, qv));
+        stage_store(i, cb, cx, Ra, Ru, Rv, qa, qu, qv, Q_out, X_out);
     }
 }
 

@@ -47,3 +47,56 @@ def test_same_bits_as_chunk_by_chunk(lb, nx, ny, m):
         assert torch.isfinite(out[0]).all()
         assert torch.equal(out[0], out[1]), group
     plan.close()
+
+
+def _lattice(lb, nx, ny, m, seed):
+    ns = li.tgv_lattice(nx, ny, m=m, jitter=0.1, seed=seed)
+    xy, h, s = (torch.tensor(a, device="cuda") for a in (ns.xy, ns.h, ns.s))
+    rp, col = lb.build_stencils(xy, h, ns.Lx, ns.Ly)
+    wb = lb.build_weights(xy, h, s, ns.Lx, ns.Ly, rp, col, m, residual=False)
+    return ns, {"row_ptr": rp, "col": col, "w": wb["w"], "kappa": wb["kappa"], "s": s}
+
+
+@pytest.mark.parametrize("walls", [False, True])
+@pytest.mark.parametrize("side", [15, 60])
+def test_recording_and_walls_same_bits_as_past_the_line(lb, walls, side):
+    # an instance alone (chunks ahead) and beside a lattice of 70,200 nodes, with which the
+    # launches read chunk by chunk: steps with and without walls, and recorded steps with the
+    # reverse sweep over what they recorded
+    if walls:
+        ns = li.channel(side + 5, side, m=6, jitter=0.1, seed=4)
+        cols, normals = li.channel_walls(ns)
+        dev = lambda a, t=torch.float64: torch.tensor(a.copy(), dtype=t, device="cuda")  # noqa: E731
+        s = dev(ns.s)
+        a = lb.build_wall_operator(dev(ns.xy), dev(ns.h), s, ns.Lx, ns.Ly, 6, 4, dev(cols, torch.int32), dev(normals),
+                                   1.7, periodic=(True, False), check=True)
+        a["s"] = s
+    else:
+        ns, a = _lattice(lb, side, side + 3, 6, 5)
+    big, b = _lattice(lb, 270, 260, 4, 6)
+    alone = lb.Plan.batched([a], dtype=torch.float32)
+    both = lb.Plan.batched([a, b], dtype=torch.float32)
+    g = torch.Generator().manual_seed(side)
+    q = (0.1 * torch.randn((3, ns.N), generator=g)).cuda()
+    if walls:
+        wn = dev(cols[:, 0], torch.int32)
+        q[1:, wn.long()] = 0.0
+        for p in (alone, both):
+            p.set_walls(wn, dev(normals))
+    Q = torch.cat([q, torch.tensor(li.tgv_fields(big.xy, C), dtype=torch.float32, device="cuda")], dim=1).contiguous()
+    ph, dt = lb.Phys(C * C, MU), 1e-5
+    assert torch.equal(lb.rk_step(both, Q.clone(), dt, 3, ph)[:, :ns.N], lb.rk_step(alone, q.clone(), dt, 3, ph))
+    if not walls:
+        out = []
+        for p, x in ((both, Q), (alone, q)):
+            lb.enable_adjoint(p)
+            z = x.clone()
+            X = lb.stage_states(p)
+            lb.rk_step_record(p, z, X, dt, ph)
+            lam = x.clone()
+            lb.rk_step_adjoint_recorded(p, X, lam, dt, ph)
+            out.append((z[:, :ns.N], lam[:, :ns.N]))
+        assert torch.isfinite(out[0][1]).all()
+        assert all(torch.equal(x, y) for x, y in zip(*out))
+    alone.close()
+    both.close()
