@@ -446,7 +446,7 @@ __device__ __forceinline__ void rank_row(const int32_t* src, int n, int lane, in
 // (256 keys in about 500 instructions, against 1,550 for ranking 152).  Bound by
 // instruction issue.  1.0M nodes of varying h at order 10 (152 entries): the whole search
 // 44.1 -> 2.46 ms, against a thread per node testing every candidate in FP64, twice for
-// the count and once to fill, and a ranking sort; half of it is the sort.  40 registers
+// the count and once to fill, and a ranking sort; half of it is the sort.  48 registers
 // (10 blocks an SM; with 92 the fill alone took 2.7 ms), and a grid of 16 blocks for each
 // that is resident (4: 2.68 ms, one node a warp: 2.72).
 template <int MODE>
