@@ -363,6 +363,10 @@ int labfm_modal_response(const double* xy, const double* s, int64_t N, double Lx
  * with the filter weights kappa_i w^hyp_ji.  For LABFM_F32 the RHS weights are stored nondimensionalised,
  * w^d_ji s_i^l (l = 1 for d/dx, d/dy; 2 for second derivatives), and the kernels
  * multiply the sums by s_i^-l.
+ * For LABFM_F64 they are held bit for bit.  The sums of a row's n terms w d, d the
+ * FP64 differences of a field, run in fixed point and are within (24 + n) 2^-52
+ * sum |w d| of the exact ones; a row where that does not hold, or whose weights or
+ * differences are not finite or out of range, is summed in FP64 arithmetic.
  *
  *   w      device, 6 x nnz doubles as written by labfm_build_weights (col and w
  *          may be NULL when nnz = 0; such a plan's steps leave the state unchanged)

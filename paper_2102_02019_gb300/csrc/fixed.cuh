@@ -29,19 +29,19 @@
 // of |w1| |d1| (four entries an instruction) as they go, and a row where that lower bound of
 // sum |w d| is below 1/16 of 2^(E_w + E_d) for any operator and field is summed in FP64
 // instead.  What is left is within (24 + n) 2^-52 sum |w d| whatever the fields; FP64's own a
-// priori bound is n 2^-53 sum |w d|.  Against exact sums on jittered lattices of orders 4 to
-// 10 (100 rows each, every operator and field), in units of 2^-53 sum |w d|: smooth fields
-// 0.04-0.07 on average and 0.65 at most (FP64 0.24-0.32, 2.2), white noise 0.07-0.12 and 0.9
-// (0.36-0.44, 2.5), pulses and fronts of a spacing's width 0.05-0.12 and 2.6 (0.28-0.45, 4.7),
-// single-node impulses 0.04-0.09 and 0.9 (0.38-0.43, 1.9), log-normal values of sigma 2 and 5
-// 0.13-0.53 and 4.7 (0.43-0.99, 6.6).  Smooth fields and noise pass on all rows, pulses on
-// nine tenths and more, fronts on half.  With shifts of 0 to 3 and 1/8, pulses had passed on a
-// fifth, and the Lamb-Oseen vortex, whose tails they are, on a fifth of its rows.  One
-// exception: differences that are tiny against the node's own value (rounding noise on a
-// uniform stream) are exact in the high digit, so that only the weights' rounding is left,
-// 2^-57 of the entry's size each, and such rows stay in fixed point.  A row that fails costs
-// as much again as FP64 kernels would.  The sizes take the right-hand side of 262,144 nodes of
-// order 8 from 403 to 434 us (490 as a high product of every entry).
+// priori bound is n 2^-53 sum |w d|.  Against exact sums, in units of 2^-53 sum |w d|, over
+// 3,840 nodes of orders 4, 6, 8 and 10, the operators x, y and xy, FP64 kernels in brackets:
+// smooth fields 0.05-0.19 on average and 1.2 at most (0.21-0.40, 2.1), white noise 0.12-0.25
+// and 2.3 (0.35-0.47, 3.5), pulses of 4 and 8 spacings 0.05-0.19 and 1.5 (0.20-0.42, 3.0),
+// fronts, impulses, log-normal values of sigma 2 and 5, small pulses and rounding noise on a
+// uniform stream 0.05-0.73 and 6.9 (0.10-0.99, 7.0).  In no class was the mean above FP64's by
+// more than 1.4 %, nor the largest by more than a quarter.  Smooth fields and noise pass on all
+// rows, pulses on nine tenths and more, fronts on half.  With shifts of 0 to 3 and 1/8, pulses
+// had passed on a fifth, and the Lamb-Oseen vortex, whose tails they are, on a fifth of its
+// rows.  A row that fails costs as much again as FP64 kernels would.  Keeping rows whose
+// differences are exact in the high digit (rounding noise) in fixed point gave errors of up to
+// 10^5.  The sizes take the right-hand side of 262,144 nodes of order 8 from 403 to 434 us (490
+// as a high product of every entry).
 //
 // No overflow: E_w is raised until sum_j |w_ji| 2^-s_j <= 32 2^E_w, so |sum w1 d1| <=
 // 2^(5 + 28 + 29) over a whole row; |sum (w1 d0 + w0 d1)| <= 2^60 + n 2^57 over n entries,
@@ -175,16 +175,11 @@ __device__ __forceinline__ uint32_t not_zero(double d) {
 
 // Whether a row needs FP64 for the sums of a field with bound T over K operators, the first
 // of them `first`: its differences lie below the range of the fixed-point sums without being
-// all zero, or span too many bits for an operator that is not zero throughout the row.  Not
-// where they are below 2^-24 of the node's value (shifts included): then they are whole
-// multiples of the high digit's last bit.
+// all zero, or span too many bits for an operator that is not zero throughout the row.
 template <int K>
-__device__ __forceinline__ bool out_of_range(int T, uint32_t seen, double own, const uint32_t* size, int first,
-                                             int zero_ops) {
+__device__ __forceinline__ bool out_of_range(int T, uint32_t seen, const uint32_t* size, int first, int zero_ops) {
     if (T == kFloorT) return seen != 0;
-    if (T < kLeastT) return true;
-    if (T + (25 << 20) <= exponent20(own)) return false;
-    bool out = false;
+    bool out = T < kLeastT;
 #pragma unroll
     for (int k = 0; k < K; ++k) out |= size[k] < kLeastSize && !(zero_ops >> (first + k) & 1);
     return out;
@@ -348,7 +343,7 @@ __device__ __forceinline__ void filter_row(const PlanView<double>& P, const F& f
 #pragma unroll
     for (int f = 0; f < 3; ++f) {
         const uint32_t all = group_add<1, G>(size[f]);
-        cold |= out_of_range<1>(T[f], seen[f], own[f], &all, 5, zero_ops);
+        cold |= out_of_range<1>(T[f], seen[f], &all, 5, zero_ops);
     }
     cold = group_max<1, G>(uint32_t(cold)) != 0;
 }
@@ -502,8 +497,8 @@ __device__ __forceinline__ void rhs_row(const PlanView<double>& P, const F& fld,
     fold(hi, mid);
 #pragma unroll
     for (int k = 0; k < 7; ++k) size[k] = k < 2 ? group_add<1, G>(size[k]) : group_add<2, G>(size[k]);
-    cold |= out_of_range<2>(T[0], seen[0], oa, size, 0, zero_ops);
-    cold |= out_of_range<5>(T[1], seen[1], of, size + 2, 0, zero_ops);
+    cold |= out_of_range<2>(T[0], seen[0], size, 0, zero_ops);
+    cold |= out_of_range<5>(T[1], seen[1], size + 2, 0, zero_ops);
     cold = group_max<1, G>(uint32_t(cold)) != 0;
 }
 
@@ -537,9 +532,9 @@ __device__ __forceinline__ double fixed_weight(const PlanView<double>& P, int i,
 // out[k][slot]: the sums' bit patterns.  Such rows come in clusters (all 16 of a warp, beside
 // a boundary), and a warp's chain through them is what the launch waits for: the next entry's
 // column, values and words are in flight while the current one's products are summed (the
-// Lamb-Oseen step of 40,000 nodes, 2.5 % of whose rows come here: 392 us, an entry at a time
-// 421, a chunk of four 423, without these rows 285; with 16 and 32 lanes a row, whose sums take
-// more of the FP64 pipe, 12 and 48 % more).
+// Lamb-Oseen step of 40,000 nodes, 5 % of whose rows come here, 409 us, without these rows 285;
+// at 2.5 % an entry at a time 421, a chunk of four 423, so 392; with 16 and 32 lanes a row,
+// whose sums take more of the FP64 pipe, 12 and 48 % more).
 template <bool FILTER, int R, int K, class F>
 __device__ __noinline__ void cold_rows(const int32_t* row_ptr, const char* rec, const int16_t* wexp, F fld,
                                        uint32_t mask, int64_t first, uint32_t slots, long long (*out)[32]) {

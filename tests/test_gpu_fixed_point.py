@@ -237,13 +237,18 @@ def _wide_field(kind, ns, rng):
         return np.stack([np.exp(-((x - 0.5) ** 2 + (y - 0.5) ** 2) / (2 * (k * s) ** 2)) for k in (2, 5, 10)])
     if kind == "impulses":
         return (rng.random((3, ns.N)) < 1 / 60) * rng.standard_normal((3, ns.N))
+    if kind == "steep":  # saturates: differences of a rounding beside those of the front
+        return np.stack([np.tanh((x - 0.5) / (k * s)) for k in (0.1, 0.3, 0.6)])
+    if kind == "on_a_stream":  # a pulse that is small against its background, sparse rounding noise
+        g = np.exp(-((x - 0.5) ** 2 + (y - 0.5) ** 2) / (2 * (6 * s) ** 2))
+        return np.stack([1 + 1e-13 * g, 1 + 2.0 ** -52 * (rng.random(ns.N) < 0.02), 3 + 1e-9 * g])
     if kind == "jump":  # small differences beside a unit one
         return 1e-9 * rng.standard_normal((3, ns.N)) + (x > 0.5)
     return 1e-6 * np.exp(5 * rng.standard_normal((3, ns.N))).clip(max=1e6)  # log-normal
 
 
 @pytest.mark.parametrize("m", [4, 6, 8, 10])
-@pytest.mark.parametrize("kind", ["front", "pulse", "impulses", "jump", "lognormal"])
+@pytest.mark.parametrize("kind", ["front", "steep", "pulse", "impulses", "jump", "on_a_stream", "lognormal"])
 def test_fields_of_a_wide_span_within_a_stencil(lb, kind, m):
     # every sum within (24 + n) 2^-53 sum |w d| of the exact one (FP64's own bound for n
     # terms and the lanes' sums), for each operator and field: the bounds of the sums that
