@@ -136,12 +136,13 @@ __global__ void k_pack_fixed(int64_t N, int64_t nnz, int64_t off, const int32_t*
                 if (top[o] > 0) below = max(below, h[o] - top[o]);
             return entry_shift(below);
         };
-        int exps[6], least[6];  // of |w| 2^-s: the largest and the smallest but zero
+        int exps[6], least[6], used[6];  // of |w| 2^-s: the largest and the smallest but zero; how many are not zero
         float sum[6];
 #pragma unroll
         for (int o = 0; o < 6; ++o) {
             exps[o] = -2000;
             least[o] = 4000;
+            used[o] = 0;
             sum[o] = 0.0f;
         }
         for (int e = lane; e < len; e += 32) {
@@ -157,7 +158,10 @@ __global__ void k_pack_fixed(int64_t N, int64_t nnz, int64_t off, const int32_t*
             for (int o = 0; o < 6; ++o) {
                 const int s = o < 5 ? sr : sf;
                 exps[o] = max(exps[o], (h[o] >> 20) - s - 1022);
-                if (h[o] > 0) least[o] = min(least[o], (h[o] >> 20) - s - 1022);
+                if (h[o] > 0) {
+                    least[o] = min(least[o], (h[o] >> 20) - s - 1022);
+                    ++used[o];
+                }
                 // |w| 2^-s over the power of two above the row's largest |w|
                 const int ex = (h[o] >> 20) - (top[o] >> 20) - s + 126;
                 if (h[o] > 0 && ex > 0) sum[o] += __int_as_float((ex << 23) | ((h[o] & 0xfffff) << 3));
@@ -179,6 +183,16 @@ __global__ void k_pack_fixed(int64_t N, int64_t nnz, int64_t off, const int32_t*
                 odd |= exps[o] + 2 - least[o] > kMostAlign;
             }
         }
+        // an operator on few of the row's entries (beside a boundary: differences along one line)
+        // meets differences that are often small against the others'
+        int most = 0;
+#pragma unroll
+        for (int o = 0; o < 5; ++o) {
+            used[o] = __reduce_add_sync(0xffffffffu, used[o]);
+            most = max(most, used[o]);
+        }
+#pragma unroll
+        for (int o = 0; o < 5; ++o) odd |= used[o] > 0 && 2 * used[o] < most;
         const bool raw = __any_sync(0xffffffffu, odd);
         if (lane == 0) {
             int4 v;

@@ -48,7 +48,8 @@
 // whose carries a lane moves up after every 32.  Rows with a weight that is not finite,
 // beyond 2^+-400 at their largest, subnormal or below 2^-500 of their row's largest hold
 // plain FP64 weights and are summed in FP64 (kRawRow), each by itself, so that a failed node
-// changes no other row.  A row whose differences are not finite or beyond 2^460 is summed in
+// changes no other row; so are rows where an operator uses less than half the entries that
+// another does, beside boundaries, most of which would fail the span test.  A row whose differences are not finite or beyond 2^460 is summed in
 // FP64 too, so that infinities and NaN come out as they would, and one whose differences of
 // a field, with their shifts, all lie below 2^-498 without being all zero.  Beside larger ones, differences below
 // 2^-1022 count as zero.  Plans of 2^28 nodes or more need the four bits for their columns:

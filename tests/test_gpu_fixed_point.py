@@ -287,6 +287,13 @@ def test_fields_of_a_wide_span_within_a_stencil(lb, kind, m):
         assert np.all(np.abs(R[k] - val) <= tol), k
     for f in range(3):
         assert np.all(np.abs(filt[f] - (q[f] + S[5, f])) <= B[5, f] + 2 * u * np.abs(filt[f])), f
+    # one sum at a time: of a field alone, R of ln rho is -u_x or -v_y
+    for f in range(3):
+        for op in range(2):
+            alone = np.zeros_like(q)
+            alone[1 + op] = q[f]
+            got = lb.rhs(plan, torch.tensor(alone, device="cuda"), lb.Phys(0.0, 0.0)).cpu().numpy()[0]
+            assert np.all(np.abs(got + S[op, f]) <= B[op, f]), (f, op)
     plan.close()
 
 
