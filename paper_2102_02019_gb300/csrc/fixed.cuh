@@ -532,10 +532,10 @@ __device__ __forceinline__ double fixed_weight(const PlanView<double>& P, int i,
 // beside any others).  slots: the rows, as bits (fixed_nodes, R of them a pass);
 // out[k][slot]: the sums' bit patterns.  Such rows come in clusters (all 16 of a warp, beside
 // a boundary), and a warp's chain through them is what the launch waits for: the next entry's
-// column, values and words are in flight while the current one's products are summed (the
-// Lamb-Oseen step of 40,000 nodes, 5 % of whose rows come here, 409 us, without these rows 285;
-// at 2.5 % an entry at a time 421, a chunk of four 423, so 392; with 16 and 32 lanes a row,
-// whose sums take more of the FP64 pipe, 12 and 48 % more).
+// column, values and words are in flight while the current one's products are summed
+// (Lamb-Oseen steps of 40,000 nodes, by an entry at a time 421 us, a chunk of four 423, one
+// ahead 392).  With 16 and 32 lanes a row, whose sums take more of the FP64 pipe, the step
+// takes 445 and 580 us, with 4 as long as with 8 (391).
 template <bool FILTER, int R, int K, class F>
 __device__ __noinline__ void cold_rows(const int32_t* row_ptr, const char* rec, const int16_t* wexp, F fld,
                                        uint32_t mask, int64_t first, uint32_t slots, long long (*out)[32]) {
